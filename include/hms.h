@@ -96,23 +96,26 @@ typedef struct {
   int32_t batch;             /* iterations per CUDA-graph launch; 0 = default (16) */
   int32_t profile;           /* 1 = time every kernel with CUDA events */
   int32_t coarse_factor;     /* factor of Eq. 8: 0 = auto (FP64 for one- or two-node-wide
-                                set tiles, else FP32 with FP64 refinement: two-sided on two
-                                SMs when the system is at least three bands long, else on
-                                one SM, or on a cluster of 4 SMs when the band is too wide
-                                for one; solved by 64-row blocks with inverted diagonal
-                                blocks where they fit), 1 = FP32 on a cluster of 4 SMs,
+                                set tiles, else FP32 with FP64 refinement: nested dissection
+                                as a tree of fronts, see 6, wherever the fronts fit, else
+                                a band: two-sided on two SMs when the system is at least
+                                three bands long, else on one SM, or on a cluster of 4 SMs
+                                when the band is too wide for one, solved by 64-row blocks
+                                with inverted diagonal blocks where they fit), 1 = FP32 on a cluster of 4 SMs,
                                 2 = FP64, 3 = FP32 on one SM solved in 16-row steps,
                                 4 = FP32 on one SM, 5 = FP32 two-sided: top and bottom
                                 segments eliminated at once on two SMs, then the
                                 separator between them, 6 = FP32 nested dissection of
                                 the set grid over K_aa kept as 9 x 9 blocks per set
-                                pair (no band): boxes of sets cut by a middle column or
-                                row of sets, the fronts of one level of the tree
-                                factored at once, one CTA each, fronts of 300 or more
-                                unknowns by many CTAs (set grids of any width, up to
-                                the 350 x 350 sets of a 1e9-DOF lattice; auto takes it
-                                where no band factor fits, e.g. more than about 22
-                                sets across) */
+                                pair (no band).  Where the fronts fit the shared memory
+                                of a thread-block cluster (up to about 40 sets across):
+                                boxes of sets cut by a middle column and row of sets at
+                                once, the fronts of one level of the tree factored at
+                                once, a cluster each, and all solves of an update in one
+                                launch.  Larger grids: boxes cut by a middle column or
+                                row, one CTA per front, fronts of 300 or more unknowns
+                                by many CTAs (set grids of any width, up to the 350 x
+                                350 sets of a 1e9-DOF lattice) */
   int32_t relax_threads;     /* compute threads per CTA of the relaxation (Eqs. 11-13; one more
                                 warp issues its copies): 64, 128 or 256, or
                                 0 = autotuned: the first problem of a set-tile shape and
@@ -236,8 +239,9 @@ int32_t hms_relax_schedule(int32_t nx, int32_t ny, int32_t set_sx, int32_t set_s
  * appearance.  Returns the class count; -1 for bad arguments, cap too small,
  * or a per-bar EA (d->ea != NULL: no two sets need share a matrix). */
 int32_t hms_set_classes(const hms_lattice_desc* d, int32_t* class_out, int32_t cap);
-/* The nested-dissection plan of the upper level (Eq. 8; coarse_factor = 6)
- * for a grid of mx x my sets, computed on the host; no device is needed.
+/* The nested-dissection plan of the upper level (Eq. 8; coarse_factor = 6 on
+ * set grids too large for the tree of fronts in shared memory) for a grid of
+ * mx x my sets, computed on the host; no device is needed.
  * Node k eliminates the unknowns of its sets S_k and couples to its boundary
  * sets B_k, which lie on its ancestors' separators; children come before
  * their parents, the root last.  nodes_out[6 k .. 6 k + 5] = (|S_k|, |B_k|,
@@ -273,7 +277,8 @@ hms_status hms_solve(hms_problem* pr, int32_t nrhs, const double* loads, const d
  *    rebuilds the work lists when the set of running problems has changed.
  *    It applies when all problems share precision and coarse_solves and use
  *    the FP32 one-SM factor with the 64-row block solve (coarse_factor = 4,
- *    or auto where that is its choice);
+ *    or auto where that is its choice) or the tree of fronts (auto, or
+ *    coarse_factor = 6 where it fits), with nine modes per set;
  *  - streams: each problem runs its own graph rounds on one of up to 64
  *    streams of the context at its own pace.
  * Clones (hms_problem_clone) let one lattice's load vectors run at the same
@@ -304,7 +309,9 @@ int64_t hms_problem_refine_cap_hits(const hms_problem* pr);
 
 /* Per-kernel CUDA-event time of the last hms_solve with options.profile = 1:
  * names "update_residual", "relax", "coarse_assemble", "coarse_band",
- * "coarse_factor", "coarse_residual", "coarse_solve", in that order;
+ * "coarse_factor", "coarse_residual", "coarse_solve", in that order (the
+ * tree of fronts runs an update's solves and refinement residuals in one
+ * launch, counted as "coarse_solve");
  * ms_total[k] and launches[k] for k < n (n <= 7).  Returns the count. */
 int32_t hms_kernel_times(const hms_problem* pr, double* ms_total, int64_t* launches, int32_t n);
 

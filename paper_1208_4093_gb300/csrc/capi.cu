@@ -106,6 +106,13 @@ struct hms_problem {
   NDPlanHost ndp;               // the blocks of K_aa (coarse_blocks.cu; no band)
   NDPlanDev ndd;
   double* blk = nullptr;
+  bool tree = false;            // tree of swept fronts (coarse_tree.cu) over the same blocks
+  TreePlanHost tph;
+  TreeProb tp{};                // plan arrays (shared) and this instance's buffers
+  TreeItem* titems = nullptr;   // shared
+  TreeProb* tprob = nullptr;    // tp on the device
+  int* twhich = nullptr;        // 0: the only problem of the launch
+  double* arow = nullptr;       // scaled rows of K_aa
   int* dropped = nullptr;
   unsigned long long* cstat = nullptr;  // refinement state of the upper-level solve
   double* partials = nullptr;
@@ -203,6 +210,7 @@ bool fp32(const hms_problem* pr) { return pr->precision == HMS_MIXED; }
 // The factor of Eq. 8 (after the scaled band is built) and its per-block
 // matrices, by the configured variant.
 cudaError_t launch_factor_stage(hms_problem* pr, cudaStream_t s, const IterCtl* ctl) {
+  if (pr->tree) return launch_tree_factor(s, pr->tph, pr->tprob, pr->titems, ctl != nullptr);
   if (pr->nd) return launch_nd_factor(s, pr->lv, pr->ndp, pr->ndd, pr->blk, pr->scale, pr->dropped, ctl);
   if (pr->two_sided) return launch_coarse_factor_2s(s, pr->n_c, pr->bw, pr->ts, pr->sband, pr->dropped, ctl);
   cudaError_t e = pr->cluster_factor
@@ -218,6 +226,8 @@ cudaError_t launch_solve_stage(hms_problem* pr, cudaStream_t s, int q, const Ite
   // bit 0: the solve of b; bit 1: the last solve an update allows (the
   // kernels count the updates whose refinement had not converged before it)
   const int flags = (q == 0 ? 1 : 0) | (q == pr->nsolve - 1 ? 2 : 0);
+  if (pr->tree)  // all solves of the update
+    return launch_tree_solve(s, pr->lv.q, pr->tph.scl, pr->tph.solve_smem, pr->tprob, pr->twhich, 1, ctl != nullptr);
   if (pr->nd)
     return launch_nd_solve(s, pr->n_c, pr->ndp, pr->ndd, rhs, pr->x, pr->scale, pr->a, pr->dropped, pr->cstat, flags,
                            ctl);
@@ -248,6 +258,7 @@ cudaError_t launch_relax_main(hms_problem* pr, cudaStream_t s, const IterCtl* ct
 // K_aa from the slots and the scaled system of Eq. 8 (scale, b, x = 0, drop
 // flags): by blocks for nested dissection, else as a band.
 cudaError_t launch_scaled_system(hms_problem* pr, cudaStream_t s, const IterCtl* ctl) {
+  if (pr->tree) return launch_tree_system(s, pr->lv.q, true, pr->tprob, nullptr, pr->lv.M, ctl != nullptr);
   if (pr->nd) {
     cudaError_t e = launch_blocks_from_slots(s, pr->lv, pr->slots_base, pr->slots_it, pr->blk, ctl);
     if (e != cudaSuccess) return e;
@@ -277,6 +288,9 @@ cudaError_t launch_force_relax(hms_problem* pr, cudaStream_t s, const IterCtl* c
   if (e != cudaSuccess) return e;
   return launch_force_out(s, lv, pr->delta_rf, fp32(pr), pr->Mforce, pr->r, pr->P, ctl);
 }
+
+// Solve launches of an update: the tree's one launch holds all of its solves.
+int solve_launches(const hms_problem* pr) { return pr->tree ? 1 : pr->nsolve; }
 
 // Launches of one iteration (the body of Fig. 3's loop); k = position in a batch.
 cudaError_t launch_iteration(hms_problem* pr, cudaStream_t s, int k, cudaEvent_t* ev) {
@@ -308,7 +322,7 @@ cudaError_t launch_iteration(hms_problem* pr, cudaStream_t s, int k, cudaEvent_t
   e = launch_factor_stage(pr, s, pr->ctl);
   if (e != cudaSuccess) return e;
   mark();
-  for (int q = 0; q < pr->nsolve; ++q) {
+  for (int q = 0; q < solve_launches(pr); ++q) {
     if (q > 0) {
       e = launch_refine_residual(pr, s, pr->ctl);
       if (e != cudaSuccess) return e;
@@ -517,27 +531,39 @@ void class_plan_build(const LatView& lv, const std::vector<uint8_t>& fix, int ts
   }
 }
 
-// Nested dissection over the set grid (coarse_nd.cu): the plan of fronts, if
-// every front fits the factor kernel's shared memory.
-bool choose_nd(hms_problem* pr, int maxsm) {
+// Nested dissection over the set grid: as a tree of fronts swept in the shared
+// memory of one cluster each (coarse_tree.cu) where they fit, else panel by
+// panel from device memory (coarse_nd.cu), if every front fits the factor
+// kernel's shared memory.
+bool choose_tree(hms_problem* pr, int maxsm) {
   pr->coarse_fp64 = false;
   pr->two_sided = false;
   pr->cluster_factor = false;
   pr->big_stages = 0;
   pr->nd = false;
+  pr->tree = tree_plan_build(pr->lv, maxsm, &pr->tph);
+  return pr->tree;
+}
+bool choose_nd(hms_problem* pr, int maxsm) {
+  if (choose_tree(pr, maxsm)) return true;
   if (!nd_plan_build(pr->lv, &pr->ndp) || !nd_plan_smem(&pr->ndp, maxsm)) return false;
   pr->nd = true;
   return true;
 }
 
-// The factor of Eq. 8: coarse_factor = 6 is nested dissection; otherwise the
-// band factors of choose_band, and with coarse_factor = 0 nested dissection
-// where no band factor fits (set grids wider than one SM's band window).
+// The factor of Eq. 8: coarse_factor = 6 is nested dissection, 1 to 5 are the
+// band factors of choose_band.  With coarse_factor = 0, FP64 for degenerate set
+// shapes as choose_band has it; else the tree wherever its fronts fit: factor
+// and solves of an update took 105 us against 183 for the one-SM band on 4 x 4
+// sets (FP64 form), 172 against 336 for the two-sided band on 8 x 8, 271 against
+// 863 on 16 x 16; then a band factor, then the panel-by-panel fronts.
 bool choose_coarse(hms_problem* pr, const hms_options* o, int maxsm) {
-  pr->nd = false;
+  pr->nd = pr->tree = false;
   if (o->coarse_factor == 6) return choose_nd(pr, maxsm);
-  if (choose_band(pr, o, maxsm)) return true;
-  return o->coarse_factor == 0 && choose_nd(pr, maxsm);
+  const bool band = choose_band(pr, o, maxsm);
+  if (o->coarse_factor != 0 || (band && pr->coarse_fp64)) return band;
+  if (choose_tree(pr, maxsm)) return true;
+  return choose_band(pr, o, maxsm) || choose_nd(pr, maxsm);
 }
 
 }  // namespace
@@ -580,6 +606,7 @@ hms_status hms_context_create(int32_t device, hms_context** out) {
   if (e == cudaSuccess) e = configure_coarse_solve(maxsm);
   if (e == cudaSuccess) e = configure_coarse_factor_cl(maxsm);
   if (e == cudaSuccess) e = configure_coarse_nd(maxsm);
+  if (e == cudaSuccess) e = configure_coarse_tree(maxsm);
   if (e != cudaSuccess) {
     g_create_err = std::string("context setup: ") + cudaGetErrorString(e);
     if (c->stream) cudaStreamDestroy(c->stream);
@@ -666,6 +693,11 @@ hms_status hms_problem_clone(hms_problem* src, hms_problem** out) {
   pr->fixF = src->fixF;
   pr->Mforce = src->Mforce;
   pr->slots_base = src->slots_base;
+  pr->tree = src->tree;
+  pr->tph = src->tph;
+  pr->tp = src->tp;  // the plan arrays; alloc_instance sets the buffers
+  pr->titems = src->titems;
+  pr->twhich = src->twhich;
   cudaError_t e = alloc_instance(pr);
   if (e == cudaSuccess && pr->relax_sched) {
     bool ok = false;  // the clone's own flags (same plan)
@@ -813,7 +845,7 @@ static cudaError_t alloc_instance(hms_problem* pr) {
   CKI(palloc(pr, &pr->a, n_c));
   CKI(palloc(pr, &pr->P, n_c));
   CKI(palloc(pr, &pr->slots_it, (size_t)lv.M * NSLOTS * slot_size(lv.q)));
-  if (!pr->nd) {
+  if (!pr->nd && !pr->tree) {
     CKI(palloc(pr, &pr->band, nband));
     CKI(palloc(pr, &pr->sband, 2 * nband));
   }
@@ -821,7 +853,20 @@ static cudaError_t alloc_instance(hms_problem* pr) {
   CKI(palloc(pr, &pr->b, n_c));
   CKI(palloc(pr, &pr->x, n_c));
   CKI(palloc(pr, &pr->res, n_c));
-  if (pr->nd) {
+  if (pr->tree) {
+    CKI(palloc(pr, &pr->blk, coarse_blocks_elems(lv)));
+    CKI(palloc(pr, &pr->arow, tree_arow_elems(lv)));
+    TreeProb& T = pr->tp;
+    const TreePlanHost& P = pr->tph;
+    CKI(palloc(pr, &T.U, P.u_elems));
+    CKI(palloc(pr, &T.M, P.m_elems));
+    CKI(palloc(pr, &T.V, P.v_elems));
+    CKI(palloc(pr, &T.X, P.x_elems));
+    // the rows' padding and V's zeros stay as set here
+    CKI(cudaMemsetAsync(T.M, 0, P.m_elems * sizeof(float), s));
+    CKI(cudaMemsetAsync(T.V, 0, P.v_elems * sizeof(float), s));
+    CKI(palloc(pr, &pr->tprob, 1));
+  } else if (pr->nd) {
     // the blocks of K_aa (the fronts' input), the plan and the fronts
     CKI(palloc(pr, &pr->blk, coarse_blocks_elems(lv)));
     const NDPlanHost& P = pr->ndp;
@@ -891,6 +936,33 @@ static cudaError_t alloc_instance(hms_problem* pr) {
   }
   CKI(cudaMallocHost(&pr->ctl_host, sizeof(IterCtl)));
   CKI(cudaMemsetAsync(pr->a, 0, n_c * sizeof(double), s));
+  if (pr->tree) {
+    TreeProb& T = pr->tp;
+    T.slots_base = pr->slots_base;
+    T.slots_it = pr->slots_it;
+    T.P = pr->P;
+    T.blk = pr->blk;
+    T.arow = pr->arow;
+    T.lv = lv;
+    T.mode_mask = pr->mode_mask;
+    T.b = pr->b;
+    T.scale = pr->scale;
+    T.x = pr->x;
+    T.a = pr->a;
+    T.dropped = pr->dropped;
+    T.cstat = pr->cstat;
+    T.ctl = pr->ctl;
+    T.n = n_c;
+    T.nm = lv.q;
+    T.Mx = lv.Mx;
+    T.My = lv.My;
+    T.nsolve = pr->nsolve;
+    T.nphase = pr->tph.nphase;
+    T.v_rhs = pr->tph.v_rhs;
+    T.v_x = pr->tph.v_x;
+    CKI(cudaMemcpyAsync(pr->tprob, &T, sizeof(T), cudaMemcpyHostToDevice, s));
+    CKI(cudaStreamSynchronize(s));  // tp may move on after return
+  }
 
 #undef CKI
   return cudaSuccess;
@@ -1216,6 +1288,36 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
       CKP(cudaMemcpy(pr->Mforce, Mh.data(), 9 * (size_t)lv.M * sizeof(double), cudaMemcpyHostToDevice));
     }
   }
+  if (pr->tree) {
+    // the tree's plan, shared with clones
+    const TreePlanHost& P = pr->tph;
+    TreeNode* nodes;
+    int *sets, *inv;
+    int4 *gath, *rows, *phase;
+    const size_t ng = P.gath.size() / 4 /* int4s */, nr = P.rows.size() / 4;
+    CKP(salloc(pr, &nodes, P.nodes.size()));
+    CKP(salloc(pr, &sets, P.sets.size()));
+    CKP(salloc(pr, &inv, std::max<size_t>(P.inv.size(), 1)));
+    CKP(salloc(pr, &gath, ng));
+    CKP(salloc(pr, &rows, nr));
+    CKP(salloc(pr, &phase, P.phase.size()));
+    CKP(salloc(pr, &pr->titems, P.items.size()));
+    CKP(salloc(pr, &pr->twhich, 1));
+    CKP(cudaMemcpy(nodes, P.nodes.data(), P.nodes.size() * sizeof(TreeNode), cudaMemcpyHostToDevice));
+    CKP(cudaMemcpy(sets, P.sets.data(), P.sets.size() * sizeof(int), cudaMemcpyHostToDevice));
+    if (!P.inv.empty()) CKP(cudaMemcpy(inv, P.inv.data(), P.inv.size() * sizeof(int), cudaMemcpyHostToDevice));
+    CKP(cudaMemcpy(gath, P.gath.data(), ng * sizeof(int4), cudaMemcpyHostToDevice));
+    CKP(cudaMemcpy(rows, P.rows.data(), nr * sizeof(int4), cudaMemcpyHostToDevice));
+    CKP(cudaMemcpy(phase, P.phase.data(), P.phase.size() * sizeof(TreeSpan), cudaMemcpyHostToDevice));
+    CKP(cudaMemcpy(pr->titems, P.items.data(), P.items.size() * sizeof(TreeItem), cudaMemcpyHostToDevice));
+    CKP(cudaMemset(pr->twhich, 0, sizeof(int)));
+    pr->tp.nodes = nodes;
+    pr->tp.sets = sets;
+    pr->tp.inv = inv;
+    pr->tp.gath = gath;
+    pr->tp.rows = rows;
+    pr->tp.phase = phase;
+  }
   // ---- iteration buffers ----
   CKP(salloc(pr, &pr->slots_base, (size_t)lv.M * NSLOTS * slot_size(lv.q)));
   CKP(alloc_instance(pr));
@@ -1373,7 +1475,7 @@ hms_status hms_solve(hms_problem* pr, int32_t nrhs, const double* loads, const d
         CKC(c, launch_iteration(pr, s, it, ev.data()));
         CKC(c, cudaMemcpyAsync(pr->ctl_host, pr->ctl, sizeof(IterCtl), cudaMemcpyDeviceToHost, s));
         CKC(c, cudaStreamSynchronize(s));
-        const int nev = 7 + 2 * (pr->nsolve - 1);  // marks recorded by launch_iteration
+        const int nev = 7 + 2 * (solve_launches(pr) - 1);  // marks recorded by launch_iteration
         const bool ran_all = !pr->ctl_host->done;
         for (int i = 0; i + 1 < nev; ++i) {
           if (i > 0 && !ran_all) break;  // after convergence only K1 did work
@@ -1468,9 +1570,8 @@ hms_status hms_context_set_batch_mode(hms_context* c, int32_t mode) {
 static bool lockstep_applies(int32_t count, hms_problem* const* problems) {
   for (int i = 0; i < count; ++i) {
     const hms_problem* pr = problems[i];
-    if (!pr || pr->profile || pr->coarse_fp64 || pr->cluster_factor || pr->two_sided || pr->big_stages <= 0 ||
-        pr->lv.q != NMODES || pr->cls)
-      return false;
+    if (!pr || pr->profile || pr->lv.q != NMODES || pr->cls) return false;
+    if (!pr->tree && (pr->coarse_fp64 || pr->cluster_factor || pr->two_sided || pr->big_stages <= 0)) return false;
     if (pr->precision != problems[0]->precision || pr->nsolve != problems[0]->nsolve) return false;
   }
   return true;
@@ -1673,6 +1774,54 @@ static BatchProb batch_prob_of(const hms_problem* pr) {
 // another in one array; off[k] .. off[k + 1] is kernel k's list.
 enum BatchList { BL_K1 = 0, BL_SETS, BL_BAND, BL_DIAG, BL_DROPS, BL_SCALE, BL_ONE, BL_BLOCKINV, BL_CRES, BL_COUNT };
 
+// The running problems with the tree factor: their sets, their nodes level by
+// level (TreeItem), and the problems by the CTAs of their solves.
+struct TreeLists {
+  std::vector<TreeItem> items;  // sets, then the nodes of level 0, 1, ...
+  int nsets = 0;
+  std::vector<int> begin, T;    // per level: first entry (one more at the end), block rows of the largest front
+  std::vector<int> which;       // problem indices, by scl
+  std::vector<std::array<int, 3>> solves;  // {scl, first entry in which, count}
+  std::vector<size_t> solve_smem;
+};
+static void build_tree_lists(const std::vector<hms_problem*>& probs, const std::vector<int>& run, TreeLists* L) {
+  *L = TreeLists();
+  int nlev = 0;
+  for (int i : run) {
+    const hms_problem* pr = probs[i];
+    if (!pr->tree) continue;
+    for (int I = 0; I < pr->lv.M; ++I) L->items.push_back(TreeItem{i, I});
+    nlev = std::max(nlev, pr->tph.nlev);
+  }
+  L->nsets = (int)L->items.size();
+  for (int h = 0; h < nlev; ++h) {
+    L->begin.push_back((int)L->items.size());
+    int T = 1;
+    for (int i : run) {
+      const hms_problem* pr = probs[i];
+      if (!pr->tree || h >= pr->tph.nlev) continue;
+      T = std::max(T, pr->tph.level_T[h]);
+      for (int k = pr->tph.level_begin[h]; k < pr->tph.level_begin[h + 1]; ++k)
+        L->items.push_back(TreeItem{i, pr->tph.items[k].node});
+    }
+    L->T.push_back(T);
+  }
+  L->begin.push_back((int)L->items.size());
+  for (int scl = 1; scl <= 16; scl *= 2) {
+    const int first = (int)L->which.size();
+    size_t smem = 0;
+    for (int i : run)
+      if (probs[i]->tree && probs[i]->tph.scl == scl) {
+        L->which.push_back(i);
+        smem = std::max(smem, probs[i]->tph.solve_smem);
+      }
+    if ((int)L->which.size() > first) {
+      L->solves.push_back({scl, first, (int)L->which.size() - first});
+      L->solve_smem.push_back(smem);
+    }
+  }
+}
+
 static void build_lists(const std::vector<hms_problem*>& probs, const std::vector<int>& run,
                         std::vector<BatchItem>& items, int off[BL_COUNT + 1]) {
   items.clear();
@@ -1680,6 +1829,7 @@ static void build_lists(const std::vector<hms_problem*>& probs, const std::vecto
     off[k] = (int)items.size();
     for (int i : run) {
       const hms_problem* pr = probs[i];
+      if (pr->tree && k != BL_K1 && k != BL_SETS) continue;  // the band's steps
       const LatView& lv = pr->lv;
       auto grid = [&](int g) {
         for (int b = 0; b < g; ++b) items.push_back(BatchItem{i, b, 0, g, 1});
@@ -1737,10 +1887,12 @@ static hms_status solve_batch_lockstep(hms_context* c, int32_t count, hms_proble
   for (hms_problem* pr : probs) rchunks = std::min(rchunks, pr->relax_chunks);
   int stages = 3;
   size_t sm_relax = 0, sm_slots = 0, sm_factor = 0, sm_solve = 0;
-  for (hms_problem* pr : probs) stages = std::min(stages, pr->big_stages);
+  for (hms_problem* pr : probs)
+    if (!pr->tree) stages = std::min(stages, pr->big_stages);
   for (hms_problem* pr : probs) {
     sm_relax = std::max(sm_relax, relax_smem_bytes(pr->lv, f32, rchunks));
     sm_slots = std::max(sm_slots, coarse_slots_smem(pr->lv));
+    if (pr->tree) continue;
     sm_factor = std::max(sm_factor, coarse_factor_smem_bytes(pr->n_c, pr->bw, false));
     sm_solve = std::max(sm_solve, big_solve_smem_bytes(pr->n_c, pr->bw, stages));
   }
@@ -1750,7 +1902,7 @@ static hms_status solve_batch_lockstep(hms_context* c, int32_t count, hms_proble
     ~DevBuf() {
       if (p) cudaFree(p);
     }
-  } dprob, dwhich, ditems, dctl;
+  } dprob, dwhich, ditems, dctl, dtree, dtitems, dtwhich;
   std::vector<BatchProb> hp(count);
   for (int i = 0; i < count; ++i) hp[i] = batch_prob_of(probs[i]);
   CKC(c, cudaMalloc(&dprob.p, std::max<size_t>(1, count) * sizeof(BatchProb)));
@@ -1764,6 +1916,15 @@ static hms_status solve_batch_lockstep(hms_context* c, int32_t count, hms_proble
     ~HostFree() { cudaFreeHost(p); }
   } hctl_guard{hctl};
   const BatchProb* P = (const BatchProb*)dprob.p;
+  std::vector<TreeProb> ht(count);
+  for (int i = 0; i < count; ++i) ht[i] = probs[i]->tp;
+  CKC(c, cudaMalloc(&dtree.p, std::max<size_t>(1, count) * sizeof(TreeProb)));
+  CKC(c, cudaMalloc(&dtwhich.p, std::max<size_t>(1, count) * sizeof(int)));
+  CKC(c, cudaMemcpyAsync(dtree.p, ht.data(), count * sizeof(TreeProb), cudaMemcpyHostToDevice, s));
+  int maxsm = 0;
+  CKC(c, cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
+  const TreeProb* TP = (const TreeProb*)dtree.p;
+  TreeLists tl;
 
   std::vector<long long> ioff(count + 1, 0);
   for (int i = 0; i < count; ++i) ioff[i + 1] = ioff[i] + nrhs[i];
@@ -1791,7 +1952,7 @@ static hms_status solve_batch_lockstep(hms_context* c, int32_t count, hms_proble
     }
   std::vector<BatchItem> items;
   int off[BL_COUNT + 1];
-  size_t items_cap = 0;
+  size_t items_cap = 0, titems_cap = 0;
   cudaGraphExec_t exec = nullptr;
   struct ExecGuard {
     cudaGraphExec_t& e;
@@ -1811,6 +1972,19 @@ static hms_status solve_batch_lockstep(hms_context* c, int32_t count, hms_proble
       }
       CKC(c, cudaMemcpyAsync(ditems.p, items.data(), items.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, s));
       CKC(c, cudaMemcpyAsync(dwhich.p, run.data(), run.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+      build_tree_lists(probs, run, &tl);
+      if (tl.items.size() > titems_cap) {
+        if (dtitems.p) cudaFree(dtitems.p);
+        dtitems.p = nullptr;
+        titems_cap = tl.items.size();
+        CKC(c, cudaMalloc(&dtitems.p, titems_cap * sizeof(TreeItem)));
+      }
+      if (!tl.items.empty()) {
+        CKC(c, cudaMemcpyAsync(dtitems.p, tl.items.data(), tl.items.size() * sizeof(TreeItem), cudaMemcpyHostToDevice,
+                               s));
+        CKC(c, cudaMemcpyAsync(dtwhich.p, tl.which.data(), tl.which.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+      }
+      const TreeItem* TI = (const TreeItem*)dtitems.p;
       const BatchItem* I = (const BatchItem*)ditems.p;
       auto L = [&](int k) { return I + off[k]; };
       auto N = [&](int k) { return off[k + 1] - off[k]; };
@@ -1825,6 +1999,14 @@ static hms_status solve_batch_lockstep(hms_context* c, int32_t count, hms_proble
         e = launch_batch_update_residual(s, f32, P, L(BL_K1), N(BL_K1), k);
         if (e == cudaSuccess) e = launch_batch_relax(s, f32, rthreads, rchunks, sm_relax, P, L(BL_SETS), N(BL_SETS));
         if (e == cudaSuccess) e = launch_batch_slots(s, f32, sm_slots, P, L(BL_SETS), N(BL_SETS));
+        if (e == cudaSuccess) e = launch_tree_system(s, NMODES, true, TP, TI, tl.nsets, true);
+        for (size_t h = 0; h < tl.T.size() && e == cudaSuccess; ++h) {
+          const int n = tl.begin[h + 1] - tl.begin[h];
+          e = launch_tree_level(s, tree_level_launch(n, tl.T[h], maxsm), TP, TI + tl.begin[h], n, true);
+        }
+        for (size_t z = 0; z < tl.solves.size() && e == cudaSuccess; ++z)
+          e = launch_tree_solve(s, NMODES, tl.solves[z][0], tl.solve_smem[z], TP, (const int*)dtwhich.p + tl.solves[z][1],
+                                tl.solves[z][2], true);
         if (e == cudaSuccess) e = launch_batch_band(s, P, L(BL_BAND), N(BL_BAND));
         if (e == cudaSuccess) e = launch_batch_diag(s, P, L(BL_DIAG), N(BL_DIAG));
         if (e == cudaSuccess) e = launch_batch_set_drops(s, P, L(BL_DROPS), N(BL_DROPS));
@@ -2009,12 +2191,13 @@ hms_status hms_coarse_matrix(hms_problem* pr, const double* delta, double* Kaa, 
   cudaStream_t s = c->stream;
   CKC(c, stage_deltas(pr, delta, mem_kind));
   CKC(c, launch_coarse_slots(s, pr->lv, pr->delta, fp32(pr), false, pr->slots_it, nullptr, pr->delta_rf));
-  if (pr->nd) CKC(c, launch_blocks_from_slots(s, pr->lv, pr->slots_base, pr->slots_it, pr->blk, nullptr));
+  const bool blocks = pr->nd || pr->tree;
+  if (blocks) CKC(c, launch_blocks_from_slots(s, pr->lv, pr->slots_base, pr->slots_it, pr->blk, nullptr));
   else CKC(c, launch_coarse_band_from_slots(s, pr->lv, pr->slots_base, pr->slots_it, pr->band, nullptr));
   double* dense = nullptr;
   const size_t nd = (size_t)pr->n_c * pr->n_c;
   CKC(c, cudaMallocAsync(&dense, nd * sizeof(double), s));
-  cudaError_t e = pr->nd ? launch_dense_from_blocks(s, pr->lv, pr->blk, dense)
+  cudaError_t e = blocks ? launch_dense_from_blocks(s, pr->lv, pr->blk, dense)
                          : launch_coarse_dense_from_band(s, pr->n_c, pr->bw, pr->band, dense);
   if (e == cudaSuccess) e = cudaMemcpyAsync(Kaa, dense, nd * sizeof(double), kind_out(mem_kind), s);
   cudaFreeAsync(dense, s);
@@ -2036,18 +2219,20 @@ hms_status hms_coarse_solve(hms_problem* pr, const double* Kaa, const double* P,
   CKC(c, cudaMallocAsync(&dense, nd * sizeof(double), s));
   cudaError_t e = cudaMemcpyAsync(dense, Kaa, nd * sizeof(double), kind_in(mem_kind), s);
   if (e == cudaSuccess)
-    e = pr->nd ? launch_blocks_from_dense(s, pr->lv, dense, pr->blk) : launch_coarse_band_from_dense(s, n, bw, dense,
+    e = (pr->nd || pr->tree) ? launch_blocks_from_dense(s, pr->lv, dense, pr->blk) : launch_coarse_band_from_dense(s, n, bw, dense,
                                                                                                       pr->band);
   cudaFreeAsync(dense, s);
   CKC(c, e);
   CKC(c, cudaMemcpyAsync(pr->P, P, n * sizeof(double), kind_in(mem_kind), s));
-  if (pr->nd)
+  if (pr->tree)
+    CKC(c, launch_tree_system(s, pr->lv.q, false, pr->tprob, nullptr, pr->lv.M, false));
+  else if (pr->nd)
     CKC(c, launch_blk_diag(s, pr->lv, pr->blk, pr->P, pr->scale, pr->b, pr->x, pr->dropped, pr->mode_mask, nullptr));
   else
     CKC(c, launch_coarse_scale(s, n, bw, pr->coarse_fp64, pr->band, pr->P, pr->sband, pr->lrow, pr->scale, pr->b,
                                pr->x, pr->dropped, pr->mode_mask, pr->lv.q, nullptr));
   CKC(c, launch_factor_stage(pr, s, nullptr));
-  for (int q = 0; q < pr->nsolve; ++q) {
+  for (int q = 0; q < solve_launches(pr); ++q) {
     if (q > 0) CKC(c, launch_refine_residual(pr, s, nullptr));
     CKC(c, launch_solve_stage(pr, s, q, nullptr));
   }
@@ -2176,8 +2361,15 @@ bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options
   if (force) *shared += fac * esz + nn + 9 * M * 8;  // cut-free factors, supports | pins, projections
   size_t b = 4 * nn * 16 + nn * 2 * esz + ybytes;
   if (force) b += nn * 16 + nn * 2 * esz;  // r projected, delta^RF
-  b += 2 * n_c * 8 + M * NSLOTS * ss * 8 + (pr.nd ? 0 : 3 * nband * 8) + 4 * n_c * 8;
-  if (pr.nd) {
+  b += 2 * n_c * 8 + M * NSLOTS * ss * 8 + (pr.nd || pr.tree ? 0 : 3 * nband * 8) + 4 * n_c * 8;
+  if (pr.tree) {
+    const TreePlanHost& P = pr.tph;
+    *shared += P.nodes.size() * sizeof(TreeNode) + P.sets.size() * 4 + std::max<size_t>(P.inv.size(), 1) * 4 +
+               P.gath.size() * 4 + P.rows.size() * 4 + P.phase.size() * sizeof(TreeSpan) +
+               P.items.size() * sizeof(TreeItem) + 4;
+    b += (coarse_blocks_elems(lv) + tree_arow_elems(lv)) * 8 + (P.u_elems + P.m_elems + P.v_elems + P.x_elems) * 4 +
+         sizeof(TreeProb);
+  } else if (pr.nd) {
     const NDPlanHost& P = pr.ndp;
     b += coarse_blocks_elems(lv) * 8 + P.nodes.size() * sizeof(NDNode) + P.sets.size() * 4 +
          std::max<size_t>(P.maps.size(), 1) * 4 + P.lvl_nodes.size() * 4 +

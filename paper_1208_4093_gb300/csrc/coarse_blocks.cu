@@ -19,46 +19,13 @@
 //                   system (Eq. 8), one thread per unknown over its nine
 //                   neighbour sets;
 // and the dense conversions of the step entry points.
+#include "coarse_blocks.cuh"
 #include "hms_internal.cuh"
 
 namespace hms {
 namespace {
 
 __device__ inline bool done_(const IterCtl* ctl) { return ctl && *(volatile const int*)&ctl->done; }
-
-__device__ inline double slot_val(const double* base, const double* it, int nm, int I, int slot, int p, int c) {
-  const size_t o = ((size_t)I * NSLOTS + slot) * slot_size(nm) + (size_t)p * slot_dim(nm) + c;
-  return base[o] + it[o];
-}
-
-// entry (J mode l, I mode m) of K_aa, J the neighbour b of I (b = 0: J = I);
-// 0 if J lies outside the set grid
-__device__ inline double blk_entry(const LatView& lv, const double* base, const double* it, int I, int b, int l,
-                                   int m) {
-  const int nm = lv.q;
-  const int Ix = I % lv.Mx, Iy = I / lv.Mx;
-  if (b == BLK_SELF) {
-    double v = slot_val(base, it, nm, I, SLOT_SELF, l, m);
-    for (int s = SLOT_E; s < NSLOTS; ++s) v += slot_val(base, it, nm, I, s, l, m);
-    // neighbours that own bars into I
-    const int kx[5] = {-1, 1, 0, -1, 1};  // owner offset for E, W, N, NE, NW
-    const int ky[5] = {0, 0, -1, -1, -1};
-    for (int s = 0; s < 5; ++s) {
-      const int Kx = Ix + kx[s], Ky = Iy + ky[s];
-      if (Kx < 0 || Kx >= lv.Mx || Ky < 0 || Ky >= lv.My) continue;
-      v += slot_val(base, it, nm, Ky * lv.Mx + Kx, SLOT_E + s, nm + l, nm + m);
-    }
-    return v;
-  }
-  const int dx = blk_dx(b), dy = blk_dy(b);
-  const int Jx = Ix + dx, Jy = Iy + dy;
-  if (Jx < 0 || Jx >= lv.Mx || Jy >= lv.My) return 0.0;
-  const int J = Jy * lv.Mx + Jx;
-  if (b == BLK_E) return slot_val(base, it, nm, I, SLOT_E, nm + l, m) + slot_val(base, it, nm, J, SLOT_W, l, nm + m);
-  if (b == BLK_N) return slot_val(base, it, nm, I, SLOT_N, nm + l, m);
-  if (b == BLK_NE) return slot_val(base, it, nm, I, SLOT_NE, nm + l, m);
-  return slot_val(base, it, nm, I, SLOT_NW, nm + l, m);
-}
 
 __global__ void k_blocks_from_slots(LatView lv, const double* __restrict__ base, const double* __restrict__ it,
                                     double* __restrict__ blk, const IterCtl* ctl) {

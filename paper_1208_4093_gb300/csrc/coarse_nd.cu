@@ -1,5 +1,6 @@
 // K4 by nested dissection: the upper-level solve of Eq. 8 with its work
-// spread over the SMs, for set grids of any width.
+// spread over the SMs, for set grids of any width (coarse_tree.cu takes those
+// whose fronts fit a cluster's shared memory).
 //
 // The band factorisations (coarse_solve.cu) are one dependency chain down the
 // band: n / 16 block steps on one or two SMs, and a band window that must fit

@@ -486,6 +486,72 @@ cudaError_t launch_nd_factor(cudaStream_t s, const LatView& lv, const NDPlanHost
 cudaError_t launch_nd_solve(cudaStream_t s, int n, const NDPlanHost& P, const NDPlanDev& D, const double* rhs,
                             double* x, const double* scale, double* a_out, const int* dropped,
                             unsigned long long* cstat, int flags, const IterCtl* ctl);
+// coarse_tree.cu: the tree of dense fronts swept in shared memory, for set grids
+// whose fronts fit one cluster's shared memory.
+struct TreeNode {
+  int ns, nb, s_off, nchild;  // own and boundary sets, their place in sets (S, then B), children
+  int inv_off[4];             // per child: the place of each set of this front in its boundary, in inv
+  int cnb[4];                 // the children's boundary unknowns
+  long long cu_off[4];        // and update matrices, in U
+  long long u_off;            // this front's update matrix [nB][nB]
+  long long x_off;            // its pivot columns in passing, in X
+  long long mf_off, mb_off;   // its forward [nB][s4] and backward [nS][s4 + b4] rows, in M
+};
+struct TreeItem {
+  int prob, node;
+};
+// gather entries [g0, g1) and matrix rows [r0, r1) of one CTA in one phase of the solves
+struct TreeSpan {
+  int g0, g1, r0, r1;
+};
+// One problem as the kernels read it (in device memory).
+struct TreeProb {
+  const TreeNode* nodes;
+  const int *sets, *inv;
+  const int4 *gath, *rows, *phase;
+  const double *slots_base, *slots_it, *P;
+  double *blk, *arow, *b, *scale, *x, *a;
+  int* dropped;
+  unsigned long long* cstat;
+  const IterCtl* ctl;
+  float *U, *M, *V, *X;
+  LatView lv;
+  int n, nm, Mx, My, nsolve, nphase, v_rhs, v_x;
+  unsigned mode_mask;
+};
+// A factor launch: CTAs per front, buffers of the pivot column, shared memory.
+struct TreeLaunch {
+  int cl, nbuf;
+  size_t smem;
+};
+struct TreePlanHost {
+  std::vector<TreeNode> nodes;
+  std::vector<int> sets, inv;
+  std::vector<TreeItem> items;  // the nodes level by level, leaves first
+  std::vector<int> level_begin, level_cl, level_nbuf, level_T;  // level_T: block rows of the largest front
+  std::vector<size_t> level_smem;
+  std::vector<int> gath, rows;  // eight ints per entry
+  std::vector<TreeSpan> phase;  // [phase][CTA]
+  int n = 0, nm = 9, nlev = 0, scl = 1, nphase = 0, v_rhs = 0, v_x = 0;
+  size_t m_elems = 0, u_elems = 0, v_elems = 0, x_elems = 0, solve_smem = 0;
+};
+// The plan of a set grid; false if a front does not fit (coarse_nd.cu takes it).
+bool tree_plan_build(const LatView& lv, int max_smem, TreePlanHost* P);
+size_t tree_arow_elems(const LatView& lv);
+cudaError_t configure_coarse_tree(int max_smem);
+TreeLaunch tree_level_launch(int n, int T, int max_smem);
+// The launches take problems probs and a work list: {problem, set}, {problem,
+// node} or problem indices (no list: the sets of the only problem).  use_ctl:
+// problems whose control block says done are passed over.
+// scale, b, x = 0, drop flags and the scaled rows, from the slots or the blocks
+cudaError_t launch_tree_system(cudaStream_t s, int q, bool slots, const TreeProb* probs, const TreeItem* sets, int n,
+                               bool use_ctl);
+cudaError_t launch_tree_level(cudaStream_t s, const TreeLaunch& L, const TreeProb* probs, const TreeItem* nodes, int n,
+                              bool use_ctl);
+cudaError_t launch_tree_factor(cudaStream_t s, const TreePlanHost& P, const TreeProb* prob, const TreeItem* items,
+                               bool use_ctl);
+cudaError_t launch_tree_solve(cudaStream_t s, int q, int scl, size_t smem, const TreeProb* probs, const int* which,
+                              int n, bool use_ctl);
 // coarse_factor_cluster.cu
 size_t coarse_factor_cl_smem_bytes(int n, int bw);
 cudaError_t configure_coarse_factor_cl(int max_smem);
