@@ -106,30 +106,46 @@ def peaks():
 
 
 # ---------------------------------------------------------------- algorithmic work
-def factor_entries(nb, h):
-    def pad4(n):
-        return (n + 3) // 4 * 4
-
-    linv = pad4(nb * (nb + 1) // 2)
-    boff = 4 * nb + (nb - 4) * nb - (nb - 4) * (nb - 3) // 2 if nb > 4 else nb * nb
-    return h * linv + (h - 1) * pad4(boff)
+def dissection_entries(w, h):
+    """Factor entries of the nested dissection of a w x h-node set: per tree node
+    with ns unknowns of its own and nb around its box, D (ns x ns) and G (nb x
+    ns) once for the way up and once, transposed, for the way down.  Boxes are
+    cut by the middle column or row, those of up to 16 nodes a side by both;
+    boxes of up to 2 x 2 nodes are not cut."""
+    total = 0
+    boxes = [(0, 0, w, h)]
+    while boxes:
+        x0, y0, bw, bh = boxes.pop()
+        around = ((min(x0 + bw + 1, w) - max(x0 - 1, 0)) * (min(y0 + bh + 1, h) - max(y0 - 1, 0))) - bw * bh
+        inner = 0
+        if bw > 2 or bh > 2:
+            both = bw > 2 and bh > 2 and max(bw, bh) <= 16 and bw <= 2 * bh and bh <= 2 * bw
+            xs, ys = [(x0, bw)], [(y0, bh)]
+            if both or bw >= bh:
+                xs = [(x0, bw // 2), (x0 + bw // 2 + 1, bw - bw // 2 - 1)]
+            if both or bw < bh:
+                ys = [(y0, bh // 2), (y0 + bh // 2 + 1, bh - bh // 2 - 1)]
+            for xa, xl in xs:
+                for ya, yl in ys:
+                    if xl > 0 and yl > 0:
+                        boxes.append((xa, ya, xl, yl))
+                        inner += xl * yl
+        ns, nb = 2 * (bw * bh - inner), 2 * around
+        total += ns * ns + 2 * ns * nb
+    return total
 
 
 def relax_work(c, fp32):
     """Per launch of the relaxation kernel: bytes the method must move (the
-    factor read by the forward and the back substitution, r read twice,
-    delta written) and flops (two FMAs per factor entry and pass)."""
+    factor read once, r read twice, delta written) and flops (one FMA per
+    factor entry)."""
     esz = 4 if fp32 else 8
     ent = 0
     nodes = c.nx * c.ny
     for Iy in range(-(-c.ny // c.sy)):
         for Ix in range(-(-c.nx // c.sx)):
-            w = min(c.sx, c.nx - Ix * c.sx)
-            h = min(c.sy, c.ny - Iy * c.sy)
-            ent += factor_entries(2 * w, h)
-    bytes_ = 2 * ent * esz + nodes * (32 + (8 if fp32 else 16))
-    flops = 4 * ent
-    return bytes_, flops
+            ent += dissection_entries(min(c.sx, c.nx - Ix * c.sx), min(c.sy, c.ny - Iy * c.sy))
+    return ent * esz + nodes * (32 + (8 if fp32 else 16)), 2 * ent
 
 
 def residual_work(c, fp32):
@@ -376,12 +392,10 @@ def run_ncu_case(args):
     c = case()
     ctx = capi.hms_context_create(0)
     prec = capi.HMS_FP64 if args.ncu_case == "fp64" else capi.HMS_MIXED
-    # the relaxation at the launch shape the autotuner picks on this workload
-    # (256 threads, one copy per matrix; the balanced schedule in FP64, one CTA
-    # per set in FP32), fixed so that no probe launches run
+    # the relaxation at the launch shape the autotuner picks on this workload,
+    # fixed so that no probe launches run
     pr = capi.hms_problem_create(ctx, c.nx, c.ny, c.sx, c.sy, ea=c.ea_array(), precision=prec, tol=0.0,
-                                 max_iter=args.ncu_iters, relax_threads=256, relax_copies=1,
-                                 relax_balance=2 if prec == capi.HMS_FP64 else 1)
+                                 max_iter=args.ncu_iters, relax_threads=256, relax_copies=1)
     p = c.load_array().reshape(1, -1)
     u = np.empty_like(p)
     capi.hms_solve(ctx, pr, p, u, allow_no_convergence=True)
@@ -922,10 +936,9 @@ def run_ours(args, rank, world, local_rank):
         prp = make(prec, profile=1)
         capi.hms_solve(ctx, prp, p_dev, u_dev, iters=its)
         kt = capi.hms_kernel_times(prp)
-        balanced = capi.hms_problem_relax_balanced(prp) == 1
         capi.hms_problem_destroy(prp)
         fp32 = prec == capi.HMS_MIXED
-        kname = ("k_relax_sched<{}>" if balanced else "k_relax<{}>").format("float" if fp32 else "double")
+        kname = "k_rtree<{}>".format("float" if fp32 else "double")
         ms, n = kt["relax"]
         b, fl = relax_work(c, fp32)
         avg = ms / max(n, 1)
@@ -948,7 +961,7 @@ def run_ours(args, rank, world, local_rank):
         roof.update({"algorithmic_bytes": b, "algorithmic_flops": fl, "avg_launch_ms": avg, "launches": n,
                      "avg_launch_ms_source": "profile pass: one solve of the same workload with options.profile "
                                              "= 1 (CUDA events on the context stream around every kernel)",
-                     "traffic": traffic_for(roof["kernel"], WORKLOAD, "relax.cu")})
+                     "traffic": traffic_for(roof["kernel"], WORKLOAD, "relax_tree.cu")})
         rb, _ = residual_work(c, fp32)
         rms, rn = kt["update_residual"]
         ravg = rms / max(rn, 1)
@@ -964,12 +977,10 @@ def run_ours(args, rank, world, local_rank):
         rooflines[name] = roof
 
     # kernels launched per solve: graph batches of 16 iterations, each iteration
-    # 10 kernels (residual, relaxation, assembly, band, diagonal, set drops,
-    # scaling, the two sides' bands, two-sided factor, block inverses) +
-    # coarse_solves solves + (coarse_solves - 1) refinement residuals (5 solves
-    # on the FP64 path), plus 1 load-norm kernel
+    # 10 kernels (residual, relaxation, assembly, the scaled system's diagonal and
+    # rows, four levels of fronts, all solves), plus 1 load-norm kernel
     batches = math.ceil((nit64 + 1) / 16)
-    per_iter = 10 + 5 + 4
+    per_iter = 10
     launches = args.steps * (batches * 16 * per_iter + 1)
 
     # ---- serving (continuous batching under the HBM budget), a bounded run ----

@@ -116,17 +116,20 @@ typedef struct {
                                 row, one CTA per front, fronts of 300 or more unknowns
                                 by many CTAs (set grids of any width, up to the 350 x
                                 350 sets of a 1e9-DOF lattice) */
-  int32_t relax_threads;     /* compute threads per CTA of the relaxation (Eqs. 11-13; one more
-                                warp issues its copies): 64, 128 or 256, or
+  int32_t relax_threads;     /* compute threads per CTA of the relaxation (Eqs. 11-13; the row
+                                substitution has one more warp that issues its copies): 64,
+                                128 or 256, or
                                 0 = autotuned: the first problem of a set-tile shape and
                                 precision on a context times each size on its own factors
                                 and the context keeps the fastest for that shape.  Results
                                 are bitwise the same for every size */
-  int32_t relax_copies;      /* bulk copies per factor matrix in the FP64 relaxation: 1, or
-                                2 (the rows of the outer and of the inner row pairs apart,
-                                half the shared memory per CTA, so two CTAs share an SM;
-                                even set widths >= 6 only), or 0 = with relax_threads = 0
-                                timed together with it, else 1.  Same results either way */
+  int32_t relax_copies;      /* shared memory per CTA of the FP64 relaxation: 1 or 2.  Row
+                                substitution: 1 or 2 bulk copies per factor matrix (2: the
+                                rows of the outer and of the inner row pairs apart, half the
+                                shared memory, so two CTAs share an SM); nested dissection:
+                                2 holds two ring slots per stream instead of three.  2 for
+                                even set widths >= 6 only; 0 = with relax_threads = 0 timed
+                                together with it, else 1.  Same results either way */
   int32_t relax_overlap;     /* extended relaxation region (Sec. 2.2, the region around a
                                 set in Fig. 1): each set relaxes together with the nodes
                                 within relax_overlap nodes of its tile (clipped to the
@@ -164,8 +167,15 @@ typedef struct {
                                 9-11 clear.  The increments equal the per-set ones up to
                                 rounding (another order of the sums) */
   int32_t relax_balance;     /* schedule of the relaxation with per-set factors:
-                                1 = one CTA per set (sets in waves of the SM count);
-                                2 = balanced: one persistent CTA per SM (cooperative
+                                0 = one CTA per set (sets in waves of the SM count), its
+                                nodes ordered by nested dissection: for set tiles of more
+                                than 64 nodes, unless its padded factors take 4 GB more
+                                than those of the row substitution; else, with
+                                relax_threads = 0, the faster of 1 and 2 by timing where
+                                both apply, else 1;
+                                1 = substitution row by row of the lattice, one CTA per
+                                set;
+                                2 = row substitution, balanced: one persistent CTA per SM (cooperative
                                 launch), each running an equal share of all sets'
                                 substitution steps, a set cut between two CTAs at a step
                                 whose state is in device memory (McNaughton's wrap-around
@@ -174,10 +184,9 @@ typedef struct {
                                 Needs more sets than SMs, none costing more than an SM's
                                 share, relax_threads 0 or 256, relax_copies 0 or 1,
                                 relax_overlap = 0 and class_factors = 0 (else
-                                HMS_ERR_ARG);
-                                0 = with relax_threads = 0 timed together with the CTA
-                                sizes where it applies, else 1.  Results are bitwise the
-                                same either way */
+                                HMS_ERR_ARG).
+                                Results of 1 and 2 are bitwise the same; nested dissection
+                                agrees with them up to rounding (other sums) */
 } hms_options;
 
 /* Context: one device, one CUDA stream.  device = CUDA ordinal. */

@@ -70,6 +70,11 @@ struct hms_problem {
   float* f32 = nullptr;
   bool cls = false;
   ClassPlanDev cpd;
+  // nested dissection of every set (relax_tree.cu): f64 / f32 in its layout (set_off),
+  // the lists of the region shapes
+  bool rtree = false;
+  RtView rt;
+  size_t rt_smem[3] = {0, 0, 0};  // by copies per matrix
   // force-controlled relaxation (q = 12): cut-free set factors with pinned DOFs,
   // supports | pins, per-set projection onto the free rigid motions (force.cu)
   double* f64F = nullptr;
@@ -247,6 +252,9 @@ cudaError_t launch_relax_main(hms_problem* pr, cudaStream_t s, const IterCtl* ct
   if (pr->cls)
     return launch_relax_class(s, pr->lv, pr->cpd, pr->f64, pr->f32, pr->r, pr->delta, pr->P, pr->yscratch, ctl,
                               pr->err, pr->relax_wait0);
+  if (pr->rtree)
+    return launch_rtree(s, pr->lv, pr->rt, pr->f64, pr->f32, pr->r, pr->delta, pr->P, ctl, pr->err,
+                        pr->relax_threads, pr->relax_chunks, pr->rt_smem[pr->relax_chunks], pr->relax_wait0);
   if (pr->relax_sched)
     return launch_relax_sched(s, pr->lv, pr->set_off, pr->f64, pr->f32, pr->r, pr->delta, pr->P, pr->yscratch, ctl,
                               pr->err, pr->sched_segs, pr->sched_cta, pr->sched_flags, pr->sched_grid,
@@ -283,8 +291,10 @@ cudaError_t launch_force_relax(hms_problem* pr, cudaStream_t s, const IterCtl* c
   const LatView& lv = pr->lv;
   cudaError_t e = launch_force_in(s, lv, pr->r, pr->Mforce, pr->fixF, pr->rproj, ctl);
   if (e != cudaSuccess) return e;
-  e = launch_relax(s, lv, pr->set_off, pr->f64F, pr->f32F, pr->rproj, pr->delta_rf, nullptr, pr->yscratch, ctl,
-                   pr->err, pr->relax_threads, pr->relax_chunks, pr->relax_wait0);
+  e = pr->rtree ? launch_rtree(s, lv, pr->rt, pr->f64F, pr->f32F, pr->rproj, pr->delta_rf, nullptr, ctl, pr->err,
+                               pr->relax_threads, pr->relax_chunks, pr->rt_smem[pr->relax_chunks], pr->relax_wait0)
+                : launch_relax(s, lv, pr->set_off, pr->f64F, pr->f32F, pr->rproj, pr->delta_rf, nullptr, pr->yscratch,
+                               ctl, pr->err, pr->relax_threads, pr->relax_chunks, pr->relax_wait0);
   if (e != cudaSuccess) return e;
   return launch_force_out(s, lv, pr->delta_rf, fp32(pr), pr->Mforce, pr->r, pr->P, ctl);
 }
@@ -531,6 +541,74 @@ void class_plan_build(const LatView& lv, const std::vector<uint8_t>& fix, int ts
   }
 }
 
+// The region shapes of a lattice's sets for the relaxation by nested dissection:
+// each set's shape and first factor element, the shapes' lists.
+struct RtPlanHost {
+  std::vector<RtShapeHost> shapes;
+  std::vector<int> sid;
+  long long elems = 0;          // of all sets' factors
+  long long scratch = 0;        // doubles per CTA of the factorisation
+  int smax = 0;
+  size_t smem[3] = {0, 0, 0};   // of the relaxation, by copies per matrix
+};
+// Whether the relaxation runs by nested dissection: with per-set factors, the
+// automatic schedule (relax_balance names a schedule of the row substitution)
+// and set tiles of more than 64 nodes whose lists and vectors fit.  Tiles of up to
+// 8 x 8 nodes take the row substitution (30 dependent steps of 16 unknowns, in a
+// few KB): at 9 x 8 nodes nested dissection takes 24 us for 41 (FP64, 18 x 15
+// sets).  Padding to 32 lanes makes small tiles' factors larger than the
+// substitution's (9 x 8 nodes: 8 K entries for 6 K; 64 x 64: 1.2 M for 2.1 M);
+// where that would cost more than RT_MORE_BYTES in all, a lattice of millions of
+// nodes, the smaller form stays, so that what fits the device still does.
+constexpr long long RT_MORE_BYTES = 4LL << 30;
+bool rt_plan(const LatView& lv, const hms_options* o, bool f32, int maxsm, RtPlanHost* P) {
+  *P = RtPlanHost();
+  if (o->class_factors || o->relax_balance != 0) return false;
+  if ((long long)std::min(lv.sx, lv.nx) * std::min(lv.sy, lv.ny) <= 64) return false;
+  std::map<std::pair<int, int>, int> ids;
+  long long rows = 0;  // the row substitution's factor elements
+  P->sid.resize(lv.M);
+  for (int I = 0; I < lv.M; ++I) {
+    const Region R = relax_region(lv, I);
+    const auto it = ids.find({R.w, R.h});
+    if (it != ids.end()) {
+      P->sid[I] = it->second;
+    } else {
+      if ((long long)R.w * R.h > 0x7fff) return false;
+      P->shapes.emplace_back();
+      RtShapeHost& S = P->shapes.back();
+      if (!rt_shape_build(R.w, R.h, &S)) return false;
+      if (rt_smem_bytes(S, f32, 1) + 1024 > (size_t)maxsm || rt_factor_smem_bytes(S.smax) + 1024 > (size_t)maxsm)
+        return false;
+      for (int k = 1; k <= 2; ++k) P->smem[k] = std::max(P->smem[k], rt_smem_bytes(S, f32, k));
+      P->smax = std::max(P->smax, S.smax);
+      P->scratch = std::max(P->scratch, (long long)S.u_max + 2LL * S.bs_max);
+      P->sid[I] = ids[{R.w, R.h}] = (int)P->shapes.size() - 1;
+    }
+    P->elems += P->shapes[P->sid[I]].elems;
+    rows += set_factor_stride(2 * R.w, R.h);
+  }
+  return (P->elems - rows) * (f32 ? 4 : 8) <= RT_MORE_BYTES;
+}
+
+// CTAs of the sets' factorisation by nested dissection, those of them that work
+// in the setup scratch (the size the row substitution's factorisation takes), and
+// the doubles of the others' work space, which the problem keeps: at 64 x 64
+// nodes 1 MB per SM beside factors of 5 or 10 MB per set.
+struct RtSetup {
+  int grid = 0, first = 0;
+  long long own = 0;
+};
+RtSetup rt_setup(const RtPlanHost& P, int M, int nsm) {
+  RtSetup S;
+  const long long room = (long long)std::max(1, std::min(M, nsm)) * b_size(MAX_NB);
+  const int fit = (int)std::min<long long>(room / std::max(P.scratch, 1LL), 2LL * nsm);
+  S.grid = std::max(1, std::min(M, std::max(fit, nsm)));
+  S.first = std::min(S.grid, fit);
+  S.own = (S.grid - S.first) * P.scratch;
+  return S;
+}
+
 // Nested dissection over the set grid: as a tree of fronts swept in the shared
 // memory of one cluster each (coarse_tree.cu) where they fit, else panel by
 // panel from device memory (coarse_nd.cu), if every front fits the factor
@@ -602,6 +680,7 @@ hms_status hms_context_create(int32_t device, hms_context** out) {
   if (e == cudaSuccess) e = configure_setup(maxsm);
   if (e == cudaSuccess) e = configure_relax(maxsm);
   if (e == cudaSuccess) e = configure_relax_class(maxsm);
+  if (e == cudaSuccess) e = configure_relax_tree(maxsm);
   if (e == cudaSuccess) e = configure_coarse_assemble(maxsm);
   if (e == cudaSuccess) e = configure_coarse_solve(maxsm);
   if (e == cudaSuccess) e = configure_coarse_factor_cl(maxsm);
@@ -684,6 +763,9 @@ hms_status hms_problem_clone(hms_problem* src, hms_problem** out) {
   pr->fix = src->fix;
   pr->rep = src->rep;
   pr->set_off = src->set_off;
+  pr->rtree = src->rtree;
+  pr->rt = src->rt;
+  for (int k = 0; k < 3; ++k) pr->rt_smem[k] = src->rt_smem[k];
   pr->f64 = src->f64;
   pr->f32 = src->f32;
   pr->cls = src->cls;
@@ -835,7 +917,7 @@ static cudaError_t alloc_instance(hms_problem* pr) {
   {
     const size_t esz = fp32(pr) ? sizeof(float) : sizeof(double);
     const size_t ybytes = pr->cls ? (size_t)pr->cpd.nitems * pr->cpd.ystride * esz
-                                  : (size_t)lv.M * relax_y_stride(lv) * esz;
+                                  : (pr->rtree ? 0 : (size_t)lv.M * relax_y_stride(lv) * esz);
     unsigned char* ys;
     CKI(palloc(pr, &ys, ybytes));
     pr->yscratch = ys;
@@ -1016,7 +1098,8 @@ static cudaError_t autotune_relax(hms_problem* pr, int copies, bool try_sched) {
   // the relaxation region's overlap changes the factors' shapes and rules out
   // two copies per matrix, so it is part of the key; so is the set count
   // where the balanced schedule applies (its gain depends on it)
-  const auto key = std::make_tuple(std::min(lv.sx, lv.nx), std::min(lv.sy, lv.ny), pr->precision * 10 + copies,
+  const auto key = std::make_tuple(std::min(lv.sx, lv.nx), std::min(lv.sy, lv.ny),
+                                   pr->precision * 10 + copies + (pr->rtree ? 100 : 0),
                                    lv.ov, sched_ok ? lv.M : 0);
   const auto it = c->relax_tuned.find(key);
   if (it != c->relax_tuned.end()) {
@@ -1047,6 +1130,9 @@ static cudaError_t autotune_relax(hms_problem* pr, int copies, bool try_sched) {
     if (nc == 0)
       return launch_relax_sched(s, lv, pr->set_off, pr->f64, pr->f32, pr->r, pr->delta, pr->P, pr->yscratch,
                                 nullptr, pr->err, pr->sched_segs, pr->sched_cta, pr->sched_flags, pr->sched_grid);
+    if (pr->rtree)
+      return launch_rtree(s, lv, pr->rt, pr->f64, pr->f32, pr->r, pr->delta, pr->P, nullptr, pr->err, nt, nc,
+                          pr->rt_smem[nc], -1);
     return launch_relax(s, lv, pr->set_off, pr->f64, pr->f32, pr->r, pr->delta, pr->P, pr->yscratch, nullptr,
                         pr->err, nt, nc);
   };
@@ -1211,6 +1297,10 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
     lv.kbar = pr->kbar;
   }
   ClassPlanHost cph;  // with class factors
+  RtPlanHost rtp;     // with the relaxation by nested dissection
+  pr->rtree = rt_plan(lv, o, fp32(pr), maxsm, &rtp);
+  RtSetup rtsu;
+  double* rtwork = nullptr;
   {
     // representing node of each set: the centroid of its nodes (Eq. 10)
     std::vector<double2> rp(lv.M);
@@ -1224,13 +1314,13 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
       rp[I].x = lv.L * ((double)i0 + 0.5 * (double)(w - 1) + 0.5 * (double)nodd / (double)h);
       rp[I].y = lv.L * SQ3_2 * ((double)j0 + 0.5 * (double)(h - 1));
       const Region R = relax_region(lv, I);  // the factor is the relaxation region's
-      so[I + 1] = so[I] + set_factor_stride(2 * R.w, R.h);
+      so[I + 1] = so[I] + (pr->rtree ? rtp.shapes[rtp.sid[I]].elems : set_factor_stride(2 * R.w, R.h));
     }
     CKP(salloc(pr, &pr->rep, lv.M));
     CKP(cudaMemcpy(pr->rep, rp.data(), lv.M * sizeof(double2), cudaMemcpyHostToDevice));
     lv.rep = pr->rep;
     rep_host = rp;
-    size_t fsz = (size_t)so[lv.M];
+    size_t fsz = (size_t)so[lv.M] + (pr->rtree ? RT_PAD : 0);
     if (o->class_factors) {
       pr->cls = true;
       class_plan_build(lv, fix_host, class_sets_per_cta(fp32(pr)), &cph);
@@ -1259,6 +1349,41 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
     } else {
       CKP(salloc(pr, &pr->set_off, lv.M + 1));
       CKP(cudaMemcpy(pr->set_off, so.data(), (lv.M + 1) * sizeof(long long), cudaMemcpyHostToDevice));
+    }
+    if (pr->rtree) {
+      std::vector<RtShape> sv;
+      cudaError_t e = cudaSuccess;
+      auto up = [&](const auto& v, auto** dst, size_t per) {  // per: elements of v in one of dst
+        using D = std::remove_reference_t<decltype(**dst)>;
+        std::remove_const_t<D>* q = nullptr;
+        if (e == cudaSuccess) e = salloc(pr, &q, v.size() / per);
+        if (e == cudaSuccess) e = cudaMemcpy(q, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
+        *dst = q;
+      };
+      for (const RtShapeHost& S : rtp.shapes) {
+        RtShape d{};
+        d.w = S.w, d.h = S.h, d.nn = S.nn, d.nup = S.nup, d.nphase = S.nphase, d.nnode = (int)S.nodes.size();
+        d.xs = S.xs, d.stg = S.stg, d.u_max = S.u_max, d.bs_max = S.bs_max;
+        d.npanel = S.npanel, d.lbytes = (int)rt_list_bytes(S);
+        for (int v = 0; v <= RT_STREAMS; ++v) d.vrow[v] = S.vrow[v];
+        up(S.inv, &d.inv, 1);
+        up(S.desc, &d.desc, 2);
+        up(S.lane, &d.lane, 8);
+        up(S.defer, &d.defer, 2);
+        up(S.dlist, &d.dlist, 1);
+        up(S.nodes, &d.nodes, 1);
+        up(S.front, &d.front, 1);
+        up(S.cmap, &d.cmap, 1);
+        up(S.place, &d.place, 1);
+        sv.push_back(d);
+      }
+      up(sv, &pr->rt.shapes, 1);
+      up(rtp.sid, &pr->rt.sid, 1);
+      CKP(e);
+      pr->rt.off = pr->set_off;
+      rtsu = rt_setup(rtp, lv.M, c->nsm);
+      if (rtsu.own > 0) CKP(salloc(pr, &rtwork, (size_t)rtsu.own));
+      for (int k = 0; k < 3; ++k) pr->rt_smem[k] = rtp.smem[k];
     }
     if (fp32(pr)) {
       CKP(salloc(pr, &pr->f32, fsz));
@@ -1357,13 +1482,20 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
       cudaFree(std64);
       cudaFree(ro_d);
       cudaFree(reps_d);
+    } else if (pr->rtree) {
+      e = launch_rtree_factor(s, lv, pr->rt, pr->f64, pr->f32, scratch, rtsu.first, rtwork, rtp.scratch, rtsu.grid,
+                              rtp.smax, pr->err, false);
     } else {
       e = launch_set_factor(s, lv, pr->set_off, pr->f64, pr->f32, scratch, grid, pr->err);
     }
     if (e == cudaSuccess && force) {
       LatView lvF = lv;  // the cut-free sets with their pinned DOFs marked as constrained
       lvF.fix = pr->fixF;
-      e = launch_set_factor(s, lvF, pr->set_off, pr->f64F, pr->f32F, scratch, grid, pr->err, true);
+      if (pr->rtree)
+        e = launch_rtree_factor(s, lvF, pr->rt, pr->f64F, pr->f32F, scratch, rtsu.first, rtwork, rtp.scratch,
+                                rtsu.grid, rtp.smax, pr->err, true);
+      else
+        e = launch_set_factor(s, lvF, pr->set_off, pr->f64F, pr->f32F, scratch, grid, pr->err, true);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFree(scratch);
@@ -1407,7 +1539,7 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
     pr->relax_threads = o->relax_threads;
     pr->relax_chunks = 1;
   } else {
-    CKP(autotune_relax(pr, o->relax_copies, o->relax_balance == 0));
+    CKP(autotune_relax(pr, o->relax_copies, o->relax_balance == 0 && !pr->rtree));
   }
   if (!pr->profile) {
     hms_status st = build_graph(pr);
@@ -1750,6 +1882,7 @@ static BatchProb batch_prob_of(const hms_problem* pr) {
   q.f64 = pr->f64;
   q.f32 = pr->f32;
   q.yscratch = pr->yscratch;
+  q.rt = pr->rt;
   q.slots_base = pr->slots_base;
   q.slots_it = pr->slots_it;
   q.band = pr->band;
@@ -1772,7 +1905,7 @@ static BatchProb batch_prob_of(const hms_problem* pr) {
 
 // Work lists of the batched launches for the running problems, one after
 // another in one array; off[k] .. off[k + 1] is kernel k's list.
-enum BatchList { BL_K1 = 0, BL_SETS, BL_BAND, BL_DIAG, BL_DROPS, BL_SCALE, BL_ONE, BL_BLOCKINV, BL_CRES, BL_COUNT };
+enum BatchList { BL_K1 = 0, BL_SETS, BL_RT, BL_RS, BL_BAND, BL_DIAG, BL_DROPS, BL_SCALE, BL_ONE, BL_BLOCKINV, BL_CRES, BL_COUNT };
 
 // The running problems with the tree factor: their sets, their nodes level by
 // level (TreeItem), and the problems by the CTAs of their solves.
@@ -1829,7 +1962,7 @@ static void build_lists(const std::vector<hms_problem*>& probs, const std::vecto
     off[k] = (int)items.size();
     for (int i : run) {
       const hms_problem* pr = probs[i];
-      if (pr->tree && k != BL_K1 && k != BL_SETS) continue;  // the band's steps
+      if (pr->tree && k >= BL_BAND) continue;  // the band's steps
       const LatView& lv = pr->lv;
       auto grid = [&](int g) {
         for (int b = 0; b < g; ++b) items.push_back(BatchItem{i, b, 0, g, 1});
@@ -1842,6 +1975,12 @@ static void build_lists(const std::vector<hms_problem*>& probs, const std::vecto
           break;
         }
         case BL_SETS: grid(lv.M); break;
+        case BL_RT:  // the sets relaxed by nested dissection, and by row substitution
+          if (pr->rtree) grid(lv.M);
+          break;
+        case BL_RS:
+          if (!pr->rtree) grid(lv.M);
+          break;
         case BL_BAND: grid(coarse_grid_for((size_t)pr->n_c * (pr->bw + 1))); break;
         case BL_DIAG: grid(coarse_grid_for((size_t)pr->n_c)); break;
         case BL_DROPS: grid(set_drops_blocks(lv.M)); break;
@@ -1886,11 +2025,12 @@ static hms_status solve_batch_lockstep(hms_context* c, int32_t count, hms_proble
   int rchunks = 2;
   for (hms_problem* pr : probs) rchunks = std::min(rchunks, pr->relax_chunks);
   int stages = 3;
-  size_t sm_relax = 0, sm_slots = 0, sm_factor = 0, sm_solve = 0;
+  size_t sm_relax = 0, sm_rt = 0, sm_slots = 0, sm_factor = 0, sm_solve = 0;
   for (hms_problem* pr : probs)
     if (!pr->tree) stages = std::min(stages, pr->big_stages);
   for (hms_problem* pr : probs) {
-    sm_relax = std::max(sm_relax, relax_smem_bytes(pr->lv, f32, rchunks));
+    if (pr->rtree) sm_rt = std::max(sm_rt, pr->rt_smem[rchunks]);
+    else sm_relax = std::max(sm_relax, relax_smem_bytes(pr->lv, f32, rchunks));
     sm_slots = std::max(sm_slots, coarse_slots_smem(pr->lv));
     if (pr->tree) continue;
     sm_factor = std::max(sm_factor, coarse_factor_smem_bytes(pr->n_c, pr->bw, false));
@@ -1997,7 +2137,8 @@ static hms_status solve_batch_lockstep(hms_context* c, int32_t count, hms_proble
       cudaError_t e = cudaSuccess;
       for (int k = 0; k < 16 && e == cudaSuccess; ++k) {
         e = launch_batch_update_residual(s, f32, P, L(BL_K1), N(BL_K1), k);
-        if (e == cudaSuccess) e = launch_batch_relax(s, f32, rthreads, rchunks, sm_relax, P, L(BL_SETS), N(BL_SETS));
+        if (e == cudaSuccess) e = launch_batch_rtree(s, f32, rthreads, rchunks, sm_rt, P, L(BL_RT), N(BL_RT));
+        if (e == cudaSuccess) e = launch_batch_relax(s, f32, rthreads, rchunks, sm_relax, P, L(BL_RS), N(BL_RS));
         if (e == cudaSuccess) e = launch_batch_slots(s, f32, sm_slots, P, L(BL_SETS), N(BL_SETS));
         if (e == cudaSuccess) e = launch_tree_system(s, NMODES, true, TP, TI, tl.nsets, true);
         for (size_t h = 0; h < tl.T.size() && e == cudaSuccess; ++h) {
@@ -2338,6 +2479,7 @@ bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options
   const size_t esz = fp32(&pr) ? 4 : 8;
   const size_t nband = n_c * (pr.bw + 1);
   size_t fac = 0, ybytes = 0, plan_bytes = 0, setup_bytes = 0;
+  RtPlanHost rtp;
   if (o->class_factors) {
     ClassPlanHost cph;
     class_plan_build(lv, fix_pattern(d), class_sets_per_cta(fp32(&pr)), &cph);
@@ -2348,6 +2490,11 @@ bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options
     const size_t nc = cph.rep.size();
     for (size_t t = 0; t < nc; ++t) setup_bytes += (size_t)set_factor_stride(2 * cph.info[t].w, cph.info[t].h) * 8;
     setup_bytes += (nc + 1) * 8 + nc * 4;
+  } else if (rt_plan(lv, o, fp32(&pr), maxsm, &rtp)) {
+    fac = (size_t)rtp.elems + RT_PAD;
+    plan_bytes = (M + 1) * 8 + M * 4 + rtp.shapes.size() * sizeof(RtShape);
+    for (const RtShapeHost& S : rtp.shapes) plan_bytes += rt_shape_bytes(S);
+    plan_bytes += (size_t)rt_setup(rtp, lv.M, c->nsm).own * 8;
   } else {
     for (int I = 0; I < lv.M; ++I) {
       const Region R = relax_region(lv, I);
@@ -2386,7 +2533,8 @@ bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options
     }
   b += n_c * 4 + 32 + (size_t)std::max(update_residual_blocks(lv), 1024) * 3 * 8 + 4 + sizeof(IterCtl) + 4 + 32;
   if (o->record_history) b += 3 * ((size_t)o->max_iter + 1) * 8;
-  if (!o->class_factors && o->relax_overlap == 0 && o->relax_balance != 1 && lv.M > c->nsm)
+  const bool rtree = !rtp.sid.empty() && rtp.elems > 0 && ybytes == 0 && !o->class_factors;
+  if (!o->class_factors && !rtree && o->relax_overlap == 0 && o->relax_balance != 1 && lv.M > c->nsm)
     b += ((size_t)lv.M + 2 * c->nsm) * sizeof(RelaxSeg) + ((size_t)c->nsm + 1) * 4 + (size_t)lv.M * 4;  // schedule
   *inst = b;
   *scratch = (size_t)std::max(1, std::min(lv.M, c->nsm)) * b_size(MAX_NB) * 8 + setup_bytes;

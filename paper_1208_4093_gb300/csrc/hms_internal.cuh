@@ -259,6 +259,61 @@ cudaError_t launch_relax(cudaStream_t s, const LatView& lv, const long long* set
                          double* P, void* yscratch, const IterCtl* ctl, int* err, int threads, int chunks,
                          int wait0 = -1);
 size_t relax_smem_bytes(const LatView& lv, bool fp32, int chunks = 1);
+// relax_tree.cu: the relaxation by nested dissection of every set.  The lists of
+// one region shape (w x h nodes), shared by all sets of that shape.
+constexpr int RT_STREAMS = 8;
+struct RtNode {
+  int ns, nb, nchild;           // own and boundary region nodes, children
+  int f_off, p_off, u_off;      // its place in front, place and the update scratch
+  int c_u[4], c_nb[4], c_map[4];  // the children's updates: scratch offset, unknowns, front -> boundary map
+};
+struct RtShape {
+  int w, h, nn, nup, nphase, nnode, xs, stg;  // (stg: inputs of a panel, at most)
+  int npanel, lbytes;             // panels; bytes of desc with the panel numbers behind it
+  int u_max, bs_max;              // doubles of the factor's scratch: updates, A_BS
+  int vrow[RT_STREAMS + 1];       // first matrix column of every stream
+  const unsigned short* inv;      // region node -> its place in the tree's order
+  const int2* desc;               // per panel: groups of four columns per segment (8 bits each); inputs, segments;
+                                  // then [phase][stream]: first panel
+  const int4* lane;               // per panel 32 + 32 of eight 16-bit numbers: per lane segment starts, unknown,
+                                  // deferred slot; then its inputs lane, lane + 32, ...
+  const int2* defer;              // per phase: deferred outputs (first in dlist, count)
+  const unsigned short* dlist;
+  const RtNode* nodes;            // children first
+  const unsigned short* front;    // per node: region nodes of S, then B
+  const short* cmap;
+  const int* place;               // per tree node and front unknown: matrix column 32 + lane of its row's start
+};
+struct RtView {
+  const RtShape* shapes = nullptr;
+  const int* sid = nullptr;        // shape of every set
+  const long long* off = nullptr;  // first element of every set's factor
+};
+struct RtShapeHost {
+  int w = 0, h = 0, nn = 0, nup = 0, nphase = 0, npanel = 0, xs = 0, stg = 0, smax = 0, u_max = 0, bs_max = 0;
+  long long elems = 0;  // of a set's factor
+  int vrow[RT_STREAMS + 1] = {};
+  std::vector<unsigned short> inv, lane, dlist, front;
+  std::vector<int> desc, vp, defer, place;
+  std::vector<RtNode> nodes;
+  std::vector<short> cmap;
+};
+// elements behind the last set's factor that the streams' fetches may touch
+constexpr int RT_PAD = 4096;
+// The lists of a region shape; false if it does not fit their 16-bit indices
+// or a panel's inputs.
+bool rt_shape_build(int w, int h, RtShapeHost* P);
+size_t rt_shape_bytes(const RtShapeHost& P);
+size_t rt_list_bytes(const RtShapeHost& P);
+size_t rt_smem_bytes(const RtShapeHost& P, bool fp32, int copies);
+size_t rt_factor_smem_bytes(int smax);
+cudaError_t launch_rtree_factor(cudaStream_t s, const LatView& lv, const RtView& rt, double* f64, float* f32,
+                                double* scratch, int first, double* work, long long stride, int grid, int smax, int* err,
+                                bool cut);
+cudaError_t launch_rtree(cudaStream_t s, const LatView& lv, const RtView& rt, const double* f64, const float* f32,
+                         const double2* r, void* delta, double* P, const IterCtl* ctl, int* err, int threads,
+                         int copies, size_t smem, int wait0);
+cudaError_t configure_relax_tree(int max_smem);
 // relax_class.cu: the relaxation with class factors (sets per CTA: 64 FP32, 32 FP64)
 int class_sets_per_cta(bool fp32);
 size_t relax_class_smem(size_t slot_elems, int nb8max, bool fp32);
@@ -339,6 +394,7 @@ struct BatchProb {
   const double* f64;
   const float* f32;
   void* yscratch;
+  RtView rt;
   const double* slots_base;
   double* slots_it;
   double* band;
@@ -364,6 +420,8 @@ struct BatchItem {
 cudaError_t launch_batch_update_residual(cudaStream_t s, bool fp32, const BatchProb* P, const BatchItem* it, int n,
                                          int k);
 cudaError_t launch_batch_relax(cudaStream_t s, bool fp32, int threads, int chunks, size_t smem, const BatchProb* P,
+                               const BatchItem* it, int n);
+cudaError_t launch_batch_rtree(cudaStream_t s, bool fp32, int threads, int copies, size_t smem, const BatchProb* P,
                                const BatchItem* it, int n);
 cudaError_t launch_batch_slots(cudaStream_t s, bool fp32, size_t smem, const BatchProb* P, const BatchItem* it,
                                int n);

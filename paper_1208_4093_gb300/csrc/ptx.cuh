@@ -44,6 +44,17 @@ __device__ inline void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint
       : "memory");
 }
 
+// 16 bytes global -> shared by the issuing thread, past L1; groups of them are
+// waited for in order by the same thread.
+__device__ inline void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ inline void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ inline void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 __device__ inline bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
