@@ -161,11 +161,13 @@ typedef struct {
                                 per-set factors would not fit in device memory: with a uniform
                                 EA, sets of the same width and height, parity of the first
                                 row, lattice edges touched and constrained DOFs have the same
-                                k^Inner, so each class is factored once and its sets are
-                                relaxed together, 64 (FP32) or 32 (FP64) right-hand sides per
-                                CTA.  Needs ea = NULL, relax_overlap = 0 and mode_mask bits
-                                9-11 clear.  The increments equal the per-set ones up to
-                                rounding (another order of the sums) */
+                                k^Inner, so each class is factored once and its sets share
+                                the factor: each set by nested dissection as with its own
+                                (FP64, and FP32 up to 26 sets per SM), or, with relax_balance
+                                = 1, set tiles of up to 64 nodes or more FP32 sets, 64 (FP32)
+                                or 32 (FP64) right-hand sides per CTA.  Needs ea = NULL,
+                                relax_overlap = 0 and mode_mask bits 9-11 clear.  The
+                                increments equal the per-set ones up to rounding */
   int32_t relax_balance;     /* schedule of the relaxation with per-set factors:
                                 0 = one CTA per set (sets in waves of the SM count), its
                                 nodes ordered by nested dissection: for set tiles of more

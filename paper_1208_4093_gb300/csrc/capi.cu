@@ -69,6 +69,7 @@ struct hms_problem {
   double* f64 = nullptr;
   float* f32 = nullptr;
   bool cls = false;
+  bool classes = false;  // class factors, in either form (cls: relax_class.cu; rtree: relax_tree.cu)
   ClassPlanDev cpd;
   // nested dissection of every set (relax_tree.cu): f64 / f32 in its layout (set_off),
   // the lists of the region shapes
@@ -546,7 +547,8 @@ void class_plan_build(const LatView& lv, const std::vector<uint8_t>& fix, int ts
 struct RtPlanHost {
   std::vector<RtShapeHost> shapes;
   std::vector<int> sid;
-  long long elems = 0;          // of all sets' factors
+  std::vector<long long> off;   // per set; sets of one class share a factor
+  long long elems = 0;          // of all factors
   long long scratch = 0;        // doubles per CTA of the factorisation
   int smax = 0;
   size_t smem[3] = {0, 0, 0};   // of the relaxation, by copies per matrix
@@ -561,13 +563,34 @@ struct RtPlanHost {
 // where that would cost more than RT_MORE_BYTES in all, a lattice of millions of
 // nodes, the smaller form stays, so that what fits the device still does.
 constexpr long long RT_MORE_BYTES = 4LL << 30;
-bool rt_plan(const LatView& lv, const hms_options* o, bool f32, int maxsm, RtPlanHost* P) {
+// With class factors (cph) a class's sets read one factor, mostly from the L2; in
+// FP32 up to RT_CLASS_SETS sets per SM, beyond which relax_class.cu's batches of
+// 64 sets fill the chip and each factor entry they load serves 64 sets (us, nested
+// dissection / batches: FP32, 32 x 32 nodes, 1015 sets 230 / 739, 4096 sets 796 /
+// 749, 16384 sets 3055 / 1491; 64 x 64 nodes, 256 sets 220 / 2941, 2304 sets 1576 /
+// 2981, 9216 sets 5847 / 3007; FP64, 32 x 32, 1015 sets 531 / 3065, 16384 sets 7212 /
+// 12189; 64 x 64, 256 sets 702 / 18405, 18432 sets 41293 / 73533).
+constexpr int RT_CLASS_SETS = 26;
+bool rt_plan(const LatView& lv, const hms_options* o, bool f32, int maxsm, int nsm, const ClassPlanHost* cph,
+             RtPlanHost* P) {
   *P = RtPlanHost();
-  if (o->class_factors || o->relax_balance != 0) return false;
+  if (o->relax_balance != 0) return false;
+  if (cph && f32 && lv.M > (long long)RT_CLASS_SETS * nsm) return false;
   if ((long long)std::min(lv.sx, lv.nx) * std::min(lv.sy, lv.ny) <= 64) return false;
   std::map<std::pair<int, int>, int> ids;
   long long rows = 0;  // the row substitution's factor elements
   P->sid.resize(lv.M);
+  P->off.resize(lv.M + 1);
+  std::vector<int> cls(lv.M);  // sets of equal factors: their number, by class or one by one
+  std::vector<long long> at;   // a factor's first element
+  if (cph) {
+    for (const ClassItem& it : cph->items)
+      for (int k = 0; k < it.count; ++k) cls[cph->sets[it.first + k]] = it.cls;
+    at.assign(cph->rep.size(), -1);
+  } else {
+    for (int I = 0; I < lv.M; ++I) cls[I] = I;
+    at.assign(lv.M, -1);
+  }
   for (int I = 0; I < lv.M; ++I) {
     const Region R = relax_region(lv, I);
     const auto it = ids.find({R.w, R.h});
@@ -585,9 +608,14 @@ bool rt_plan(const LatView& lv, const hms_options* o, bool f32, int maxsm, RtPla
       P->scratch = std::max(P->scratch, (long long)S.u_max + 2LL * S.bs_max);
       P->sid[I] = ids[{R.w, R.h}] = (int)P->shapes.size() - 1;
     }
-    P->elems += P->shapes[P->sid[I]].elems;
-    rows += set_factor_stride(2 * R.w, R.h);
+    if (at[cls[I]] < 0) {
+      at[cls[I]] = P->elems;
+      P->elems += P->shapes[P->sid[I]].elems;
+      rows += set_factor_stride(2 * R.w, R.h);
+    }
+    P->off[I] = at[cls[I]];
   }
+  P->off[lv.M] = P->elems;
   return (P->elems - rows) * (f32 ? 4 : 8) <= RT_MORE_BYTES;
 }
 
@@ -769,6 +797,7 @@ hms_status hms_problem_clone(hms_problem* src, hms_problem** out) {
   pr->f64 = src->f64;
   pr->f32 = src->f32;
   pr->cls = src->cls;
+  pr->classes = src->classes;
   pr->cpd = src->cpd;
   pr->f64F = src->f64F;
   pr->f32F = src->f32F;
@@ -1298,7 +1327,15 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
   }
   ClassPlanHost cph;  // with class factors
   RtPlanHost rtp;     // with the relaxation by nested dissection
-  pr->rtree = rt_plan(lv, o, fp32(pr), maxsm, &rtp);
+  if (o->class_factors) {
+    pr->classes = true;
+    class_plan_build(lv, fix_host, class_sets_per_cta(fp32(pr)), &cph);
+    if (relax_class_smem(cph.slot_elems, cph.nb8max, fp32(pr)) + 1024 > (size_t)maxsm) {
+      hms_problem_destroy(pr);
+      return fail(c, HMS_ERR_ARG, "set tile too large for the class-factor relaxation's shared memory");
+    }
+  }
+  pr->rtree = rt_plan(lv, o, fp32(pr), maxsm, c->nsm, o->class_factors ? &cph : nullptr, &rtp);
   RtSetup rtsu;
   double* rtwork = nullptr;
   {
@@ -1314,20 +1351,16 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
       rp[I].x = lv.L * ((double)i0 + 0.5 * (double)(w - 1) + 0.5 * (double)nodd / (double)h);
       rp[I].y = lv.L * SQ3_2 * ((double)j0 + 0.5 * (double)(h - 1));
       const Region R = relax_region(lv, I);  // the factor is the relaxation region's
-      so[I + 1] = so[I] + (pr->rtree ? rtp.shapes[rtp.sid[I]].elems : set_factor_stride(2 * R.w, R.h));
+      so[I + 1] = so[I] + set_factor_stride(2 * R.w, R.h);
     }
+    if (pr->rtree) so = rtp.off;
     CKP(salloc(pr, &pr->rep, lv.M));
     CKP(cudaMemcpy(pr->rep, rp.data(), lv.M * sizeof(double2), cudaMemcpyHostToDevice));
     lv.rep = pr->rep;
     rep_host = rp;
     size_t fsz = (size_t)so[lv.M] + (pr->rtree ? RT_PAD : 0);
-    if (o->class_factors) {
+    if (o->class_factors && !pr->rtree) {
       pr->cls = true;
-      class_plan_build(lv, fix_host, class_sets_per_cta(fp32(pr)), &cph);
-      if (relax_class_smem(cph.slot_elems, cph.nb8max, fp32(pr)) + 1024 > (size_t)maxsm) {
-        hms_problem_destroy(pr);
-        return fail(c, HMS_ERR_ARG, "set tile too large for the class-factor relaxation's shared memory");
-      }
       ClassPlanDev& cp = pr->cpd;
       ClassInfo* info;
       ClassItem* items;
@@ -1381,7 +1414,7 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
       up(rtp.sid, &pr->rt.sid, 1);
       CKP(e);
       pr->rt.off = pr->set_off;
-      rtsu = rt_setup(rtp, lv.M, c->nsm);
+      rtsu = rt_setup(rtp, pr->classes ? (int)cph.rep.size() : lv.M, c->nsm);
       if (rtsu.own > 0) CKP(salloc(pr, &rtwork, (size_t)rtsu.own));
       for (int k = 0; k < 3; ++k) pr->rt_smem[k] = rtp.smem[k];
     }
@@ -1483,8 +1516,19 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
       cudaFree(ro_d);
       cudaFree(reps_d);
     } else if (pr->rtree) {
-      e = launch_rtree_factor(s, lv, pr->rt, pr->f64, pr->f32, scratch, rtsu.first, rtwork, rtp.scratch, rtsu.grid,
-                              rtp.smax, pr->err, false);
+      int* reps_d = nullptr;  // a class's factor is its first set's
+      const int nc = (int)cph.rep.size();
+      if (pr->classes) {
+        e = cudaMalloc(&reps_d, nc * sizeof(int));
+        if (e == cudaSuccess) e = cudaMemcpy(reps_d, cph.rep.data(), nc * sizeof(int), cudaMemcpyHostToDevice);
+      }
+      if (e == cudaSuccess)
+        e = launch_rtree_factor(s, lv, pr->rt, pr->f64, pr->f32, scratch, rtsu.first, rtwork, rtp.scratch, rtsu.grid,
+                                rtp.smax, pr->err, false, reps_d, nc);
+      if (reps_d) {
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        cudaFree(reps_d);
+      }
     } else {
       e = launch_set_factor(s, lv, pr->set_off, pr->f64, pr->f32, scratch, grid, pr->err);
     }
@@ -1518,8 +1562,8 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
     hms_problem_destroy(pr);
     return fail(c, HMS_ERR_ARG, "relax_copies = 2 needs the FP64 path and even set widths >= 6");
   }
-  if (pr->cls) {
-    pr->relax_threads = 256;  // the class-factor kernel's fixed shape
+  if (pr->classes) {
+    pr->relax_threads = 256;  // the class-factor kernel's fixed shape, and the best or within 4 % by nested dissection
     pr->relax_chunks = 1;
   } else if (o->relax_balance == 2) {
     bool ok = false;
@@ -1702,7 +1746,7 @@ hms_status hms_context_set_batch_mode(hms_context* c, int32_t mode) {
 static bool lockstep_applies(int32_t count, hms_problem* const* problems) {
   for (int i = 0; i < count; ++i) {
     const hms_problem* pr = problems[i];
-    if (!pr || pr->profile || pr->lv.q != NMODES || pr->cls) return false;
+    if (!pr || pr->profile || pr->lv.q != NMODES || pr->classes) return false;
     if (!pr->tree && (pr->coarse_fp64 || pr->cluster_factor || pr->two_sided || pr->big_stages <= 0)) return false;
     if (pr->precision != problems[0]->precision || pr->nsolve != problems[0]->nsolve) return false;
   }
@@ -2480,21 +2524,25 @@ bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options
   const size_t nband = n_c * (pr.bw + 1);
   size_t fac = 0, ybytes = 0, plan_bytes = 0, setup_bytes = 0;
   RtPlanHost rtp;
+  ClassPlanHost cph;
   if (o->class_factors) {
-    ClassPlanHost cph;
     class_plan_build(lv, fix_pattern(d), class_sets_per_cta(fp32(&pr)), &cph);
     if (relax_class_smem(cph.slot_elems, cph.nb8max, fp32(&pr)) + 1024 > (size_t)maxsm) return false;
-    fac = (size_t)cph.fac_elems;
-    plan_bytes = cph.info.size() * sizeof(ClassInfo) + cph.items.size() * sizeof(ClassItem) + cph.sets.size() * 4;
-    ybytes = cph.items.size() * (size_t)cph.hmax * cph.nb8max * class_sets_per_cta(fp32(&pr)) * esz;
-    const size_t nc = cph.rep.size();
-    for (size_t t = 0; t < nc; ++t) setup_bytes += (size_t)set_factor_stride(2 * cph.info[t].w, cph.info[t].h) * 8;
-    setup_bytes += (nc + 1) * 8 + nc * 4;
-  } else if (rt_plan(lv, o, fp32(&pr), maxsm, &rtp)) {
+  }
+  const size_t nc = cph.rep.size();
+  const bool rtree = rt_plan(lv, o, fp32(&pr), maxsm, c->nsm, o->class_factors ? &cph : nullptr, &rtp);
+  if (rtree) {
     fac = (size_t)rtp.elems + RT_PAD;
     plan_bytes = (M + 1) * 8 + M * 4 + rtp.shapes.size() * sizeof(RtShape);
     for (const RtShapeHost& S : rtp.shapes) plan_bytes += rt_shape_bytes(S);
-    plan_bytes += (size_t)rt_setup(rtp, lv.M, c->nsm).own * 8;
+    plan_bytes += (size_t)rt_setup(rtp, o->class_factors ? (int)nc : lv.M, c->nsm).own * 8;
+    if (o->class_factors) setup_bytes = nc * 4;
+  } else if (o->class_factors) {
+    fac = (size_t)cph.fac_elems;
+    plan_bytes = cph.info.size() * sizeof(ClassInfo) + cph.items.size() * sizeof(ClassItem) + cph.sets.size() * 4;
+    ybytes = cph.items.size() * (size_t)cph.hmax * cph.nb8max * class_sets_per_cta(fp32(&pr)) * esz;
+    for (size_t t = 0; t < nc; ++t) setup_bytes += (size_t)set_factor_stride(2 * cph.info[t].w, cph.info[t].h) * 8;
+    setup_bytes += (nc + 1) * 8 + nc * 4;
   } else {
     for (int I = 0; I < lv.M; ++I) {
       const Region R = relax_region(lv, I);
@@ -2533,7 +2581,6 @@ bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options
     }
   b += n_c * 4 + 32 + (size_t)std::max(update_residual_blocks(lv), 1024) * 3 * 8 + 4 + sizeof(IterCtl) + 4 + 32;
   if (o->record_history) b += 3 * ((size_t)o->max_iter + 1) * 8;
-  const bool rtree = !rtp.sid.empty() && rtp.elems > 0 && ybytes == 0 && !o->class_factors;
   if (!o->class_factors && !rtree && o->relax_overlap == 0 && o->relax_balance != 1 && lv.M > c->nsm)
     b += ((size_t)lv.M + 2 * c->nsm) * sizeof(RelaxSeg) + ((size_t)c->nsm + 1) * 4 + (size_t)lv.M * 4;  // schedule
   *inst = b;

@@ -309,7 +309,7 @@ size_t rt_smem_bytes(const RtShapeHost& P, bool fp32, int copies);
 size_t rt_factor_smem_bytes(int smax);
 cudaError_t launch_rtree_factor(cudaStream_t s, const LatView& lv, const RtView& rt, double* f64, float* f32,
                                 double* scratch, int first, double* work, long long stride, int grid, int smax, int* err,
-                                bool cut);
+                                bool cut, const int* sets = nullptr, int n = 0);
 cudaError_t launch_rtree(cudaStream_t s, const LatView& lv, const RtView& rt, const double* f64, const float* f32,
                          const double2* r, void* delta, double* P, const IterCtl* ctl, int* err, int threads,
                          int copies, size_t smem, int wait0);

@@ -2,6 +2,10 @@
 // controlled relaxation of Eqs. 11-13 and the forces P = V^T r of Eq. 7 for
 // lattices too large to hold one factor per set.
 //
+// Runs where its batches fill the chip (FP32 lattices of more than 26 sets per SM),
+// for set tiles of up to 64 nodes, and with relax_balance = 1; else the sets of a
+// class share a factor of relax_tree.cu.
+//
 // With a uniform bar stiffness, k^Inner of a set depends only on its width and
 // height, the parity of its first row (the row offset of the triangle
 // lattice), which lattice edges it touches (bars to nodes outside the lattice

@@ -443,7 +443,7 @@ __device__ inline double inner_entry(const LatView& lv, const Region& R, int a, 
   return -k * (ca ? SQ3_2 : ex) * (cb ? SQ3_2 : ex);
 }
 
-// One CTA per set (grid-stride), FP64: the tree's fronts one after another,
+// One CTA per set (grid-stride over all sets, or over the n sets of a list), FP64: the tree's fronts one after another,
 // children first.  Per front: A_SS gathered into shared memory, A_BS and A_BB into
 // a work space of the CTA's (original entries plus the children's updates), A_SS swept pivot by
 // pivot to -D, G = A_BS D, the update A_BB - G A_BS^T for the parent; D, G and G^T
@@ -454,13 +454,14 @@ template <bool CUT>
 __global__ void __launch_bounds__(FTH) k_rtree_factor(LatView lv, RtView rt, double* __restrict__ f64,
                                                       float* __restrict__ f32, double* __restrict__ scratch,
                                                       int first, double* __restrict__ work, long long stride,
-                                                      int* err) {
+                                                      int* err, const int* __restrict__ sets, int n) {
   extern __shared__ double S[];  // packed lower triangle of A_SS, then the pivot column
   __shared__ int bad;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   double* X = (int)blockIdx.x < first ? scratch + (size_t)blockIdx.x * stride
                                       : work + (size_t)((int)blockIdx.x - first) * stride;
-  for (int I = blockIdx.x; I < lv.M; I += gridDim.x) {
+  for (int k0 = blockIdx.x; k0 < n; k0 += gridDim.x) {
+    const int I = sets ? sets[k0] : k0;
     const RtShape& sh = rt.shapes[rt.sid[I]];
     const Region R = relax_region(lv, I);
     const long long base = rt.off[I];
@@ -934,10 +935,11 @@ size_t rt_factor_smem_bytes(int smax) { return ((size_t)smax * (smax + 1) / 2 + 
 
 cudaError_t launch_rtree_factor(cudaStream_t s, const LatView& lv, const RtView& rt, double* f64, float* f32,
                                 double* scratch, int first, double* work, long long stride, int grid, int smax,
-                                int* err, bool cut) {
+                                int* err, bool cut, const int* sets, int n) {
   const size_t smem = rt_factor_smem_bytes(smax);
-  if (cut) k_rtree_factor<true><<<grid, FTH, smem, s>>>(lv, rt, f64, f32, scratch, first, work, stride, err);
-  else k_rtree_factor<false><<<grid, FTH, smem, s>>>(lv, rt, f64, f32, scratch, first, work, stride, err);
+  if (!sets) n = lv.M;
+  if (cut) k_rtree_factor<true><<<grid, FTH, smem, s>>>(lv, rt, f64, f32, scratch, first, work, stride, err, sets, n);
+  else k_rtree_factor<false><<<grid, FTH, smem, s>>>(lv, rt, f64, f32, scratch, first, work, stride, err, sets, n);
   return cudaGetLastError();
 }
 

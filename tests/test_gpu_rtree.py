@@ -70,3 +70,26 @@ def test_force_relax_step(hms_ctx, nx, ny, sx, sy):
     finally:
         capi.hms_problem_destroy(pr)
     assert rel(d, hms.ForceFactors(tr, g).relax(r)) < 1e-8  # as in test_gpu_force
+
+
+@pytest.mark.parametrize("nx,ny,sx,sy", [(64, 64, 16, 16), (71, 45, 16, 12), (140, 20, 64, 7)])
+@pytest.mark.parametrize("prec", [0, 1], ids=["fp64", "mixed"])
+def test_class_relax_forms(hms_ctx, nx, ny, sx, sy, prec):
+    """Class factors: sets sharing a dissected factor equal sets with their own
+    bit for bit (the same k^Inner); the batched form (relax_balance = 1) to
+    rounding."""
+    from paper_1208_4093_gb300 import capi
+    tr = truss.Truss(nx, ny)
+    g = hms.SetGrid(nx, ny, sx, sy)
+    r = tr.free * np.random.default_rng(9).standard_normal(tr.ndof)
+    outs = []
+    for kw in (dict(), dict(class_factors=1), dict(class_factors=1, relax_balance=1)):
+        pr = capi.hms_problem_create(hms_ctx, nx, ny, sx, sy, precision=prec, relax_threads=256, relax_copies=1, **kw)
+        try:
+            d, P = np.empty(tr.ndof), np.empty(9 * g.M)
+            capi.hms_relax(hms_ctx, pr, r, d, P)
+            outs.append((d, P))
+        finally:
+            capi.hms_problem_destroy(pr)
+    assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
+    assert rel(outs[2][0], hms.LocalFactors(tr, g).relax(r)) < (2e-5 if prec else 1e-11)
