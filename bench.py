@@ -156,14 +156,13 @@ def residual_work(c, fp32):
 
 
 # FP64 instructions per node of the update/residual kernel, each one slot of the
-# FP64 pipe whatever its flops: 37 for the six bar forces, r and the three norm
-# terms, plus 17 for the upper-level update u += V a of each staged node (node
-# position, xi and eta, the mode sums; int-to-double conversions not counted),
-# of which a 32 x 8 tile stages (34 x 10) / (32 x 8) = 1.33 per node.  The
-# mixed form forms the increment in FP32 and spends 4 FP64 instructions per
-# staged node on it (two conversions, two adds).
-RESIDUAL_FP64_INSTR_PER_NODE = 37 + 17 * (34 * 10) / (32 * 8)
-RESIDUAL_FP64_INSTR_PER_NODE_MIXED = 37 + 4 * (34 * 10) / (32 * 8)
+# FP64 pipe whatever its flops: 18 for the bar forces and r, 8 for the three norm
+# terms, 8 for the upper-level update u += V a (4 in the mixed form: two
+# conversions, two adds), in warps of 32 columns of which 30 are their own, and of
+# 10 rows (1024^2 nodes) plus the update of the rows below and above and the
+# forces of the bars from the row below.
+RESIDUAL_FP64_INSTR_PER_NODE = (34 + (2 * 8 + 10) / 10) * 32 / 30
+RESIDUAL_FP64_INSTR_PER_NODE_MIXED = (30 + (2 * 4 + 10) / 10) * 32 / 30
 
 
 def residual_fp64_instr(fp32):

@@ -1246,6 +1246,7 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
   lv.sy = d->set_sy;
   lv.Mx = (d->nx + d->set_sx - 1) / d->set_sx;
   lv.My = (d->ny + d->set_sy - 1) / d->set_sy;
+  lv.rr = update_residual_rr(lv);
   lv.M = lv.Mx * lv.My;
   lv.ov = o->relax_overlap;
   lv.q = force ? NMODES_RF : NMODES;

@@ -54,6 +54,7 @@ struct LatView {
   int nx, ny, sx, sy, Mx, My, M;
   int ov;          // relaxation region: the set's tile grown by ov nodes (Sec. 2.2)
   int q = 9;       // incremental modes per set: 9, or 12 with the force-controlled modes
+  int rr = 1;      // rows of a warp of the residual kernel (update_residual_rr)
   double L;        // bar length
   double k_u;      // EA/L when kbar == nullptr
   const double* kbar;
@@ -231,6 +232,7 @@ cudaError_t launch_update_residual(cudaStream_t s, const LatView& lv, const doub
                                    unsigned* ticket, double* norms_out, IterCtl* ctl, double* hist,
                                    int hist_cap, const void* delta_rf);
 int update_residual_blocks(const LatView& lv);
+int update_residual_rr(const LatView& lv);
 cudaError_t launch_reactions(cudaStream_t s, const LatView& lv, const double2* u, double2* f);
 cudaError_t launch_load_norms(cudaStream_t s, const LatView& lv, double2* p, double* partials,
                               unsigned* ticket, IterCtl* ctl);
