@@ -12,6 +12,8 @@
 #include <unordered_map>
 #include <vector>
 
+#include <cuda.h>
+
 #include "../../include/hms.h"
 #include "hms_internal.cuh"
 
@@ -188,9 +190,11 @@ __global__ void k_mask_u(LatView lv, double2* u) {
     }
   }
 }
-__global__ void k_d2f(const double* in, float* out, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    out[i] = (float)in[i];
+__global__ void k_d2f(const double2* in, float2* out, size_t n) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const double2 v = in[i];
+    out[i] = make_float2((float)v.x, (float)v.y);
+  }
 }
 __global__ void k_f2d(const float* in, double* out, size_t n) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
@@ -2258,6 +2262,41 @@ static hms_status solve_batch_lockstep(hms_context* c, int32_t count, hms_proble
   return result;
 }
 
+namespace {
+// 1 if ptr is device or managed memory of `device`, with the given alignment
+bool device_ptr_ok(const void* ptr, int device, size_t align) {
+  if (!ptr || ((uintptr_t)ptr % align) != 0) return false;
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, ptr) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (at.type == cudaMemoryTypeManaged) return true;
+  return at.type == cudaMemoryTypeDevice && at.device == device;
+}
+}  // namespace
+
+// A caller's buffer that a kernel may read or write in place: 16-byte aligned
+// memory of the device, inside one allocation (what lies outside is left to the
+// copies, which report it).
+static bool in_place(const void* ptr, size_t bytes, int device) {
+  if (!device_ptr_ok(ptr, device, 16)) return false;
+  using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const Range range = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult st;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &st) != cudaSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return (Range)f;
+  }();
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  if (!range || range(&base, &size, (CUdeviceptr)ptr) != CUDA_SUCCESS) return false;
+  return (CUdeviceptr)ptr - base + bytes <= size;
+}
+
 hms_status hms_residual(hms_problem* pr, const double* p, const double* u, double* r, double* norms,
                         int32_t mem_kind) {
   return hms_update_residual(pr, p, u, nullptr, nullptr, (double*)nullptr, r, norms, mem_kind);
@@ -2290,8 +2329,12 @@ static cudaError_t stage_deltas(hms_problem* pr, const double* delta, int32_t me
     const double* src = delta + 2 * nn * k;
     cudaError_t e;
     if (fp32(pr)) {
-      if ((e = cudaMemcpyAsync(pr->r, src, vb, kind_in(mem_kind), s)) != cudaSuccess) return e;  // staging
-      if ((e = launch_d2f(s, (const double*)pr->r, (float*)dst, 2 * nn)) != cudaSuccess) return e;
+      const double* from = src;
+      if (mem_kind != HMS_MEM_DEVICE || !in_place(src, vb, pr->ctx->device)) {
+        if ((e = cudaMemcpyAsync(pr->r, src, vb, kind_in(mem_kind), s)) != cudaSuccess) return e;  // staging
+        from = (const double*)pr->r;
+      }
+      if ((e = launch_d2f(s, from, (float*)dst, 2 * nn)) != cudaSuccess) return e;
     } else {
       if ((e = cudaMemcpyAsync(dst, src, vb, kind_in(mem_kind), s)) != cudaSuccess) return e;
     }
@@ -2320,18 +2363,54 @@ hms_status hms_update_residual(hms_problem* pr, const double* p, const double* u
   CKC(c, cudaSetDevice(c->device));
   cudaStream_t s = c->stream;
   const size_t nn = nnodes(pr), vb = nn * sizeof(double2);
-  CKC(c, cudaMemcpyAsync(pr->p, p, vb, kind_in(mem_kind), s));
-  CKC(c, cudaMemcpyAsync(pr->u[0], u, vb, kind_in(mem_kind), s));
-  CKC(c, launch_mask_u(s, pr->lv, pr->u[0]));
-  if (delta) {
-    CKC(c, stage_deltas(pr, delta, mem_kind));
-    CKC(c, cudaMemcpyAsync(pr->a, a, pr->n_c * sizeof(double), kind_in(mem_kind), s));
+  // Device buffers are used in place where no output may overlap another buffer
+  // (a CTA writes while others still read); else through the problem's own: 4096^2
+  // nodes, mixed, 1722 -> 1261 us, hms_residual on 64^2 nodes 60 -> 42 us.
+  const double2 *pp = pr->p, *up = pr->u[0];
+  double2 *rp = pr->r, *uo = pr->u[1];
+  double* np = pr->norms;
+  const void *dp = pr->delta, *dfp = pr->delta_rf;
+  const double* ap = pr->a;
+  if (mem_kind == HMS_MEM_DEVICE) {
+    const size_t db = delta ? (pr->lv.q == NMODES_RF ? 2 : 1) * vb : 0, ab = delta ? pr->n_c * sizeof(double) : 0;
+    struct Buf {
+      const void* p;
+      size_t n;
+      bool ok;
+    } in[4] = {{p, vb, false}, {u, vb, false}, {delta, db, false}, {a, ab, false}},
+      out[3] = {{r, vb, false}, {u_out, vb, false}, {norms, 3 * sizeof(double), false}};
+    auto apart = [](const Buf& x, const Buf& y) {
+      return !x.p || !y.p || (const char*)x.p + x.n <= (const char*)y.p || (const char*)y.p + y.n <= (const char*)x.p;
+    };
+    bool all = true;  // the outputs lie apart from everything else
+    for (int k = 0; k < 3; ++k) {
+      for (const Buf& x : in) all = all && apart(x, out[k]);
+      for (int l = 0; l < k; ++l) all = all && apart(out[l], out[k]);
+    }
+    if (all) {
+      for (Buf& x : in) x.ok = x.p && in_place(x.p, x.n, c->device);
+      for (Buf& x : out) x.ok = x.p && in_place(x.p, x.n, c->device);
+    }
+    if (in[0].ok) pp = (const double2*)p;
+    if (in[1].ok) up = (const double2*)u;
+    if (in[2].ok && !fp32(pr)) dp = delta, dfp = delta + 2 * nn;
+    if (in[3].ok) ap = a;
+    if (out[0].ok) rp = (double2*)r;
+    if (out[1].ok) uo = (double2*)u_out;
+    if (out[2].ok) np = norms;
   }
-  CKC(c, launch_update_residual(s, pr->lv, pr->u[0], pr->u[1], pr->p, pr->delta, fp32(pr), delta ? pr->a : nullptr,
-                                pr->r, pr->partials, pr->ticket, pr->norms, nullptr, nullptr, 0, pr->delta_rf));
-  CKC(c, cudaMemcpyAsync(r, pr->r, vb, kind_out(mem_kind), s));
-  if (u_out) CKC(c, cudaMemcpyAsync(u_out, pr->u[1], vb, kind_out(mem_kind), s));
-  if (norms) CKC(c, cudaMemcpyAsync(norms, pr->norms, 3 * sizeof(double), kind_out(mem_kind), s));
+  if (!u_out) uo = nullptr;
+  if (pp == pr->p) CKC(c, cudaMemcpyAsync(pr->p, p, vb, kind_in(mem_kind), s));
+  if (up == pr->u[0]) CKC(c, cudaMemcpyAsync(pr->u[0], u, vb, kind_in(mem_kind), s));
+  if (delta) {
+    if (dp == pr->delta) CKC(c, stage_deltas(pr, delta, mem_kind));
+    if (ap == pr->a) CKC(c, cudaMemcpyAsync(pr->a, a, pr->n_c * sizeof(double), kind_in(mem_kind), s));
+  }
+  CKC(c, launch_update_residual(s, pr->lv, up, uo, pp, dp, fp32(pr), delta ? ap : nullptr, rp, pr->partials,
+                                pr->ticket, np, nullptr, nullptr, 0, dfp));
+  if (rp == pr->r) CKC(c, cudaMemcpyAsync(r, pr->r, vb, kind_out(mem_kind), s));
+  if (uo == pr->u[1]) CKC(c, cudaMemcpyAsync(u_out, pr->u[1], vb, kind_out(mem_kind), s));
+  if (norms && np == pr->norms) CKC(c, cudaMemcpyAsync(norms, pr->norms, 3 * sizeof(double), kind_out(mem_kind), s));
   CKC(c, cudaStreamSynchronize(s));
   return HMS_OK;
 }
@@ -2427,20 +2506,6 @@ hms_status hms_coarse_solve(hms_problem* pr, const double* Kaa, const double* P,
   CKC(c, cudaStreamSynchronize(s));
   return HMS_OK;
 }
-
-namespace {
-// 1 if ptr is device or managed memory of `device`, with the given alignment
-bool device_ptr_ok(const void* ptr, int device, size_t align) {
-  if (!ptr || ((uintptr_t)ptr % align) != 0) return false;
-  cudaPointerAttributes at{};
-  if (cudaPointerGetAttributes(&at, ptr) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  if (at.type == cudaMemoryTypeManaged) return true;
-  return at.type == cudaMemoryTypeDevice && at.device == device;
-}
-}  // namespace
 
 hms_status hms_residual_noalloc(hms_problem* pr, const double* p, const double* u, double* r, double* norms) {
   if (!pr) return HMS_ERR_ARG;
@@ -2879,7 +2944,7 @@ hms_status hms_server_take(hms_server* s, int64_t id, double* u_out, int32_t* it
 
 namespace hms {
 cudaError_t launch_d2f(cudaStream_t s, const double* in, float* out, size_t n) {
-  k_d2f<<<grid1d(n), 256, 0, s>>>(in, out, n);
+  k_d2f<<<grid1d(n / 2), 256, 0, s>>>((const double2*)in, (float2*)out, n / 2);  // n even, 16-byte aligned
   return cudaGetLastError();
 }
 cudaError_t launch_f2d(cudaStream_t s, const float* in, double* out, size_t n) {

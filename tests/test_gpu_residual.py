@@ -79,3 +79,42 @@ def test_update_residual(hms_ctx, case, prec):
     assert np.array_equal(r0, ro) and np.array_equal(n0, nrm)
     ref = [np.abs(ro).sum(), ro @ ro, uo @ (p + ro)]
     assert np.allclose(nrm[:2], ref[:2], rtol=1e-12) and abs(nrm[2] - ref[2]) < 1e-12 * np.abs(uo) @ np.abs(p + ro)
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["fp64", "mixed"])
+@pytest.mark.parametrize("mask", [0x1FF, 0xFFF])
+def test_update_residual_device_buffers(hms_ctx, prec, mask):
+    """Device buffers used in place, buffers that start off a 16-byte boundary
+    and outputs that overlap inputs (both through the problem's own buffers)
+    give the bits of the host call."""
+    torch = pytest.importorskip("torch")
+    from paper_1208_4093_gb300 import capi
+    nx, ny, sx, sy = 50, 42, 24, 20
+    tr = truss.Truss(nx, ny)
+    g = hms.SetGrid(nx, ny, sx, sy)
+    q = 12 if mask == 0xFFF else 9
+    rng = np.random.default_rng(1)
+    # u not zero on constrained DOFs: it is read as zero there
+    p, u = rng.standard_normal(tr.ndof), rng.standard_normal(tr.ndof)
+    d, a = rng.standard_normal(tr.ndof * (2 if q == 12 else 1)), rng.standard_normal(q * g.M)
+    pr = capi.hms_problem_create(hms_ctx, nx, ny, sx, sy, precision=prec, mode_mask=mask)
+    try:
+        host = [np.empty(tr.ndof), np.empty(tr.ndof), np.empty(3)]
+        capi.hms_update_residual(hms_ctx, pr, p, u, d, a, *host)
+        for off in (0, 1):
+            def dev(x):
+                t = torch.empty(x.size + off, dtype=torch.float64, device="cuda")[off:]
+                t.copy_(torch.from_numpy(x))
+                return t
+            P, U, D, A = dev(p), dev(u), dev(d), dev(a)
+            outs = [dev(np.zeros(tr.ndof)), dev(np.zeros(tr.ndof)), dev(np.zeros(3))]
+            torch.cuda.synchronize()
+            capi.hms_update_residual(hms_ctx, pr, P, U, D, A, *outs)
+            for h, o in zip(host, outs):
+                assert np.array_equal(h, o.cpu().numpy())
+            assert np.array_equal(U.cpu().numpy(), u) and np.array_equal(P.cpu().numpy(), p)
+            capi.hms_update_residual(hms_ctx, pr, P, U, D, A, U, P, outs[2])  # u and p overwritten
+            assert np.array_equal(host[0], U.cpu().numpy()) and np.array_equal(host[1], P.cpu().numpy())
+            assert np.array_equal(host[2], outs[2].cpu().numpy())
+    finally:
+        capi.hms_problem_destroy(pr)
