@@ -18,7 +18,10 @@
 // constrained DOF use the general 9-term form.  All sums run in a fixed order
 // (per-thread node order, then a fixed-shape tree), so the result is the same
 // on every run.
+#include <type_traits>
+
 #include "hms_internal.cuh"
+#include "ptx.cuh"
 
 namespace hms {
 namespace {
@@ -385,6 +388,7 @@ __device__ __forceinline__ void slots_body(const LatView lv, const DT* __restric
 template <typename DT, bool FULL, typename AT>
 __global__ void __launch_bounds__(NT) k_coarse_slots(LatView lv, const DT* __restrict__ delta,
                                                      double* __restrict__ slots, const IterCtl* ctl) {
+  dep_wait();
   slots_body<DT, FULL, AT>(lv, delta, slots, ctl, blockIdx.x);
 }
 
@@ -571,6 +575,7 @@ template <typename DT, bool FULL, typename AT>
 __global__ void __launch_bounds__(NT) k_coarse_slots12(LatView lv, const DT* __restrict__ delta,
                                                        const DT* __restrict__ delta_rf, double* __restrict__ slots,
                                                        const IterCtl* ctl) {
+  dep_wait();
   slots12_body<DT, FULL, AT>(lv, delta, delta_rf, slots, ctl, blockIdx.x);
 }
 
@@ -836,26 +841,23 @@ size_t coarse_slots_smem(const LatView& lv) {
 cudaError_t launch_coarse_slots(cudaStream_t s, const LatView& lv, const void* delta, bool delta_fp32,
                                 bool full, double* slots, const IterCtl* ctl, const void* delta_rf) {
   const size_t smem = coarse_slots_smem(lv);
+  auto go12 = [&](auto k, auto* d) {
+    using DT = std::remove_pointer_t<decltype(d)>;
+    return launch_dep(k, s, lv.M, NT, smem, 0, lv, (const DT*)delta, (const DT*)delta_rf, slots, ctl);
+  };
+  auto go = [&](auto k, auto* d) {
+    using DT = std::remove_pointer_t<decltype(d)>;
+    return launch_dep(k, s, lv.M, NT, smem, 0, lv, (const DT*)delta, slots, ctl);
+  };
+  float2* const f2 = nullptr;
+  double2* const d2 = nullptr;
   if (lv.q == NMODES_RF) {
-    if (delta_fp32) {
-      const float2 *d = (const float2*)delta, *f = (const float2*)delta_rf;
-      if (full) k_coarse_slots12<float2, true, double><<<lv.M, NT, smem, s>>>(lv, d, f, slots, ctl);
-      else k_coarse_slots12<float2, false, float><<<lv.M, NT, smem, s>>>(lv, d, f, slots, ctl);
-    } else {
-      const double2 *d = (const double2*)delta, *f = (const double2*)delta_rf;
-      if (full) k_coarse_slots12<double2, true, double><<<lv.M, NT, smem, s>>>(lv, d, f, slots, ctl);
-      else k_coarse_slots12<double2, false, double><<<lv.M, NT, smem, s>>>(lv, d, f, slots, ctl);
-    }
-    return cudaGetLastError();
+    if (delta_fp32)
+      return full ? go12(k_coarse_slots12<float2, true, double>, f2) : go12(k_coarse_slots12<float2, false, float>, f2);
+    return full ? go12(k_coarse_slots12<double2, true, double>, d2) : go12(k_coarse_slots12<double2, false, double>, d2);
   }
-  if (delta_fp32) {
-    if (full) k_coarse_slots<float2, true, double><<<lv.M, NT, smem, s>>>(lv, (const float2*)delta, slots, ctl);
-    else k_coarse_slots<float2, false, float><<<lv.M, NT, smem, s>>>(lv, (const float2*)delta, slots, ctl);
-  } else {
-    if (full) k_coarse_slots<double2, true, double><<<lv.M, NT, smem, s>>>(lv, (const double2*)delta, slots, ctl);
-    else k_coarse_slots<double2, false, double><<<lv.M, NT, smem, s>>>(lv, (const double2*)delta, slots, ctl);
-  }
-  return cudaGetLastError();
+  if (delta_fp32) return full ? go(k_coarse_slots<float2, true, double>, f2) : go(k_coarse_slots<float2, false, float>, f2);
+  return full ? go(k_coarse_slots<double2, true, double>, d2) : go(k_coarse_slots<double2, false, double>, d2);
 }
 
 cudaError_t configure_coarse_assemble(int max_smem) {

@@ -42,6 +42,7 @@
 
 #include "coarse_blocks.cuh"
 #include "hms_internal.cuh"
+#include "ptx.cuh"
 
 namespace hms {
 namespace {
@@ -74,6 +75,8 @@ __global__ void __launch_bounds__(128) k_tree_diag(const TreeProb* __restrict__ 
                                                    const TreeItem* __restrict__ items, int use_ctl) {
   const TreeItem it = item_of(items, blockIdx.x);
   const TreeProb& pb = probs[it.prob];
+  dep_wait();
+  dep_launch();
   if (use_ctl && tree_done(pb.ctl)) return;
   constexpr unsigned FULL = 0xffffffffu;
   const int I = it.node, lane = threadIdx.x & 31;
@@ -144,6 +147,8 @@ __global__ void __launch_bounds__(256) k_tree_rows(const TreeProb* __restrict__ 
                                                    const TreeItem* __restrict__ items, int use_ctl) {
   const TreeItem it = item_of(items, blockIdx.x);
   const TreeProb& pb = probs[it.prob];
+  dep_wait();
+  dep_launch();
   if (use_ctl && tree_done(pb.ctl)) return;
   const int nm = pb.nm, bs = nm * nm, R = 9 * nm, Mx = pb.Mx, My = pb.My, I = it.node;
   const double *blk = pb.blk, *scale = pb.scale;
@@ -316,7 +321,6 @@ __global__ void __launch_bounds__(FT, 1) k_tree_factor(const TreeProb* __restric
   const int cl = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const TreeItem it = items[blockIdx.x / cl];
   const TreeProb pb = probs[it.prob];
-  if (use_ctl && tree_done(pb.ctl)) return;  // the same in every CTA of the cluster
   const TreeNode nd = pb.nodes[it.node];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nm = pb.nm;
@@ -368,6 +372,10 @@ __global__ void __launch_bounds__(FT, 1) k_tree_factor(const TreeProb* __restric
     for (int J = lane; J <= I; J += 32) list[row_tile(q) + J] = (I << 16) | J;
   }
   if (tid == 0) qhead = 0;
+  // the tables hold nothing but the plan: built while the kernel before runs
+  dep_wait();
+  dep_launch();
+  if (use_ctl && tree_done(pb.ctl)) return;  // the same in every CTA of the cluster
   __syncthreads();
 
   // ---- assemble: original entries of the S columns and the children's updates,
@@ -687,7 +695,6 @@ __global__ void __launch_bounds__(ST, 1) k_tree_solve(const TreeProb* __restrict
   cg::cluster_group cluster = cg::this_cluster();
   const int cl = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const TreeProb pb = probs[which[blockIdx.x / cl]];
-  if (use_ctl && tree_done(pb.ctl)) return;
   const int tid = threadIdx.x;
   const int n = pb.n, Mx = pb.Mx, My = pb.My;
   constexpr int Rw = 9 * Q;
@@ -701,6 +708,9 @@ __global__ void __launch_bounds__(ST, 1) k_tree_solve(const TreeProb* __restrict
   const float4* M4 = reinterpret_cast<const float4*>(pb.M);
   // this CTA's share of the unknowns
   const int ub = (int)((long long)n * rank / cl), ue = (int)((long long)n * (rank + 1) / cl);
+  for (int ph = tid; ph < nphase; ph += ST) span[ph] = phase[ph * cl + rank];
+  dep_wait();
+  if (use_ctl && tree_done(pb.ctl)) return;
   double bm = 0.0;
   for (int i = ub + tid; i < ue; i += ST) {
     const double v = pb.dropped[i] ? 0.0 : pb.b[i];
@@ -712,7 +722,6 @@ __global__ void __launch_bounds__(ST, 1) k_tree_solve(const TreeProb* __restrict
   // n: the ones being fetched)
   int4 ge, gf, re, ro, gen, gfn, ren, ron;
   float4 mh[PM];
-  for (int ph = tid; ph < nphase; ph += ST) span[ph] = phase[ph * cl + rank];
   __syncthreads();
   auto load_row = [&](int r, int end) {
     ren = make_int4(0, 0, 0, 0), ron = make_int4(0, 0, 0, 0);
@@ -1121,42 +1130,17 @@ cudaError_t launch_tree_system(cudaStream_t s, int q, bool slots, const TreeProb
                                bool use_ctl) {
   if (n <= 0) return cudaSuccess;
   const int c = (int)use_ctl;
-  if (q == NMODES_RF) {
-    if (slots) k_tree_diag<NMODES_RF, true><<<n, 128, 0, s>>>(probs, sets, c);
-    else k_tree_diag<NMODES_RF, false><<<n, 128, 0, s>>>(probs, sets, c);
-  } else {
-    if (slots) k_tree_diag<NMODES, true><<<n, 128, 0, s>>>(probs, sets, c);
-    else k_tree_diag<NMODES, false><<<n, 128, 0, s>>>(probs, sets, c);
-  }
-  cudaError_t e = cudaGetLastError();
+  const auto diag = q == NMODES_RF ? (slots ? k_tree_diag<NMODES_RF, true> : k_tree_diag<NMODES_RF, false>)
+                                   : (slots ? k_tree_diag<NMODES, true> : k_tree_diag<NMODES, false>);
+  const cudaError_t e = launch_dep(diag, s, n, 128, 0, 0, probs, sets, c);
   if (e != cudaSuccess) return e;
-  k_tree_rows<<<n, 256, 0, s>>>(probs, sets, c);
-  return cudaGetLastError();
+  return launch_dep(k_tree_rows, s, n, 256, 0, 0, probs, sets, c);
 }
-
-namespace {
-template <typename... KA, typename... A>
-cudaError_t launch_cluster(void (*k)(KA...), cudaStream_t s, int grid, int threads, int cl, size_t smem, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)cl;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, args...);
-}
-}  // namespace
 
 cudaError_t launch_tree_level(cudaStream_t s, const TreeLaunch& L, const TreeProb* probs, const TreeItem* nodes, int n,
                               bool use_ctl) {
   if (n <= 0) return cudaSuccess;
-  return launch_cluster(k_tree_factor, s, n * L.cl, FT, L.cl, L.smem, probs, nodes, L.nbuf, (int)use_ctl);
+  return launch_dep(k_tree_factor, s, n * L.cl, FT, L.smem, L.cl, probs, nodes, L.nbuf, (int)use_ctl);
 }
 
 cudaError_t launch_tree_factor(cudaStream_t s, const TreePlanHost& P, const TreeProb* prob, const TreeItem* items,
@@ -1173,8 +1157,8 @@ cudaError_t launch_tree_factor(cudaStream_t s, const TreePlanHost& P, const Tree
 cudaError_t launch_tree_solve(cudaStream_t s, int q, int scl, size_t smem, const TreeProb* probs, const int* which,
                               int n, bool use_ctl) {
   if (n <= 0) return cudaSuccess;
-  if (q == NMODES_RF) return launch_cluster(k_tree_solve<NMODES_RF>, s, n * scl, ST, scl, smem, probs, which, (int)use_ctl);
-  return launch_cluster(k_tree_solve<NMODES>, s, n * scl, ST, scl, smem, probs, which, (int)use_ctl);
+  return launch_dep(q == NMODES_RF ? k_tree_solve<NMODES_RF> : k_tree_solve<NMODES>, s, n * scl, ST, smem, scl, probs, which,
+                    (int)use_ctl);
 }
 
 cudaError_t configure_coarse_tree(int max_smem) {

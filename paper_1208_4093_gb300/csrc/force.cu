@@ -31,6 +31,7 @@
 #include <vector>
 
 #include "hms_internal.cuh"
+#include "ptx.cuh"
 
 namespace hms {
 namespace {
@@ -80,6 +81,7 @@ __device__ inline void st2<float2>(float2* p, size_t n, double2 v) { p[n] = make
 __global__ void __launch_bounds__(NT) k_force_in(LatView lv, const double2* __restrict__ r,
                                                  const double* __restrict__ M, const uint8_t* __restrict__ fixF,
                                                  double2* __restrict__ rp, const IterCtl* ctl) {
+  dep_wait();
   if (ctl && *(volatile const int*)&ctl->done) return;
   __shared__ double red[(NT / 32) * 3], tot[3];
   const int I = blockIdx.x;
@@ -120,6 +122,7 @@ template <typename T2>
 __global__ void __launch_bounds__(NT) k_force_out(LatView lv, T2* __restrict__ d, const double* __restrict__ M,
                                                   const double2* __restrict__ r, double* __restrict__ P,
                                                   const IterCtl* ctl) {
+  dep_wait();
   if (ctl && *(volatile const int*)&ctl->done) return;
   __shared__ double red[(NT / 32) * 3], tot[3];
   const int I = blockIdx.x;
@@ -168,15 +171,13 @@ __global__ void __launch_bounds__(NT) k_force_out(LatView lv, T2* __restrict__ d
 
 cudaError_t launch_force_in(cudaStream_t s, const LatView& lv, const double2* r, const double* M,
                             const uint8_t* fixF, double2* rproj, const IterCtl* ctl) {
-  k_force_in<<<lv.M, NT, 0, s>>>(lv, r, M, fixF, rproj, ctl);
-  return cudaGetLastError();
+  return launch_dep(k_force_in, s, lv.M, NT, 0, 0, lv, r, M, fixF, rproj, ctl);
 }
 
 cudaError_t launch_force_out(cudaStream_t s, const LatView& lv, void* drf, bool fp32, const double* M,
                              const double2* r, double* P, const IterCtl* ctl) {
-  if (fp32) k_force_out<float2><<<lv.M, NT, 0, s>>>(lv, (float2*)drf, M, r, P, ctl);
-  else k_force_out<double2><<<lv.M, NT, 0, s>>>(lv, (double2*)drf, M, r, P, ctl);
-  return cudaGetLastError();
+  if (fp32) return launch_dep(k_force_out<float2>, s, lv.M, NT, 0, 0, lv, (float2*)drf, M, r, P, ctl);
+  return launch_dep(k_force_out<double2>, s, lv.M, NT, 0, 0, lv, (double2*)drf, M, r, P, ctl);
 }
 
 }  // namespace hms

@@ -5,6 +5,16 @@
 
 namespace hms {
 
+// Programmatic dependent launch: dep_wait holds a CTA until the kernels before in
+// the stream are complete and their writes visible (every thread of every CTA
+// calls it before its first access to anything they write, and before any
+// return, so that completion carries on from kernel to kernel); dep_launch lets
+// the next kernel's CTAs be placed once all CTAs of this one have called it.
+// Without effect in a kernel launched the ordinary way.
+__device__ inline void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ inline void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+
 __device__ inline uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }

@@ -122,7 +122,6 @@ __device__ __forceinline__ void rtree_body(const LatView& lv, const RtView& rt, 
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ uint64_t bar;
   __shared__ int posv[NV], vrow[NV + 1];
-  if (ctl && *(volatile const int*)&ctl->done) return;
   using T2 = typename Vec2<T>::type;
   constexpr int NW = NT / 32, PER = NV / NW;  // streams per warp
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -174,6 +173,13 @@ __device__ __forceinline__ void rtree_body(const LatView& lv, const RtView& rt, 
       const int v = warp + q * NW;
       fetch(ring0 + (v * NS + c) * CB, fac0 + (size_t)vrow[v] * (32 * sizeof(T)) + (size_t)c * CB);
     }
+  // the lists and the factor are the plan's: fetched while the kernel before runs
+  dep_wait();
+  if (ctl && *(volatile const int*)&ctl->done) {  // the copies in flight land before the CTA exits
+    cp_async_wait<0>();
+    mbar_wait_bounded(&bar, 0u);
+    return;
+  }
   // z = r in the tree's order (four nodes in flight per thread)
   {
     const double2* rg = r + (size_t)RG.j0 * lv.nx + RG.i0;
@@ -967,8 +973,8 @@ cudaError_t launch_rtree(cudaStream_t s, const LatView& lv, const RtView& rt, co
     const T* fac;
     if constexpr (sizeof(T) == 4) fac = f32;
     else fac = f64;
-    k_rtree<T, decltype(nt)::value, decltype(ns)::value><<<lv.M, decltype(nt)::value, smem, s>>>(
-        lv, rt, fac, r, (T*)delta, P, ctl, err, wait0);
+    (void)launch_dep(k_rtree<T, decltype(nt)::value, decltype(ns)::value>, s, lv.M, decltype(nt)::value, smem, 0, lv, rt,
+                     fac, r, (T*)delta, P, ctl, err, wait0);  // rt_dispatch returns its error
   });
 }
 

@@ -34,6 +34,7 @@
 #include <type_traits>
 
 #include "hms_internal.cuh"
+#include "ptx.cuh"
 
 namespace hms {
 namespace {
@@ -370,6 +371,7 @@ __global__ void __launch_bounds__(RNT) k_update_residual(
     const double2* __restrict__ p, const DT* __restrict__ delta, const DT* __restrict__ delta_rf,
     const double* __restrict__ a, double2* __restrict__ r, double* __restrict__ partials, unsigned* ticket,
     double* norms_out, IterCtl* ctl, double* hist, int hist_cap) {
+  dep_wait();
   update_residual_body<DT, RF>(lv, u_in, u_out, p, delta, delta_rf, a, r, partials, ticket, norms_out, ctl, hist,
                                hist_cap, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
 }
@@ -514,24 +516,16 @@ cudaError_t launch_update_residual(cudaStream_t s, const LatView& lv, const doub
                                    int hist_cap, const void* delta_rf) {
   const dim3 grid(update_residual_grid_x(lv), (lv.ny + RW * lv.rr - 1) / (RW * lv.rr));
   const bool rf = lv.q == NMODES_RF;
-  if (delta_fp32) {
-    if (rf)
-      k_update_residual<float2, true><<<grid, RNT, 0, s>>>(lv, u_in, u_out, p, (const float2*)delta,
-                                                          (const float2*)delta_rf, a, r, partials, ticket,
-                                                          norms_out, ctl, hist, hist_cap);
-    else
-      k_update_residual<float2, false><<<grid, RNT, 0, s>>>(lv, u_in, u_out, p, (const float2*)delta, nullptr, a, r,
-                                                           partials, ticket, norms_out, ctl, hist, hist_cap);
-  } else {
-    if (rf)
-      k_update_residual<double2, true><<<grid, RNT, 0, s>>>(lv, u_in, u_out, p, (const double2*)delta,
-                                                           (const double2*)delta_rf, a, r, partials, ticket,
-                                                           norms_out, ctl, hist, hist_cap);
-    else
-      k_update_residual<double2, false><<<grid, RNT, 0, s>>>(lv, u_in, u_out, p, (const double2*)delta, nullptr, a,
-                                                            r, partials, ticket, norms_out, ctl, hist, hist_cap);
-  }
-  return cudaGetLastError();
+  auto go = [&](auto k, auto* d) {
+    using DT = std::remove_pointer_t<decltype(d)>;
+    return launch_dep(k, s, grid, RNT, 0, 0, lv, u_in, u_out, p, (const DT*)delta, rf ? (const DT*)delta_rf : nullptr, a,
+                      r, partials, ticket, norms_out, ctl, hist, hist_cap);
+  };
+  if (delta_fp32)
+    return rf ? go(k_update_residual<float2, true>, (float2*)nullptr)
+              : go(k_update_residual<float2, false>, (float2*)nullptr);
+  return rf ? go(k_update_residual<double2, true>, (double2*)nullptr)
+            : go(k_update_residual<double2, false>, (double2*)nullptr);
 }
 
 cudaError_t launch_load_norms(cudaStream_t s, const LatView& lv, double2* p, double* partials,
