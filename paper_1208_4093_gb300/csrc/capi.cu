@@ -251,15 +251,30 @@ cudaError_t launch_solve_stage(hms_problem* pr, cudaStream_t s, int q, const Ite
                              pr->x, pr->scale, pr->a, pr->cstat, flags, ctl, pr->err);
 }
 
+// The relaxation by nested dissection: the displacement-controlled one (main), the
+// cut-free sets' of the force-controlled modes, or both in one launch.
+cudaError_t launch_relax_tree(hms_problem* pr, cudaStream_t s, const IterCtl* ctl, bool main, bool cut) {
+  const bool f = fp32(pr);
+  const void* fac = f ? (const void*)pr->f32 : pr->f64;
+  const void* cfac = f ? (const void*)pr->f32F : pr->f64F;
+  const size_t smem = pr->rt_smem[pr->relax_chunks];
+  if (main && cut)
+    return launch_rtree(s, pr->lv, pr->rt, fac, f, pr->r, pr->delta, pr->P, ctl, pr->err, pr->relax_threads,
+                        pr->relax_chunks, smem, pr->relax_wait0, cfac, pr->rproj, pr->delta_rf);
+  if (cut)
+    return launch_rtree(s, pr->lv, pr->rt, cfac, f, pr->rproj, pr->delta_rf, nullptr, ctl, pr->err, pr->relax_threads,
+                        pr->relax_chunks, smem, pr->relax_wait0);
+  return launch_rtree(s, pr->lv, pr->rt, fac, f, pr->r, pr->delta, pr->P, ctl, pr->err, pr->relax_threads,
+                      pr->relax_chunks, smem, pr->relax_wait0);
+}
+
 // The displacement-controlled relaxation of every set (K2), with per-set or
 // class factors.
 cudaError_t launch_relax_main(hms_problem* pr, cudaStream_t s, const IterCtl* ctl) {
   if (pr->cls)
     return launch_relax_class(s, pr->lv, pr->cpd, pr->f64, pr->f32, pr->r, pr->delta, pr->P, pr->yscratch, ctl,
                               pr->err, pr->relax_wait0);
-  if (pr->rtree)
-    return launch_rtree(s, pr->lv, pr->rt, pr->f64, pr->f32, pr->r, pr->delta, pr->P, ctl, pr->err,
-                        pr->relax_threads, pr->relax_chunks, pr->rt_smem[pr->relax_chunks], pr->relax_wait0);
+  if (pr->rtree) return launch_relax_tree(pr, s, ctl, true, false);
   if (pr->relax_sched)
     return launch_relax_sched(s, pr->lv, pr->set_off, pr->f64, pr->f32, pr->r, pr->delta, pr->P, pr->yscratch, ctl,
                               pr->err, pr->sched_segs, pr->sched_cta, pr->sched_flags, pr->sched_grid,
@@ -289,15 +304,17 @@ cudaError_t launch_refine_residual(hms_problem* pr, cudaStream_t s, const IterCt
   return launch_coarse_residual(s, pr->n_c, pr->bw, pr->sband, pr->b, pr->x, pr->dropped, pr->res, pr->cstat, ctl);
 }
 
-// The force-controlled relaxation of every set (Eqs. 15-17, force.cu) after the
-// displacement-controlled one: r projected, the cut-free solve, delta^RF and
-// the upper-level forces of the modes 10-12 (P[12 I + 9 .. 11]).
-cudaError_t launch_force_relax(hms_problem* pr, cudaStream_t s, const IterCtl* ctl) {
+// The force-controlled relaxation of every set (Eqs. 15-17, force.cu): r projected,
+// the cut-free solve, delta^RF and the upper-level forces of the modes 10-12
+// (P[12 I + 9 .. 11]); with main the displacement-controlled relaxation before it
+// or in its launch.
+cudaError_t launch_force_relax(hms_problem* pr, cudaStream_t s, const IterCtl* ctl, bool main) {
   const LatView& lv = pr->lv;
-  cudaError_t e = launch_force_in(s, lv, pr->r, pr->Mforce, pr->fixF, pr->rproj, ctl);
+  cudaError_t e = cudaSuccess;
+  if (main && !pr->rtree) e = launch_relax_main(pr, s, ctl);
+  if (e == cudaSuccess) e = launch_force_in(s, lv, pr->r, pr->Mforce, pr->fixF, pr->rproj, ctl);
   if (e != cudaSuccess) return e;
-  e = pr->rtree ? launch_rtree(s, lv, pr->rt, pr->f64F, pr->f32F, pr->rproj, pr->delta_rf, nullptr, ctl, pr->err,
-                               pr->relax_threads, pr->relax_chunks, pr->rt_smem[pr->relax_chunks], pr->relax_wait0)
+  e = pr->rtree ? launch_relax_tree(pr, s, ctl, main, true)
                 : launch_relax(s, lv, pr->set_off, pr->f64F, pr->f32F, pr->rproj, pr->delta_rf, nullptr, pr->yscratch,
                                ctl, pr->err, pr->relax_threads, pr->relax_chunks, pr->relax_wait0);
   if (e != cudaSuccess) return e;
@@ -321,12 +338,8 @@ cudaError_t launch_iteration(hms_problem* pr, cudaStream_t s, int k, cudaEvent_t
                              pr->delta_rf);
   if (e != cudaSuccess) return e;
   mark();
-  e = launch_relax_main(pr, s, pr->ctl);
+  e = lv.q == NMODES_RF ? launch_force_relax(pr, s, pr->ctl, true) : launch_relax_main(pr, s, pr->ctl);
   if (e != cudaSuccess) return e;
-  if (lv.q == NMODES_RF) {
-    e = launch_force_relax(pr, s, pr->ctl);
-    if (e != cudaSuccess) return e;
-  }
   mark();
   e = launch_coarse_slots(s, lv, pr->delta, fp32(pr), false, pr->slots_it, pr->ctl, pr->delta_rf);
   if (e != cudaSuccess) return e;
@@ -1164,8 +1177,8 @@ static cudaError_t autotune_relax(hms_problem* pr, int copies, bool try_sched) {
       return launch_relax_sched(s, lv, pr->set_off, pr->f64, pr->f32, pr->r, pr->delta, pr->P, pr->yscratch,
                                 nullptr, pr->err, pr->sched_segs, pr->sched_cta, pr->sched_flags, pr->sched_grid);
     if (pr->rtree)
-      return launch_rtree(s, lv, pr->rt, pr->f64, pr->f32, pr->r, pr->delta, pr->P, nullptr, pr->err, nt, nc,
-                          pr->rt_smem[nc], -1);
+      return launch_rtree(s, lv, pr->rt, fp32(pr) ? (const void*)pr->f32 : pr->f64, fp32(pr), pr->r, pr->delta, pr->P,
+                          nullptr, pr->err, nt, nc, pr->rt_smem[nc], -1);
     return launch_relax(s, lv, pr->set_off, pr->f64, pr->f32, pr->r, pr->delta, pr->P, pr->yscratch, nullptr,
                         pr->err, nt, nc);
   };
@@ -2424,8 +2437,7 @@ hms_status hms_relax(hms_problem* pr, const double* r, double* delta, double* P,
   const size_t nn = nnodes(pr), vb = nn * sizeof(double2);
   CKC(c, cudaMemcpyAsync(pr->r, r, vb, kind_in(mem_kind), s));
   CKC(c, launch_mask_u(s, pr->lv, pr->r));
-  CKC(c, launch_relax_main(pr, s, nullptr));
-  if (pr->lv.q == NMODES_RF) CKC(c, launch_force_relax(pr, s, nullptr));
+  CKC(c, pr->lv.q == NMODES_RF ? launch_force_relax(pr, s, nullptr, true) : launch_relax_main(pr, s, nullptr));
   CKC(c, copy_delta_out(pr, pr->delta, delta, mem_kind));
   CKC(c, cudaMemcpyAsync(P, pr->P, pr->n_c * sizeof(double), kind_out(mem_kind), s));
   CKC(c, cudaStreamSynchronize(s));
@@ -2442,7 +2454,7 @@ hms_status hms_relax_force(hms_problem* pr, const double* r, double* delta_rf, i
   const size_t nn = nnodes(pr), vb = nn * sizeof(double2);
   CKC(c, cudaMemcpyAsync(pr->r, r, vb, kind_in(mem_kind), s));
   CKC(c, launch_mask_u(s, pr->lv, pr->r));
-  CKC(c, launch_force_relax(pr, s, nullptr));
+  CKC(c, launch_force_relax(pr, s, nullptr, false));
   CKC(c, copy_delta_out(pr, pr->delta_rf, delta_rf, mem_kind));
   CKC(c, cudaStreamSynchronize(s));
   return check_dev_err(pr);

@@ -340,9 +340,10 @@ size_t rt_factor_smem_bytes(int smax);
 cudaError_t launch_rtree_factor(cudaStream_t s, const LatView& lv, const RtView& rt, double* f64, float* f32,
                                 double* scratch, int first, double* work, long long stride, int grid, int smax, int* err,
                                 bool cut, const int* sets = nullptr, int n = 0);
-cudaError_t launch_rtree(cudaStream_t s, const LatView& lv, const RtView& rt, const double* f64, const float* f32,
+cudaError_t launch_rtree(cudaStream_t s, const LatView& lv, const RtView& rt, const void* fac, bool fp32,
                          const double2* r, void* delta, double* P, const IterCtl* ctl, int* err, int threads,
-                         int copies, size_t smem, int wait0);
+                         int copies, size_t smem, int wait0, const void* fac2 = nullptr, const double2* r2 = nullptr,
+                         void* delta2 = nullptr);
 cudaError_t configure_relax_tree(int max_smem);
 // relax_class.cu: the relaxation with class factors (sets per CTA: 64 FP32, 32 FP64)
 int class_sets_per_cta(bool fp32);
