@@ -67,45 +67,60 @@ __device__ inline TreeItem item_of(const TreeItem* items, int k) {
 // One CTA per set: its five blocks of K_aa from the slots (SLOTS; else the
 // blocks are there), then, in one warp with lane = mode, the scale s_i =
 // D_ii^-1/2, b = s P, x = 0 and the modes that take no part (mode mask,
-// vanishing diagonal, a pivot <= 1e-14 in the FP64 Cholesky of the scaled
-// diagonal block in mode order): the rules and the arithmetic of k_blk_diag,
-// whose dependent pivots in one thread per set took 40 us.
+// vanishing diagonal, a pivot <= 1e-14 in the FP64 elimination of the scaled
+// diagonal block in mode order): the rules of k_blk_diag, whose dependent pivots in
+// one thread per set took 40 us.  Bound by the chain of FP64 operations, 64 clocks
+// each for one warp of an SM: one entry per thread, the pivots' reciprocals by two
+// Newton steps from FP32, and L D L^T instead of square roots and divisions take
+// 14 us where 128 threads and the Cholesky form took 23 (16 to 256 sets; q = 12: 15
+// and 34).  Beyond two sets per SM the entries' loads and sums of one set hide the
+// others' chains, and CTAs of 128 threads all fit at once (1015 sets: 12 us less per
+// update than one entry per thread).
+template <int Q>
+constexpr int DIAG_T = (NBLK * Q * Q + 31) / 32 * 32;
 template <int Q, bool SLOTS>
-__global__ void __launch_bounds__(128) k_tree_diag(const TreeProb* __restrict__ probs,
-                                                   const TreeItem* __restrict__ items, int use_ctl) {
+__global__ void __launch_bounds__(DIAG_T<Q>) k_tree_diag(const TreeProb* __restrict__ probs,
+                                                         const TreeItem* __restrict__ items, int use_ctl) {
   const TreeItem it = item_of(items, blockIdx.x);
   const TreeProb& pb = probs[it.prob];
+  constexpr unsigned FULL = 0xffffffffu;
+  const int I = it.node, lane = threadIdx.x & 31, tid = threadIdx.x;
+  __shared__ double S[Q * Q];
+  const LatView lv = pb.lv;
+  const double *base = pb.slots_base, *now = pb.slots_it, *Pv = pb.P;
+  double *blk = pb.blk, *scale = pb.scale, *bv = pb.b, *xv = pb.x;
+  int* dropped = pb.dropped;
+  const IterCtl* ctl = pb.ctl;
+  const unsigned mask = pb.mode_mask;
   dep_wait();
   dep_launch();
-  if (use_ctl && tree_done(pb.ctl)) return;
-  constexpr unsigned FULL = 0xffffffffu;
-  const int I = it.node, lane = threadIdx.x & 31;
-  __shared__ double S[Q * Q];
-  {
-    const LatView lv = pb.lv;
-    double* B = pb.blk + (size_t)I * NBLK * Q * Q;
-    for (int e = threadIdx.x; e < (SLOTS ? NBLK : 1) * Q * Q; e += 128) {
-      double v;
-      if constexpr (SLOTS) {
-        const int b = e / (Q * Q), l = e % (Q * Q) / Q, m = e % Q;
-        v = blk_entry(lv, pb.slots_base, pb.slots_it, I, b, l, m);
-        B[e] = v;
-      } else {
-        v = B[e];
-      }
-      if (e < Q * Q) S[e] = v;
+  if (use_ctl && tree_done(ctl)) return;
+  const double rhs = tid < Q ? Pv[Q * I + tid] : 0.0;
+  double* B = blk + (size_t)I * NBLK * Q * Q;
+  for (int e = tid; e < (SLOTS ? NBLK : 1) * Q * Q; e += blockDim.x) {
+    double v;
+    if constexpr (SLOTS) {
+      v = blk_entry(lv, base, now, I, e / (Q * Q), e % (Q * Q) / Q, e % Q);
+      B[e] = v;
+    } else {
+      v = B[e];
     }
+    if (e < Q * Q) S[e] = v;
   }
   __syncthreads();
-  if (threadIdx.x >= 32) return;
+  if (tid >= 32) return;
   const int row = lane < Q ? lane : Q - 1;
   const double D = S[row * Q + row];
-  const bool in = lane < Q && ((pb.mode_mask >> row) & 1u);
-  double dmax = in ? D : 0.0;
+  const bool in = lane < Q && ((mask >> row) & 1u);
+  // the largest positive diagonal (positive doubles order as their bits do)
+  long long top = in && D > 0.0 ? __double_as_longlong(D) : 0;
 #pragma unroll
-  for (int m = 16; m > 0; m >>= 1) dmax = fmax(dmax, __shfl_xor_sync(FULL, dmax, m));
-  bool dr = !in || !(D > 1e-300) || !(D > 1e-28 * dmax);
-  const double sc = dr ? 0.0 : 1.0 / sqrt(D);
+  for (int m = 16; m > 0; m >>= 1) {
+    const long long o = __shfl_xor_sync(FULL, top, m);
+    top = o > top ? o : top;
+  }
+  bool dr = !in || !(D > 1e-300) || !(D > 1e-28 * __longlong_as_double(top));
+  const double sc = dr ? 0.0 : rsqrt(D);
   double A[Q];
 #pragma unroll
   for (int l = 0; l < Q; ++l) {
@@ -115,25 +130,27 @@ __global__ void __launch_bounds__(128) k_tree_diag(const TreeProb* __restrict__ 
   const unsigned dr0 = __ballot_sync(FULL, dr);
 #pragma unroll
   for (int m = 0; m < Q; ++m) {
-    if ((dr0 >> m) & 1u) continue;  // left out beforehand: its row and column are zero
     const double piv = __shfl_sync(FULL, A[m], m);
-    if (!(piv > 1e-14)) {
-      if (lane == m) dr = true;
-      A[m] = 0.0;
-      continue;
-    }
-    const double d = sqrt(piv);
-    A[m] = A[m] / d;
-    const double lm = A[m];
+    const bool out = (dr0 >> m) & 1u;  // left out beforehand: its row and column are zero
+    const bool low = !out && !(piv > 1e-14);
+    if (low && lane == m) dr = true;
+    // 1 / piv: FP32, then 24 -> 48 -> 53 bits (piv <= 1 but for rounding, > 1e-14)
+    double ri = (double)__frcp_rn((float)piv);
+    ri = fma(ri, fma(-piv, ri, 1.0), ri);
+    ri = fma(ri, fma(-piv, ri, 1.0), ri);
+    const double t = out || low ? 0.0 : A[m] * ri;
 #pragma unroll
-    for (int l = m + 1; l < Q; ++l) A[l] -= lm * __shfl_sync(FULL, lm, l);
+    for (int l = m + 1; l < Q; ++l) {
+      const double al = __shfl_sync(FULL, A[m], l);
+      A[l] = out || low ? A[l] : fma(-t, al, A[l]);
+    }
   }
   if (lane < Q) {
     const int i = Q * I + lane;
-    pb.scale[i] = sc;
-    pb.b[i] = dr ? 0.0 : sc * pb.P[i];
-    pb.x[i] = 0.0;
-    pb.dropped[i] = dr ? 1 : 0;
+    scale[i] = sc;
+    bv[i] = dr ? 0.0 : sc * rhs;
+    xv[i] = 0.0;
+    dropped[i] = dr ? 1 : 0;
   }
 }
 
@@ -1132,7 +1149,8 @@ cudaError_t launch_tree_system(cudaStream_t s, int q, bool slots, const TreeProb
   const int c = (int)use_ctl;
   const auto diag = q == NMODES_RF ? (slots ? k_tree_diag<NMODES_RF, true> : k_tree_diag<NMODES_RF, false>)
                                    : (slots ? k_tree_diag<NMODES, true> : k_tree_diag<NMODES, false>);
-  const cudaError_t e = launch_dep(diag, s, n, 128, 0, 0, probs, sets, c);
+  const int dt = n > 304 ? 128 : (q == NMODES_RF ? DIAG_T<NMODES_RF> : DIAG_T<NMODES>);
+  const cudaError_t e = launch_dep(diag, s, n, dt, 0, 0, probs, sets, c);
   if (e != cudaSuccess) return e;
   return launch_dep(k_tree_rows, s, n, 256, 0, 0, probs, sets, c);
 }
