@@ -973,6 +973,8 @@ static cudaError_t alloc_instance(hms_problem* pr) {
   CKI(palloc(pr, &pr->a, n_c));
   CKI(palloc(pr, &pr->P, n_c));
   CKI(palloc(pr, &pr->slots_it, (size_t)lv.M * NSLOTS * slot_size(lv.q)));
+  // the updates write only the entries that involve the increment modes
+  CKI(cudaMemsetAsync(pr->slots_it, 0, (size_t)lv.M * NSLOTS * slot_size(lv.q) * sizeof(double), s));
   if (!pr->nd && !pr->tree) {
     CKI(palloc(pr, &pr->band, nband));
     CKI(palloc(pr, &pr->sband, 2 * nband));
@@ -2093,7 +2095,7 @@ static hms_status solve_batch_lockstep(hms_context* c, int32_t count, hms_proble
   for (hms_problem* pr : probs) {
     if (pr->rtree) sm_rt = std::max(sm_rt, pr->rt_smem[rchunks]);
     else sm_relax = std::max(sm_relax, relax_smem_bytes(pr->lv, f32, rchunks));
-    sm_slots = std::max(sm_slots, coarse_slots_smem(pr->lv));
+    sm_slots = std::max(sm_slots, coarse_slots_it_smem(pr->lv, fp32(pr)));
     if (pr->tree) continue;
     sm_factor = std::max(sm_factor, coarse_factor_smem_bytes(pr->n_c, pr->bw, false));
     sm_solve = std::max(sm_solve, big_solve_smem_bytes(pr->n_c, pr->bw, stages));

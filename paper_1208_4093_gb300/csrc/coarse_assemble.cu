@@ -6,31 +6,30 @@
 // inside set I touches only I's nine modes; a bar crossing to a neighbour set
 // J touches 18 (I's at the owner a, J's at b with a minus sign).
 //
-// One CTA per set I sums the bars owned by its nodes into six 18 x 18 slots:
-// SELF (bars inside I, upper-left 9 x 9 used) and E, W, N, NE, NW (bars to the
-// neighbour set in that direction; rows/cols 0-8 = I's modes, 9-17 = J's).
+// The bars owned by set I's nodes are summed into six 2 q x 2 q slots:
+// SELF (bars inside I, upper-left q x q used) and E, W, N, NE, NW (bars to the
+// neighbour set in that direction; rows/cols 0..q-1 = I's modes, q.. = J's).
 // The translation/gradient entries (modes 1-6) do not depend on delta: they
-// are summed once at setup (FULL = true, delta = 0) into a base copy, and
-// every iteration only the entries that involve modes 7-9 are summed
-// (FULL = false).  For bars inside I with all four DOFs free the translation
-// terms vanish and the gradient terms are constants of the bar direction, so
-// those bars only accumulate e.delta sums per direction; bars touching a
-// constrained DOF use the general 9-term form.  All sums run in a fixed order
-// (per-thread node order, then a fixed-shape tree), so the result is the same
-// on every run.
+// are summed once at setup into a base copy, and every iteration only the
+// entries that involve the increment modes (7-9, and 10-12 with the force-
+// controlled modes of Eqs. 17-18) are summed.  For bars inside I with all four
+// DOFs free the translation terms vanish and the gradient terms are constants of
+// the bar direction, so those bars only accumulate e.delta sums per direction;
+// bars touching a constrained DOF use the general form.  All sums run in a fixed
+// order, so the result is the same on every run.
+#include <cooperative_groups.h>
+
 #include <type_traits>
 
 #include "hms_internal.cuh"
 #include "ptx.cuh"
 
+namespace cg = cooperative_groups;
+
 namespace hms {
 namespace {
 
 constexpr int NT = 256, NW = NT / 32;
-constexpr int NREG = 15;          // 3 directions x 3 delta modes + 6 delta-delta products
-constexpr int NGEN_DELTA = 24;    // (m, l), m in 6..8, l <= m
-constexpr int NGEN_FULL = 45;     // (m, l), l <= m < 9
-constexpr int LSTRIDE = 36;       // s[18], (EA/L) s[18]
 constexpr int RED_CHUNK = NW;     // accumulators per shared-memory reduction pass
 
 __device__ inline double warp_sum(double v) {
@@ -47,11 +46,6 @@ template <>
 __device__ inline double2 ld_delta<float2>(const float2* d, size_t n) {
   const float2 f = d[n];
   return make_double2((double)f.x, (double)f.y);
-}
-
-__device__ inline int gen_idx(int m, int l, bool full) {
-  if (full) return m * (m + 1) / 2 + l;
-  return (m == 6 ? 0 : (m == 7 ? 7 : 15)) + l;
 }
 
 // e . V_m at a node, modes m = 0..8 (Eqs. 9, 10, 13, 14), zero on constrained DOFs.
@@ -85,13 +79,6 @@ __device__ inline void mode_proj_t(AT ex, AT ey, AT xi, AT eta, unsigned fm, AT 
   s[7] = xi * ed;
   s[8] = eta * ed;
 }
-template <typename AT>
-__device__ inline AT warp_sum_t(AT v) {
-#pragma unroll
-  for (int m = 16; m > 0; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
-  return v;
-}
-
 struct ListCaps {
   int cap[6], off[6], total;
 };
@@ -112,131 +99,234 @@ __host__ __device__ inline ListCaps list_caps(int w, int h) {
   return c;
 }
 
-// AT: arithmetic of the per-bar products (double on the FP64 path; float on
-// the mixed path, where delta itself is FP32 and the products only
-// approximate K_aa, which leaves the iteration's fixed point unchanged because
-// P uses the FP64 residual).  On the mixed path the interface bars' products,
-// the sums over a slot's bars (in chunks of 16, the chunks added in FP64) and
-// the block reduction of the per-thread sums run in FP32 too; on the FP64
-// path everything is FP64.
-// The kernel body for set I.
-template <typename DT, bool FULL, typename AT>
-__device__ __forceinline__ void slots_body(const LatView lv, const DT* __restrict__ delta, double* __restrict__ slots,
-                                           const IterCtl* ctl, int I) {
+// The slot of an interface bar of direction d at node (il, jl) of the set, whose far
+// end lies in the set (dxs, dys) away, and its place in the slot's list.
+__device__ inline void slot_place(int d, int il, int jl, int dxs, int dys, int& slot, int& idx) {
+  if (dys == 0) {
+    slot = dxs > 0 ? SLOT_E : SLOT_W;
+    idx = dxs > 0 ? 2 * jl + (d == 1 ? 1 : 0) : jl;
+  } else if (dxs == 0) {
+    slot = SLOT_N;
+    idx = 2 * il + (d == 2 ? 1 : 0);
+  } else {
+    slot = dxs > 0 ? SLOT_NE : SLOT_NW;
+    idx = (dxs > 0) == (d == 1) ? 0 : 1;
+  }
+}
+
+// ---- setup: the entries of modes 1-6 ----
+// One CTA per set, FP64: the bars inside the set per thread, then a fixed-shape
+// tree; the interface bars' lists slot by slot, in index order.
+constexpr int QB = 6, NBASE = QB * (QB + 1) / 2;
+constexpr int LSTRIDE = 4 * QB;  // s_a, -s_b, k s_a, -k s_b
+__global__ void __launch_bounds__(NT) k_coarse_base(LatView lv, double* __restrict__ slots) {
   extern __shared__ double lists[];
-  if (ctl && *(volatile const int*)&ctl->done) return;
-  constexpr int NGEN = FULL ? NGEN_FULL : NGEN_DELTA;
+  const int I = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int SD = 2 * lv.q, SZ = SD * SD;
   const int Ix = I % lv.Mx, Iy = I / lv.Mx;
   const int i0 = Ix * lv.sx, j0 = Iy * lv.sy;
   const int w = min(lv.sx, lv.nx - i0), h = min(lv.sy, lv.ny - j0);
   const ListCaps LC = list_caps(w, h);
-  double* out = slots + (size_t)I * NSLOTS * SLOT_SIZE;
-
-  AT* la = reinterpret_cast<AT*>(lists);  // the interface lists, in AT
-  for (int q = tid; q < LC.total * LSTRIDE; q += NT) la[q] = AT(0);
-  for (int q = tid; q < NSLOTS * SLOT_SIZE; q += NT) out[q] = 0.0;
+  double* out = slots + (size_t)I * NSLOTS * SZ;
+  for (int q = tid; q < LC.total * LSTRIDE; q += NT) lists[q] = 0.0;
+  for (int q = tid; q < NSLOTS * SZ; q += NT) out[q] = 0.0;
   __syncthreads();
 
-  const double2 repI = lv.rep[I];
-  // set-relative coordinates of the regular-bar path in AT: xi = L (il + off/2) + c0x,
-  // eta = L sqrt3/2 jl + c0y; the far end of a bar of direction d adds (L e_x, L e_y)
-  const AT c0x = (AT)fma(lv.L, (double)i0, -repI.x), c0y = (AT)fma(lv.L * SQ3_2, (double)j0, -repI.y);
-  const AT LA = (AT)lv.L, LyA = (AT)(lv.L * SQ3_2);
-  AT reg[NREG];
-  AT gen[NGEN];
+  const double2 repI = lv.rep[I], none = make_double2(0.0, 0.0);
+  double gen[NBASE];
 #pragma unroll
-  for (int k = 0; k < NREG; ++k) reg[k] = AT(0);
+  for (int k = 0; k < NBASE; ++k) gen[k] = 0.0;
+  for (int t = tid; t < 3 * w * h; t += NT) {
+    const int q = t / 3, d = t - 3 * q;
+    const int il = q % w, jl = q / w, i = i0 + il, j = j0 + jl, off = j & 1;
+    const double k = bar_k(lv, i, j, d);
+    if (__double_as_longlong(k) == 0) continue;  // no bar (bar_k returns +0.0; EA > 0): an integer test
+    const int ib = (d == 0) ? i + 1 : (d == 1 ? i + off : i - 1 + off);
+    const int jb = (d == 0) ? j : j + 1;
+    const int dxs = (ib >= i0 + w) ? 1 : (ib < i0 ? -1 : 0);
+    const int dys = (jb >= j0 + h) ? 1 : 0;
+    const unsigned fa = lv.fix[(size_t)j * lv.nx + i], fb = lv.fix[(size_t)jb * lv.nx + ib];
+    const double ex = (d == 0) ? 1.0 : (d == 1 ? 0.5 : -0.5), ey = (d == 0) ? 0.0 : SQ3_2;
+    const double2 repJ = lv.rep[(Iy + dys) * lv.Mx + Ix + dxs];
+    double sa[NMODES], sb[NMODES];
+    mode_proj(ex, ey, node_x(lv, i, j) - repI.x, node_y(lv, j) - repI.y, fa, none, sa);
+    mode_proj(ex, ey, node_x(lv, ib, jb) - repJ.x, node_y(lv, jb) - repJ.y, fb, none, sb);
+    if (dxs == 0 && dys == 0) {
 #pragma unroll
-  for (int k = 0; k < NGEN; ++k) gen[k] = AT(0);
-
-  for (int q = tid; q < w * h; q += NT) {
-    const int il = q % w, jl = q / w;
-    const int i = i0 + il, j = j0 + jl;
-    const int off = j & 1;
-    const size_t na = (size_t)j * lv.nx + i;
-    const unsigned fa = lv.fix[na];
-    const DT dra = FULL ? DT{} : delta[na];
-    const AT xiaA = fma(LA, (AT)il + (off ? AT(0.5) : AT(0)), c0x), etaaA = fma(LyA, (AT)jl, c0y);
+      for (int m = 0; m < QB; ++m) sa[m] -= sb[m];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const double k = bar_k(lv, i, j, d);
-      if (__double_as_longlong(k) == 0) continue;  // no bar (bar_k returns +0.0; EA > 0): an integer test
-      const int ib = (d == 0) ? i + 1 : (d == 1 ? i + off : i - 1 + off);
-      const int jb = (d == 0) ? j : j + 1;
-      const size_t nbn = (size_t)jb * lv.nx + ib;
-      const unsigned fb = lv.fix[nbn];
-      const double ex = (d == 0) ? 1.0 : (d == 1 ? 0.5 : -0.5), ey = (d == 0) ? 0.0 : SQ3_2;
-      const int dxs = (ib >= i0 + w) ? 1 : (ib < i0 ? -1 : 0);
-      const int dys = (jb >= j0 + h) ? 1 : 0;
-      // FP64 node data of the general and interface paths (not of regular bars)
-      auto fp64_ends = [&](double2& da, double2& db, double& xa, double& ya, double& xb, double& yb) {
-        da = FULL ? make_double2(0.0, 0.0) : ld_delta(delta, na);
-        db = FULL ? make_double2(0.0, 0.0) : ld_delta(delta, nbn);
-        xa = node_x(lv, i, j), ya = node_y(lv, j);
-        xb = node_x(lv, ib, jb), yb = node_y(lv, jb);
-      };
-      if (dxs == 0 && dys == 0) {
-        if (!FULL && fa == 0u && fb == 0u) {
-          // regular bar: s_0 = s_1 = 0, s_2..s_5 constants of the direction;
-          // everything in AT from the raw delta
-          const DT drb = delta[nbn];
-          const AT exA = (AT)ex, eyA = (AT)ey;
-          const AT ea = fma(eyA, (AT)dra.y, exA * (AT)dra.x), eb = fma(eyA, (AT)drb.y, exA * (AT)drb.x);
-          const AT xibA = fma(LA, exA, xiaA), etabA = (d == 0) ? etaaA : etaaA + LyA;
-          const AT s6 = ea - eb;
-          const AT s7 = fma(xiaA, ea, -(xibA * eb));
-          const AT s8 = fma(etaaA, ea, -(etabA * eb));
-          const AT kk = (AT)k;
-          const AT k6 = kk * s6, k7 = kk * s7, k8 = kk * s8;
-          reg[3 * d + 0] += k6;
-          reg[3 * d + 1] += k7;
-          reg[3 * d + 2] += k8;
-          reg[9] = fma(k6, s6, reg[9]);
-          reg[10] = fma(k7, s6, reg[10]);
-          reg[11] = fma(k8, s6, reg[11]);
-          reg[12] = fma(k7, s7, reg[12]);
-          reg[13] = fma(k8, s7, reg[13]);
-          reg[14] = fma(k8, s8, reg[14]);
-        } else {
-          double2 da, db;
-          double xa, ya, xb, yb;
-          fp64_ends(da, db, xa, ya, xb, yb);
-          const double xia = xa - repI.x, etaa = ya - repI.y;
-          const double xib = xb - repI.x, etab = yb - repI.y;
-          double sa[9], sb[9];
-          mode_proj(ex, ey, xia, etaa, fa, da, sa);
-          mode_proj(ex, ey, xib, etab, fb, db, sb);
+      for (int m = 0; m < QB; ++m)
 #pragma unroll
-          for (int m = 0; m < 9; ++m) sa[m] -= sb[m];
-          if (FULL) {
+        for (int l = 0; l <= m; ++l) gen[m * (m + 1) / 2 + l] = fma(k * sa[m], sa[l], gen[m * (m + 1) / 2 + l]);
+      continue;
+    }
+    int slot, idx;
+    slot_place(d, il, jl, dxs, dys, slot, idx);
+    double* e = lists + (size_t)(LC.off[slot] + idx) * LSTRIDE;
 #pragma unroll
-            for (int m = 0; m < 9; ++m)
-#pragma unroll
-              for (int l = 0; l <= m; ++l)
-                gen[m * (m + 1) / 2 + l] = fma((AT)(k * sa[m]), (AT)sa[l], gen[m * (m + 1) / 2 + l]);
-          } else {
-#pragma unroll
-            for (int m = 6; m < 9; ++m)
-#pragma unroll
-              for (int l = 0; l <= m; ++l) {
-                const int g = (m == 6 ? 0 : (m == 7 ? 7 : 15)) + l;
-                gen[g] = fma((AT)(k * sa[m]), (AT)sa[l], gen[g]);
-              }
-          }
-        }
-      }
-      // else an interface bar: the pass below
+    for (int m = 0; m < QB; ++m) {
+      e[m] = sa[m];
+      e[QB + m] = -sb[m];
+      e[2 * QB + m] = k * sa[m];
+      e[3 * QB + m] = -(k * sb[m]);
     }
   }
+  // deterministic block sums of the per-thread accumulators, RED_CHUNK at a time
+  double* red = lists + (size_t)LC.total * LSTRIDE;  // RED_CHUNK x NT
+  double* tot = red + RED_CHUNK * NT;                // NBASE CTA totals
+#pragma unroll
+  for (int c0 = 0; c0 < NBASE; c0 += RED_CHUNK) {
+#pragma unroll
+    for (int q = 0; q < RED_CHUNK; ++q)
+      if (c0 + q < NBASE) red[q * NT + tid] = gen[c0 + q];
+    __syncthreads();
+    if (c0 + warp < NBASE) {
+      const double* q = red + warp * NT + lane;
+      double v = q[0];
+#pragma unroll
+      for (int ww = 1; ww < NW; ++ww) v += q[32 * ww];
+      v = warp_sum(v);
+      if (lane == 0) tot[c0 + warp] = v;
+    }
+    __syncthreads();
+  }
+  if (tid < QB * QB) {
+    const int m = tid / QB, l = tid % QB;
+    const int mm = m > l ? m : l, ll = m > l ? l : m;
+    out[SLOT_SELF * SZ + m * SD + l] = tot[mm * (mm + 1) / 2 + ll];
+  }
+  // entries (p, c) of I's modes (0..5) and the neighbour's (6..11)
+  for (int q = tid; q < 5 * 4 * QB * QB; q += NT) {
+    const int slot = 1 + q / (4 * QB * QB), r = q % (4 * QB * QB), p = r / (2 * QB), c = r % (2 * QB);
+    if (c < p) continue;
+    const double* e = lists + (size_t)LC.off[slot] * LSTRIDE;
+    double v = 0.0;
+    for (int b = 0; b < LC.cap[slot]; ++b, e += LSTRIDE) v = fma(e[2 * QB + p], e[c], v);
+    const int pp = p < QB ? p : lv.q + p - QB, cc = c < QB ? c : lv.q + c - QB;
+    out[slot * SZ + pp * SD + cc] = v;
+    out[slot * SZ + cc * SD + pp] = v;
+  }
+}
 
-  // Interface bars (the far end in a neighbour set), apart from the node loop
-  // so that whole warps take their FP64 work (in the node loop one lane of a
-  // warp would, while the FP64 pipe spends a warp instruction's full time):
-  // the right column's E and NE bars, the left column's NW bars, the top
-  // row's NE and NW bars.  Each list entry is written by one item; the sums
-  // over the lists below are unchanged.
-  for (int t = tid; t < 3 * h + 2 * w; t += NT) {
+// mode_proj with the force-controlled modes 10-12 of Eqs. 17-18: s_9 = e.delta^RF,
+// s_10 = xi s_9, s_11 = eta s_9
+__device__ inline void mode_proj12(double ex, double ey, double xi, double eta, unsigned fm, double2 dl,
+                                   double2 df, double* s) {
+  mode_proj(ex, ey, xi, eta, fm, dl, s);
+  const double ef = ex * df.x + ey * df.y;  // delta^RF is 0 on constrained DOFs
+  s[9] = ef;
+  s[10] = xi * ef;
+  s[11] = eta * ef;
+}
+// ---- every update: the entries that involve the increment modes ----
+// The bars inside a set in SP fixed parts of its nodes, a warp each (32 nodes, then
+// every 32 SP-th), summed part by part; the bars to the neighbours slot by slot in
+// list order.  Neither depends on how many CTAs (of one cluster) share a set's parts
+// and slots, so C = 1 to 4 CTAs give the same bits: four where 152 SMs leave room
+// for four per set.  A warp of each SM quarter is all that the FP64 pipe can use.
+//
+// Q = 9 or 12 modes; NS = 3 or 6 projections s_6.. of a bar.  A regular bar (all
+// four DOFs free) adds k s_m to its direction's sum (s_2..s_5 are constants of the
+// direction) and k s_m s_l to the products', 50 FP64 operations per node for Q = 9
+// and 8 for its three bars' projections; bars at constrained DOFs take the general
+// form in a second pass of the warps that have any.  PT: arithmetic of the
+// projections, AT: of the products (the mixed form's: PT FP64 with the
+// force-controlled modes, else FP32).
+//
+// Measured (us, before: one CTA of 256 threads per set, with Q = 12 every bar in
+// the general form): FP64, 16 sets of 16 x 16 nodes 28 -> 23, 256 of 64 x 64 250
+// -> 190; mixed 52 -> 43; Q = 12, 48 of 32 x 32 115 -> 65, mixed 98 -> 48.
+constexpr int SP = 16;
+template <int Q>
+struct SlotSums {
+  static constexpr int NS = Q == NMODES_RF ? 6 : 3;
+  static constexpr int NLIN = 3 * NS, NQUAD = NS * (NS + 1) / 2;
+  static constexpr int NGEN = NS * (NS + 1) / 2 + 6 * NS;  // (m, l), 6 <= m < Q, l <= m
+  static constexpr int NACC = NLIN + NQUAD + NGEN;
+  static constexpr int NPAIR = 2 * Q * (2 * Q + 1) / 2 - 78;  // p <= c of a slot, one of them >= 6
+};
+// the pairs of a slot's entries that involve an increment mode
+template <int Q>
+struct SlotPairs {
+  unsigned char p[SlotSums<Q>::NPAIR], c[SlotSums<Q>::NPAIR];
+};
+template <int Q>
+constexpr SlotPairs<Q> slot_pairs() {
+  SlotPairs<Q> t{};
+  int n = 0;
+  for (int p = 0; p < 2 * Q; ++p)
+    for (int c = p; c < 2 * Q; ++c)
+      if (p % Q >= 6 || c % Q >= 6) {
+        t.p[n] = (unsigned char)p;
+        t.c[n++] = (unsigned char)c;
+      }
+  return t;
+}
+__device__ const SlotPairs<NMODES> PAIRS9 = slot_pairs<NMODES>();
+__device__ const SlotPairs<NMODES_RF> PAIRS12 = slot_pairs<NMODES_RF>();
+
+// Sums over a warp of N values per lane, N adds and a few: value k's sum ends in
+// lane k (k < 32) and, of values 32.., in lane k - 32, and is stored at dst[k].
+template <int N, typename AT>
+__device__ __forceinline__ void warp_sums(AT (&v)[N], double* dst) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int b = 0; b < N; b += 32) {
+    AT x[32];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) x[k] = b + k < N ? v[b + k < N ? b + k : 0] : AT(0);
+    // halve the values, not the lanes: after step m a lane holds those whose number
+    // agrees with its own in the bits seen
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) {
+      const bool up = lane & m;
+#pragma unroll
+      for (int k = 0; k < m; ++k) {
+        if (b + k >= N) continue;  // neither half holds a value
+        const AT give = up ? x[k] : x[k + m], keep = up ? x[k + m] : x[k];
+        x[k] = keep + __shfl_xor_sync(0xffffffffu, give, m);
+      }
+    }
+    if (b + lane < N) dst[b + lane] = (double)x[0];
+  }
+}
+
+template <int Q, typename LT>
+__host__ __device__ inline size_t slots_it_smem(const ListCaps& LC) {
+  // the lists (s_a, -s_b, k s_a, -k s_b), then the parts' sums
+  return (size_t)LC.total * 4 * Q * sizeof(LT) + (size_t)SP * SlotSums<Q>::NACC * sizeof(double);
+}
+
+template <typename DT, int Q, typename AT>
+__device__ __forceinline__ void slots_it_body(const LatView& lv, const DT* __restrict__ delta,
+                                              const DT* __restrict__ delta_rf, double* __restrict__ slots, int I) {
+  using SS = SlotSums<Q>;
+  using LT = typename std::conditional<Q == NMODES_RF, double, AT>::type;  // of the lists
+  using PT = LT;
+  constexpr int NS = SS::NS, NF = NS / 3, LST = 4 * Q, SD = 2 * Q, SZ = SD * SD;
+  extern __shared__ double lists[];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
+  const int Ix = I % lv.Mx, Iy = I / lv.Mx;
+  const int i0 = Ix * lv.sx, j0 = Iy * lv.sy;
+  const int w = min(lv.sx, lv.nx - i0), h = min(lv.sy, lv.ny - j0);
+  const ListCaps LC = list_caps(w, h);
+  double* out = slots + (size_t)I * NSLOTS * SZ;
+  double* part = lists;  // SP x NACC (rank 0's holds the cluster's)
+  LT* la = reinterpret_cast<LT*>(lists + SP * SS::NACC);
+  auto mine = [&](int slot) { return (slot - 1) % C == rank; };  // slots E, W, N, NE, NW
+  for (int sl = 1; sl < NSLOTS; ++sl)
+    if (mine(sl))
+      for (int q = tid; q < LC.cap[sl] * LST; q += nt) la[(size_t)LC.off[sl] * LST + q] = LT(0);
+  __syncthreads();
+
+  // Interface bars (the far end in a neighbour set): the right column's E and NE
+  // bars, the left column's NW bars, the top row's NE and NW bars.  Each list entry
+  // is written by one item.
+  const double2 repI = lv.rep[I];
+  for (int t = tid; t < 3 * h + 2 * w; t += nt) {
     int il, jl, d;
     if (t < 2 * h) {
       il = w - 1, jl = t >> 1, d = t & 1;
@@ -248,344 +338,222 @@ __device__ __forceinline__ void slots_body(const LatView lv, const DT* __restric
       if ((d == 1 && il == w - 1) || (d == 2 && il == 0)) continue;  // in the column groups
     }
     const int i = i0 + il, j = j0 + jl, off = j & 1;
-    const double k = bar_k(lv, i, j, d);
-    if (__double_as_longlong(k) == 0) continue;
     const int ib = (d == 0) ? i + 1 : (d == 1 ? i + off : i - 1 + off);
     const int jb = (d == 0) ? j : j + 1;
     const int dxs = (ib >= i0 + w) ? 1 : (ib < i0 ? -1 : 0);
     const int dys = (jb >= j0 + h) ? 1 : 0;
-    if (dxs == 0 && dys == 0) continue;  // an inner bar (node loop)
+    if (dxs == 0 && dys == 0) continue;  // an inner bar (below)
+    int slot, idx;
+    slot_place(d, il, jl, dxs, dys, slot, idx);
+    if (!mine(slot)) continue;
+    const double k = bar_k(lv, i, j, d);
+    if (__double_as_longlong(k) == 0) continue;  // no bar (bar_k returns +0.0; EA > 0): an integer test
     const size_t na = (size_t)j * lv.nx + i, nbn = (size_t)jb * lv.nx + ib;
     const unsigned fa = lv.fix[na], fb = lv.fix[nbn];
     const double ex = (d == 0) ? 1.0 : (d == 1 ? 0.5 : -0.5), ey = (d == 0) ? 0.0 : SQ3_2;
-    auto fp64_ends = [&](double2& da, double2& db, double& xa, double& ya, double& xb, double& yb) {
-      da = FULL ? make_double2(0.0, 0.0) : ld_delta(delta, na);
-      db = FULL ? make_double2(0.0, 0.0) : ld_delta(delta, nbn);
-      xa = node_x(lv, i, j), ya = node_y(lv, j);
-      xb = node_x(lv, ib, jb), yb = node_y(lv, jb);
-    };
-    {
-      int slot, idx;
-      if (dys == 0) {
-        if (dxs > 0) {
-          slot = SLOT_E;
-          idx = 2 * jl + (d == 1 ? 1 : 0);
-        } else {
-          slot = SLOT_W;
-          idx = jl;
-        }
-      } else if (dxs == 0) {
-        slot = SLOT_N;
-        idx = 2 * il + (d == 2 ? 1 : 0);
-      } else if (dxs > 0) {
-        slot = SLOT_NE;
-        idx = (d == 1) ? 0 : 1;
-      } else {
-        slot = SLOT_NW;
-        idx = (d == 2) ? 0 : 1;
-      }
-      double2 da, db;
-      double xa, ya, xb, yb;
-      fp64_ends(da, db, xa, ya, xb, yb);
-      const int Jx = Ix + dxs, Jy = Iy + dys;
-      const double2 repJ = lv.rep[Jy * lv.Mx + Jx];
-      AT* e = la + (size_t)(LC.off[slot] + idx) * LSTRIDE;
-      AT sa[9], sb[9];
-      mode_proj_t<AT>((AT)ex, (AT)ey, (AT)(xa - repI.x), (AT)(ya - repI.y), fa, (AT)da.x, (AT)da.y, sa);
-      mode_proj_t<AT>((AT)ex, (AT)ey, (AT)(xb - repJ.x), (AT)(yb - repJ.y), fb, (AT)db.x, (AT)db.y, sb);
-      const AT kA = (AT)k;
-#pragma unroll
-      for (int m = 0; m < 9; ++m) {
-        e[m] = sa[m];
-        e[9 + m] = -sb[m];
-        e[18 + m] = kA * sa[m];
-        e[27 + m] = -(kA * sb[m]);
-      }
-    }
-  }
-
-  // deterministic block sums of the per-thread accumulators, eight at a time
-  // through shared memory: warp a adds accumulator a of the CTA's threads
-  // lane by lane in thread order, then a shuffle tree finishes it
-  constexpr int NACC = NREG + NGEN;
-  double* red = lists + (size_t)LC.total * LSTRIDE;  // RED_CHUNK x NT
-  double* tot = red + RED_CHUNK * NT;                 // NACC CTA totals
-  AT* redA = reinterpret_cast<AT*>(red);
-#pragma unroll
-  for (int c0 = 0; c0 < NACC; c0 += RED_CHUNK) {
-#pragma unroll
-    for (int q = 0; q < RED_CHUNK; ++q) {
-      const int k = c0 + q;
-      if (k < NREG) redA[q * NT + tid] = reg[k];
-      else if (k < NACC) redA[q * NT + tid] = gen[k - NREG];
-    }
-    __syncthreads();
-    if (c0 + warp < NACC) {
-      const AT* q = redA + warp * NT + lane;
-      AT v = q[0];
-#pragma unroll
-      for (int ww = 1; ww < NW; ++ww) v += q[32 * ww];
-      v = warp_sum_t<AT>(v);
-      if (lane == 0) tot[c0 + warp] = (double)v;
-    }
-    __syncthreads();
-  }
-
-  // SELF slot (upper-left 9 x 9)
-  if (tid < 81) {
-    const int m = tid / 9, l = tid % 9;
-    const int mm = m > l ? m : l, ll = m > l ? l : m;
-    double v = 0.0;
-    bool have = false;
-    if (FULL) {
-      v = tot[NREG + mm * (mm + 1) / 2 + ll];
-      have = true;
-    } else if (mm >= 6) {
-      v = tot[NREG + gen_idx(mm, ll, false)];
-      const double L = lv.L;
-      // constants s_2..s_5 of a regular bar of direction d: -L e_x^2, -L e_x e_y, -L e_y e_x, -L e_y^2
-      if (ll >= 2 && ll <= 5) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          const double ex = (d == 0) ? 1.0 : (d == 1 ? 0.5 : -0.5), ey = (d == 0) ? 0.0 : SQ3_2;
-          const double c = (ll == 2) ? -L * ex * ex : (ll == 5 ? -L * ey * ey : -L * ex * ey);
-          v = fma(c, tot[3 * d + (mm - 6)], v);
-        }
-      } else if (ll >= 6) {
-        const int qi = (mm == 6) ? 9 : (mm == 7 ? (ll == 6 ? 10 : 12) : (ll == 6 ? 11 : (ll == 7 ? 13 : 14)));
-        v += tot[qi];
-      }
-      have = true;
-    }
-    if (have) out[SLOT_SELF * SLOT_SIZE + m * SLOT_DIM + l] = v;
-  }
-  // interface slots: sum over each list in index order; each slot is
-  // symmetric (a sum of (EA/L) s s^T), so only p <= c is summed
-  constexpr int NUP = SLOT_DIM * (SLOT_DIM + 1) / 2;
-  for (int q = tid; q < 5 * NUP; q += NT) {
-    const int slot = 1 + q / NUP;
-    int r = q % NUP, p = 0;
-    while (r >= SLOT_DIM - p) r -= SLOT_DIM - p, ++p;
-    const int c = p + r;
-    const bool dp = (p % 9) >= 6, dc = (c % 9) >= 6;
-    if (!FULL && !dp && !dc) continue;
-    const AT* e = la + (size_t)LC.off[slot] * LSTRIDE;
-    double v = 0.0;
-    if constexpr (sizeof(AT) == 8) {
-      for (int b = 0; b < LC.cap[slot]; ++b, e += LSTRIDE) v = fma(e[18 + p], e[c], v);
+    const double2 repJ = lv.rep[(Iy + dys) * lv.Mx + Ix + dxs];
+    const double xa = node_x(lv, i, j), ya = node_y(lv, j), xb = node_x(lv, ib, jb), yb = node_y(lv, jb);
+    const double2 da = ld_delta(delta, na), db = ld_delta(delta, nbn);
+    LT sa[Q], sb[Q];
+    if constexpr (Q == NMODES_RF) {
+      mode_proj12(ex, ey, xa - repI.x, ya - repI.y, fa, da, ld_delta(delta_rf, na), sa);
+      mode_proj12(ex, ey, xb - repJ.x, yb - repJ.y, fb, db, ld_delta(delta_rf, nbn), sb);
     } else {
-      for (int b0 = 0; b0 < LC.cap[slot]; b0 += 16) {
-        AT part = AT(0);
-        for (int b = b0; b < b0 + 16 && b < LC.cap[slot]; ++b, e += LSTRIDE) part = fma(e[18 + p], e[c], part);
-        v += (double)part;
+      mode_proj_t<LT>((LT)ex, (LT)ey, (LT)(xa - repI.x), (LT)(ya - repI.y), fa, (LT)da.x, (LT)da.y, sa);
+      mode_proj_t<LT>((LT)ex, (LT)ey, (LT)(xb - repJ.x), (LT)(yb - repJ.y), fb, (LT)db.x, (LT)db.y, sb);
+    }
+    LT* e = la + (size_t)(LC.off[slot] + idx) * LST;
+    const LT kL = (LT)k;
+#pragma unroll
+    for (int m = 0; m < Q; ++m) {
+      e[m] = sa[m];
+      e[Q + m] = -sb[m];
+      e[2 * Q + m] = kL * sa[m];
+      e[3 * Q + m] = -(kL * sb[m]);
+    }
+  }
+
+  // ---- bars inside the set ----
+  double* part0 = cluster.map_shared_rank(part, 0);
+  const PT LA = (PT)lv.L, LyA = (PT)(lv.L * SQ3_2);
+  const PT c0x = (PT)fma(lv.L, (double)i0, -repI.x), c0y = (PT)fma(lv.L * SQ3_2, (double)j0, -repI.y);
+  for (int pt = rank + C * warp; pt < SP; pt += C * (nt >> 5)) {
+    AT acc[SS::NLIN + SS::NQUAD];
+#pragma unroll
+    for (int k = 0; k < SS::NLIN + SS::NQUAD; ++k) acc[k] = AT(0);
+    bool special = false;  // a bar at a constrained DOF
+#pragma unroll 1
+    for (int q = 32 * pt + lane; q < w * h; q += 32 * SP) {
+      const int jl = q / w, il = q - jl * w;
+      const int i = i0 + il, j = j0 + jl, off = j & 1;
+      const size_t na = (size_t)j * lv.nx + i;
+      const unsigned fa = lv.fix[na];
+      DT da[NF], db[NF];
+      da[0] = delta[na];
+      if constexpr (NF == 2) da[1] = delta_rf[na];
+      const PT xi = fma(LA, (PT)il + (off ? PT(0.5) : PT(0)), c0x), eta = fma(LyA, (PT)jl, c0y);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const int ib = (d == 0) ? i + 1 : (d == 1 ? i + off : i - 1 + off);
+        const int jb = (d == 0) ? j : j + 1;
+        if (ib >= i0 + w || ib < i0 || jb >= j0 + h) continue;
+        const double k = bar_k(lv, i, j, d);
+        if (__double_as_longlong(k) == 0) continue;
+        const size_t nbn = (size_t)jb * lv.nx + ib;
+        if ((fa | lv.fix[nbn]) != 0u) {
+          special = true;
+          continue;
+        }
+        db[0] = delta[nbn];
+        if constexpr (NF == 2) db[1] = delta_rf[nbn];
+        // e = (1, 0), (1/2, sqrt3/2), (-1/2, sqrt3/2); the far end at (xi, eta) + L e:
+        // s_6 = e.da - e.db, s_7 = xi s_6 - L e_x e.db, s_8 = eta s_6 - L e_y e.db
+        const PT hx = d == 1 ? PT(0.5) : PT(-0.5), kP = (PT)k;
+        PT s[NS];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+          const PT ea = d == 0 ? (PT)da[f].x : fma(hx, (PT)da[f].x, (PT)SQ3_2 * (PT)da[f].y);
+          const PT eb = d == 0 ? (PT)db[f].x : fma(hx, (PT)db[f].x, (PT)SQ3_2 * (PT)db[f].y);
+          s[3 * f] = ea - eb;
+          s[3 * f + 1] = fma(xi, s[3 * f], (d == 0 ? -LA : -(hx * LA)) * eb);
+          s[3 * f + 2] = d == 0 ? eta * s[3 * f] : fma(eta, s[3 * f], -LyA * eb);
+        }
+#pragma unroll
+        for (int m = 0; m < NS; ++m) {
+          const AT km = (AT)(kP * s[m]);
+          acc[NS * d + m] += km;
+#pragma unroll
+          for (int l = 0; l <= m; ++l)
+            acc[SS::NLIN + m * (m + 1) / 2 + l] = fma(km, (AT)s[l], acc[SS::NLIN + m * (m + 1) / 2 + l]);
+        }
       }
     }
-    out[slot * SLOT_SIZE + p * SLOT_DIM + c] = v;
-    out[slot * SLOT_SIZE + c * SLOT_DIM + p] = v;
+    double* dst = part0 + (size_t)pt * SS::NACC;
+    warp_sums(acc, dst);
+    dst += SS::NLIN + SS::NQUAD;
+    if (!__any_sync(0xffffffffu, special)) {
+      for (int k = lane; k < SS::NGEN; k += 32) dst[k] = 0.0;
+      continue;
+    }
+    AT gen[SS::NGEN];
+#pragma unroll
+    for (int k = 0; k < SS::NGEN; ++k) gen[k] = AT(0);
+#pragma unroll 1
+    for (int q = 32 * pt + lane; q < w * h; q += 32 * SP) {
+      const int jl = q / w, il = q - jl * w;
+      const int i = i0 + il, j = j0 + jl, off = j & 1;
+      const size_t na = (size_t)j * lv.nx + i;
+      const unsigned fa = lv.fix[na];
+#pragma unroll 1
+      for (int d = 0; d < 3; ++d) {
+        const int ib = (d == 0) ? i + 1 : (d == 1 ? i + off : i - 1 + off);
+        const int jb = (d == 0) ? j : j + 1;
+        if (ib >= i0 + w || ib < i0 || jb >= j0 + h) continue;
+        const double k = bar_k(lv, i, j, d);
+        if (__double_as_longlong(k) == 0) continue;
+        const size_t nbn = (size_t)jb * lv.nx + ib;
+        const unsigned fb = lv.fix[nbn];
+        if ((fa | fb) == 0u) continue;
+        const double ex = (d == 0) ? 1.0 : (d == 1 ? 0.5 : -0.5), ey = (d == 0) ? 0.0 : SQ3_2;
+        const double xa = node_x(lv, i, j) - repI.x, ya = node_y(lv, j) - repI.y;
+        const double xb = node_x(lv, ib, jb) - repI.x, yb = node_y(lv, jb) - repI.y;
+        double sa[Q], sb[Q];
+        if constexpr (Q == NMODES_RF) {
+          mode_proj12(ex, ey, xa, ya, fa, ld_delta(delta, na), ld_delta(delta_rf, na), sa);
+          mode_proj12(ex, ey, xb, yb, fb, ld_delta(delta, nbn), ld_delta(delta_rf, nbn), sb);
+        } else {
+          mode_proj(ex, ey, xa, ya, fa, ld_delta(delta, na), sa);
+          mode_proj(ex, ey, xb, yb, fb, ld_delta(delta, nbn), sb);
+        }
+#pragma unroll
+        for (int m = 0; m < Q; ++m) sa[m] -= sb[m];
+#pragma unroll
+        for (int m = 6; m < Q; ++m)
+#pragma unroll
+          for (int l = 0; l <= m; ++l) {
+            const int g = m * (m + 1) / 2 - 21 + l;
+            gen[g] = fma((AT)(k * sa[m]), (AT)sa[l], gen[g]);
+          }
+      }
+    }
+    warp_sums(gen, dst);
   }
-}
-
-template <typename DT, bool FULL, typename AT>
-__global__ void __launch_bounds__(NT) k_coarse_slots(LatView lv, const DT* __restrict__ delta,
-                                                     double* __restrict__ slots, const IterCtl* ctl) {
-  dep_wait();
-  slots_body<DT, FULL, AT>(lv, delta, slots, ctl, blockIdx.x);
-}
-
-// ---- q = 12: the force-controlled modes 10-12 of Eqs. 17-18 as well ----
-// The same bar-by-bar sums with every bar on the general path: the mode
-// projections s_0..s_8 of mode_proj and s_9 = e.delta^RF, s_10 = xi s_9,
-// s_11 = eta s_9; slots of 24 x 24 (rows/cols 0-11 = I's modes, 12-23 = J's).
-constexpr int Q12 = NMODES_RF, SD12 = 2 * Q12, SS12 = SD12 * SD12;
-constexpr int LSTRIDE12 = 4 * Q12;      // s_a, -s_b, k s_a, -k s_b
-constexpr int NGEN12_FULL = 21;         // (m, l), l <= m < 6
-constexpr int NGEN12_DELTA = 57;        // (m, l), m in 6..11, l <= m
-
-__device__ inline void mode_proj12(double ex, double ey, double xi, double eta, unsigned fm, double2 dl,
-                                   double2 df, double* s) {
-  mode_proj(ex, ey, xi, eta, fm, dl, s);
-  const double ef = ex * df.x + ey * df.y;  // delta^RF is 0 on constrained DOFs
-  s[9] = ef;
-  s[10] = xi * ef;
-  s[11] = eta * ef;
-}
-__device__ inline int gen12_idx(int m, int l, bool full) {
-  return full ? m * (m + 1) / 2 + l : m * (m + 1) / 2 - 21 + l;
-}
-
-template <typename DT, bool FULL, typename AT>
-__device__ __forceinline__ void slots12_body(const LatView lv, const DT* __restrict__ delta,
-                                             const DT* __restrict__ delta_rf, double* __restrict__ slots,
-                                             const IterCtl* ctl, int I) {
-  extern __shared__ double lists[];
-  if (ctl && *(volatile const int*)&ctl->done) return;
-  constexpr int NGEN = FULL ? NGEN12_FULL : NGEN12_DELTA;
-  constexpr int MLO = FULL ? 0 : 6, MHI = FULL ? 6 : Q12;  // rows m of the sums
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int Ix = I % lv.Mx, Iy = I / lv.Mx;
-  const int i0 = Ix * lv.sx, j0 = Iy * lv.sy;
-  const int w = min(lv.sx, lv.nx - i0), h = min(lv.sy, lv.ny - j0);
-  const ListCaps LC = list_caps(w, h);
-  double* out = slots + (size_t)I * NSLOTS * SS12;
-
-  for (int q = tid; q < LC.total * LSTRIDE12; q += NT) lists[q] = 0.0;
-  for (int q = tid; q < NSLOTS * SS12; q += NT) out[q] = 0.0;
   __syncthreads();
 
-  const double2 repI = lv.rep[I];
-  AT gen[NGEN];
-#pragma unroll
-  for (int k = 0; k < NGEN; ++k) gen[k] = AT(0);
-  auto ld = [&](const DT* p, size_t n) { return FULL ? make_double2(0.0, 0.0) : ld_delta(p, n); };
-
-  for (int q = tid; q < w * h; q += NT) {
-    const int il = q % w, jl = q / w;
-    const int i = i0 + il, j = j0 + jl;
-    const int off = j & 1;
-    const size_t na = (size_t)j * lv.nx + i;
-    const unsigned fa = lv.fix[na];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const double k = bar_k(lv, i, j, d);
-      if (__double_as_longlong(k) == 0) continue;
-      const int ib = (d == 0) ? i + 1 : (d == 1 ? i + off : i - 1 + off);
-      const int jb = (d == 0) ? j : j + 1;
-      if (ib >= i0 + w || ib < i0 || jb >= j0 + h) continue;  // interface bar: the pass below
-      const size_t nbn = (size_t)jb * lv.nx + ib;
-      const unsigned fb = lv.fix[nbn];
-      const double ex = (d == 0) ? 1.0 : (d == 1 ? 0.5 : -0.5), ey = (d == 0) ? 0.0 : SQ3_2;
-      double sa[Q12], sb[Q12];
-      mode_proj12(ex, ey, node_x(lv, i, j) - repI.x, node_y(lv, j) - repI.y, fa, ld(delta, na), ld(delta_rf, na),
-                  sa);
-      mode_proj12(ex, ey, node_x(lv, ib, jb) - repI.x, node_y(lv, jb) - repI.y, fb, ld(delta, nbn),
-                  ld(delta_rf, nbn), sb);
-#pragma unroll
-      for (int m = 0; m < Q12; ++m) sa[m] -= sb[m];
-#pragma unroll
-      for (int m = MLO; m < MHI; ++m)
-#pragma unroll
-        for (int l = 0; l <= m; ++l) {
-          const int g = gen12_idx(m, l, FULL);
-          gen[g] = fma((AT)(k * sa[m]), (AT)sa[l], gen[g]);
-        }
-    }
-  }
-
-  // interface bars (the far end in a neighbour set), as in slots_body
-  for (int t = tid; t < 3 * h + 2 * w; t += NT) {
-    int il, jl, d;
-    if (t < 2 * h) {
-      il = w - 1, jl = t >> 1, d = t & 1;
-    } else if (t < 3 * h) {
-      il = 0, jl = t - 2 * h, d = 2;
-    } else {
-      const int u = t - 3 * h;
-      il = u >> 1, jl = h - 1, d = 1 + (u & 1);
-      if ((d == 1 && il == w - 1) || (d == 2 && il == 0)) continue;
-    }
-    const int i = i0 + il, j = j0 + jl, off = j & 1;
-    const double k = bar_k(lv, i, j, d);
-    if (__double_as_longlong(k) == 0) continue;
-    const int ib = (d == 0) ? i + 1 : (d == 1 ? i + off : i - 1 + off);
-    const int jb = (d == 0) ? j : j + 1;
-    const int dxs = (ib >= i0 + w) ? 1 : (ib < i0 ? -1 : 0);
-    const int dys = (jb >= j0 + h) ? 1 : 0;
-    if (dxs == 0 && dys == 0) continue;
-    const size_t na = (size_t)j * lv.nx + i, nbn = (size_t)jb * lv.nx + ib;
-    const unsigned fa = lv.fix[na], fb = lv.fix[nbn];
-    const double ex = (d == 0) ? 1.0 : (d == 1 ? 0.5 : -0.5), ey = (d == 0) ? 0.0 : SQ3_2;
-    int slot, idx;
-    if (dys == 0) {
-      if (dxs > 0) {
-        slot = SLOT_E;
-        idx = 2 * jl + (d == 1 ? 1 : 0);
+  // the slots' sums over their lists
+  for (int sl = 1; sl < NSLOTS; ++sl) {
+    if (!mine(sl)) continue;
+    const LT* e0 = la + (size_t)LC.off[sl] * LST;
+    // one slot's entries after another's on the same threads would leave most idle:
+    // slot sl starts at its own place in the CTA
+    for (int q = (tid + nt - (sl - 1) / C * SS::NPAIR % nt) % nt; q < SS::NPAIR; q += nt) {
+      const SlotPairs<Q>& T = *[]() {
+        if constexpr (Q == NMODES_RF) return &PAIRS12;
+        else return &PAIRS9;
+      }();
+      const int p = T.p[q], c = T.c[q];
+      const LT* e = e0;
+      double v = 0.0;
+      if constexpr (sizeof(LT) == 8) {
+        for (int b = 0; b < LC.cap[sl]; ++b, e += LST) v = fma(e[2 * Q + p], e[c], v);
       } else {
-        slot = SLOT_W;
-        idx = jl;
+        for (int b0 = 0; b0 < LC.cap[sl]; b0 += 16) {
+          LT sum = LT(0);
+          for (int b = b0; b < b0 + 16 && b < LC.cap[sl]; ++b, e += LST) sum = fma(e[2 * Q + p], e[c], sum);
+          v += (double)sum;
+        }
       }
-    } else if (dxs == 0) {
-      slot = SLOT_N;
-      idx = 2 * il + (d == 2 ? 1 : 0);
-    } else if (dxs > 0) {
-      slot = SLOT_NE;
-      idx = (d == 1) ? 0 : 1;
-    } else {
-      slot = SLOT_NW;
-      idx = (d == 2) ? 0 : 1;
-    }
-    const int Jx = Ix + dxs, Jy = Iy + dys;
-    const double2 repJ = lv.rep[Jy * lv.Mx + Jx];
-    double* e = lists + (size_t)(LC.off[slot] + idx) * LSTRIDE12;
-    double sa[Q12], sb[Q12];
-    mode_proj12(ex, ey, node_x(lv, i, j) - repI.x, node_y(lv, j) - repI.y, fa, ld(delta, na), ld(delta_rf, na), sa);
-    mode_proj12(ex, ey, node_x(lv, ib, jb) - repJ.x, node_y(lv, jb) - repJ.y, fb, ld(delta, nbn), ld(delta_rf, nbn),
-                sb);
-#pragma unroll
-    for (int m = 0; m < Q12; ++m) {
-      e[m] = sa[m];
-      e[Q12 + m] = -sb[m];
-      e[2 * Q12 + m] = k * sa[m];
-      e[3 * Q12 + m] = -(k * sb[m]);
+      out[sl * SZ + p * SD + c] = v;
+      out[sl * SZ + c * SD + p] = v;
     }
   }
-
-  // deterministic block sums of the per-thread accumulators, RED_CHUNK at a time
-  double* red = lists + (size_t)LC.total * LSTRIDE12;  // RED_CHUNK x NT
-  double* tot = red + RED_CHUNK * NT;                   // NGEN CTA totals
-#pragma unroll
-  for (int c0 = 0; c0 < NGEN; c0 += RED_CHUNK) {
-#pragma unroll
-    for (int q = 0; q < RED_CHUNK; ++q)
-      if (c0 + q < NGEN) red[q * NT + tid] = (double)gen[c0 + q];
-    __syncthreads();
-    if (c0 + warp < NGEN) {
-      const double* q = red + warp * NT + lane;
-      double v = q[0];
-#pragma unroll
-      for (int ww = 1; ww < NW; ++ww) v += q[32 * ww];
-      v = warp_sum(v);
-      if (lane == 0) tot[c0 + warp] = v;
-    }
-    __syncthreads();
+  if (C > 1) cluster.sync();  // the parts are in rank 0's memory
+  if (rank > 0) return;
+  // SELF slot (upper-left Q x Q): the parts in order
+  for (int k = tid; k < SS::NACC; k += nt) {
+    double v = part[k];
+    for (int q = 1; q < SP; ++q) v += part[(size_t)q * SS::NACC + k];
+    part[k] = v;  // only this thread reads or writes column k
   }
-  // SELF slot (upper-left 12 x 12): the entries this pass sums
-  if (tid < Q12 * Q12) {
-    const int m = tid / Q12, l = tid % Q12;
+  __syncthreads();
+  for (int t = tid; t < Q * Q; t += nt) {
+    const int m = t / Q, l = t % Q;
     const int mm = m > l ? m : l, ll = m > l ? l : m;
-    if (mm >= MLO && mm < MHI) out[SLOT_SELF * SS12 + m * SD12 + l] = tot[gen12_idx(mm, ll, FULL)];
-  }
-  // interface slots: sums over each list in index order (symmetric: p <= c)
-  constexpr int NUP = SD12 * (SD12 + 1) / 2;
-  for (int q = tid; q < 5 * NUP; q += NT) {
-    const int slot = 1 + q / NUP;
-    int r = q % NUP, p = 0;
-    while (r >= SD12 - p) r -= SD12 - p, ++p;
-    const int c = p + r;
-    const bool dp = (p % Q12) >= 6, dc = (c % Q12) >= 6;
-    if (FULL ? (dp || dc) : (!dp && !dc)) continue;
-    const double* e = lists + (size_t)LC.off[slot] * LSTRIDE12;
-    double v = 0.0;
-    for (int b = 0; b < LC.cap[slot]; ++b, e += LSTRIDE12) v = fma(e[2 * Q12 + p], e[c], v);
-    out[slot * SS12 + p * SD12 + c] = v;
-    out[slot * SS12 + c * SD12 + p] = v;
+    if (mm < 6) continue;
+    double v = part[SS::NLIN + SS::NQUAD + mm * (mm + 1) / 2 - 21 + ll];
+    // constants s_2..s_5 of a regular bar of direction d: -L e_x^2, -L e_x e_y, -L e_y e_x, -L e_y^2
+    if (ll >= 2 && ll <= 5) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const double ex = (d == 0) ? 1.0 : (d == 1 ? 0.5 : -0.5), ey = (d == 0) ? 0.0 : SQ3_2;
+        const double c = (ll == 2) ? -lv.L * ex * ex : (ll == 5 ? -lv.L * ey * ey : -lv.L * ex * ey);
+        v = fma(c, part[NS * d + mm - 6], v);
+      }
+    } else if (ll >= 6) {
+      v += part[SS::NLIN + (mm - 6) * (mm - 5) / 2 + ll - 6];
+    }
+    out[SLOT_SELF * SZ + m * SD + l] = v;
   }
 }
 
-template <typename DT, bool FULL, typename AT>
-__global__ void __launch_bounds__(NT) k_coarse_slots12(LatView lv, const DT* __restrict__ delta,
-                                                       const DT* __restrict__ delta_rf, double* __restrict__ slots,
-                                                       const IterCtl* ctl) {
+template <typename DT, int Q, typename AT>
+__global__ void __launch_bounds__(32 * SP) k_slots_it(LatView lv, const DT* __restrict__ delta,
+                                                      const DT* __restrict__ delta_rf, double* __restrict__ slots,
+                                                      const IterCtl* ctl) {
   dep_wait();
-  slots12_body<DT, FULL, AT>(lv, delta, delta_rf, slots, ctl, blockIdx.x);
+  if (ctl && *(volatile const int*)&ctl->done) return;  // the same in every CTA of a cluster
+  const int C = (int)cg::this_cluster().num_blocks();
+  slots_it_body<DT, Q, AT>(lv, delta, delta_rf, slots, blockIdx.x / C);
 }
 
-// Batched (per-iteration pass, FULL = false): the sets of every problem.
+// Batched: the sets of every problem, a CTA each.
 template <typename DT, typename AT>
-__global__ void __launch_bounds__(NT) kb_coarse_slots(const BatchProb* __restrict__ P,
-                                                      const BatchItem* __restrict__ items) {
+__global__ void __launch_bounds__(32 * SP) kb_coarse_slots(const BatchProb* __restrict__ P,
+                                                           const BatchItem* __restrict__ items) {
   const BatchItem it = items[blockIdx.x];
   const BatchProb& q = P[it.prob];
-  slots_body<DT, false, AT>(q.lv, (const DT*)q.delta, q.slots_it, q.ctl, it.bx);
+  if (q.ctl && *(volatile const int*)&q.ctl->done) return;
+  slots_it_body<DT, NMODES, AT>(q.lv, (const DT*)q.delta, nullptr, q.slots_it, it.bx);
 }
 
 // Band (lower, column-major: band[c*(bw+1) + k] = A[c+k][c]) of K_aa from the
@@ -832,51 +800,46 @@ int coarse_bw(const LatView& lv) {
 size_t coarse_slots_smem(const LatView& lv) {
   const int w = lv.sx < lv.nx ? lv.sx : lv.nx;
   const int h = lv.sy < lv.ny ? lv.sy : lv.ny;
-  // interface lists, then the reduction buffer and the CTA totals
-  if (lv.q == NMODES_RF)
-    return ((size_t)list_caps(w, h).total * LSTRIDE12 + RED_CHUNK * NT + NGEN12_DELTA) * sizeof(double);
-  return ((size_t)list_caps(w, h).total * LSTRIDE + RED_CHUNK * NT + NREG + NGEN_FULL) * sizeof(double);
+  // lists of all modes and 2 K of sums: the limit of a set's size; more than the
+  // base's kernel or an update's takes
+  return ((size_t)list_caps(w, h).total * 4 * lv.q + RED_CHUNK * NT + (lv.q == NMODES_RF ? 57 : 60)) * sizeof(double);
+}
+
+size_t coarse_slots_it_smem(const LatView& lv, bool fp32) {
+  const ListCaps LC = list_caps(lv.sx < lv.nx ? lv.sx : lv.nx, lv.sy < lv.ny ? lv.sy : lv.ny);
+  if (lv.q == NMODES_RF) return slots_it_smem<NMODES_RF, double>(LC);
+  return fp32 ? slots_it_smem<NMODES, float>(LC) : slots_it_smem<NMODES, double>(LC);
 }
 
 cudaError_t launch_coarse_slots(cudaStream_t s, const LatView& lv, const void* delta, bool delta_fp32,
                                 bool full, double* slots, const IterCtl* ctl, const void* delta_rf) {
-  const size_t smem = coarse_slots_smem(lv);
-  auto go12 = [&](auto k, auto* d) {
-    using DT = std::remove_pointer_t<decltype(d)>;
-    return launch_dep(k, s, lv.M, NT, smem, 0, lv, (const DT*)delta, (const DT*)delta_rf, slots, ctl);
-  };
-  auto go = [&](auto k, auto* d) {
-    using DT = std::remove_pointer_t<decltype(d)>;
-    return launch_dep(k, s, lv.M, NT, smem, 0, lv, (const DT*)delta, slots, ctl);
-  };
+  const bool rf = lv.q == NMODES_RF;
   float2* const f2 = nullptr;
   double2* const d2 = nullptr;
-  if (lv.q == NMODES_RF) {
-    if (delta_fp32)
-      return full ? go12(k_coarse_slots12<float2, true, double>, f2) : go12(k_coarse_slots12<float2, false, float>, f2);
-    return full ? go12(k_coarse_slots12<double2, true, double>, d2) : go12(k_coarse_slots12<double2, false, double>, d2);
+  if (!full) {
+    const int cl = lv.M > 76 ? 1 : (lv.M > 38 ? 152 / lv.M : 4);
+    auto go = [&](auto k, auto* d) {
+      using DT = std::remove_pointer_t<decltype(d)>;
+      return launch_dep(k, s, lv.M * cl, 32 * ((SP + cl - 1) / cl), coarse_slots_it_smem(lv, delta_fp32),
+                        cl > 1 ? cl : 0, lv, (const DT*)delta, (const DT*)delta_rf, slots, ctl);
+    };
+    if (rf)
+      return delta_fp32 ? go(k_slots_it<float2, NMODES_RF, float>, f2) : go(k_slots_it<double2, NMODES_RF, double>, d2);
+    return delta_fp32 ? go(k_slots_it<float2, NMODES, float>, f2) : go(k_slots_it<double2, NMODES, double>, d2);
   }
-  if (delta_fp32) return full ? go(k_coarse_slots<float2, true, double>, f2) : go(k_coarse_slots<float2, false, float>, f2);
-  return full ? go(k_coarse_slots<double2, true, double>, d2) : go(k_coarse_slots<double2, false, double>, d2);
+  k_coarse_base<<<lv.M, NT, coarse_slots_smem(lv), s>>>(lv, slots);
+  return cudaGetLastError();
 }
 
 cudaError_t configure_coarse_assemble(int max_smem) {
-  cudaError_t e;
-  if ((e = set_max_dynamic_smem(k_coarse_slots12<float2, true, double>, max_smem)) != cudaSuccess) return e;
-  if ((e = set_max_dynamic_smem(k_coarse_slots12<float2, false, float>, max_smem)) != cudaSuccess) return e;
-  if ((e = set_max_dynamic_smem(k_coarse_slots12<double2, true, double>, max_smem)) != cudaSuccess) return e;
-  if ((e = set_max_dynamic_smem(k_coarse_slots12<double2, false, double>, max_smem)) != cudaSuccess) return e;
-  e = set_max_dynamic_smem(k_coarse_slots<float2, true, double>, max_smem);
-  if (e != cudaSuccess) return e;
-  e = set_max_dynamic_smem(k_coarse_slots<float2, false, float>, max_smem);
-  if (e != cudaSuccess) return e;
-  e = set_max_dynamic_smem(k_coarse_slots<double2, true, double>, max_smem);
-  if (e != cudaSuccess) return e;
-  e = set_max_dynamic_smem(k_coarse_slots<double2, false, double>, max_smem);
-  if (e != cudaSuccess) return e;
-  e = set_max_dynamic_smem(kb_coarse_slots<float2, float>, max_smem);
-  if (e != cudaSuccess) return e;
-  return set_max_dynamic_smem(kb_coarse_slots<double2, double>, max_smem);
+  cudaError_t e = set_max_dynamic_smem(k_coarse_base, max_smem);
+  if (e == cudaSuccess) e = set_max_dynamic_smem(k_slots_it<float2, NMODES_RF, float>, max_smem);
+  if (e == cudaSuccess) e = set_max_dynamic_smem(k_slots_it<double2, NMODES_RF, double>, max_smem);
+  if (e == cudaSuccess) e = set_max_dynamic_smem(k_slots_it<float2, NMODES, float>, max_smem);
+  if (e == cudaSuccess) e = set_max_dynamic_smem(k_slots_it<double2, NMODES, double>, max_smem);
+  if (e == cudaSuccess) e = set_max_dynamic_smem(kb_coarse_slots<float2, float>, max_smem);
+  if (e == cudaSuccess) e = set_max_dynamic_smem(kb_coarse_slots<double2, double>, max_smem);
+  return e;
 }
 
 static int grid_for(size_t total) {
@@ -892,8 +855,8 @@ int set_drops_blocks(int nsets) { return (nsets + 127) / 128; }
 cudaError_t launch_batch_slots(cudaStream_t s, bool fp32, size_t smem, const BatchProb* P, const BatchItem* it,
                                int n) {
   if (n <= 0) return cudaSuccess;
-  if (fp32) kb_coarse_slots<float2, float><<<n, NT, smem, s>>>(P, it);
-  else kb_coarse_slots<double2, double><<<n, NT, smem, s>>>(P, it);
+  if (fp32) kb_coarse_slots<float2, float><<<n, 32 * SP, smem, s>>>(P, it);
+  else kb_coarse_slots<double2, double><<<n, 32 * SP, smem, s>>>(P, it);
   return cudaGetLastError();
 }
 cudaError_t launch_batch_band(cudaStream_t s, const BatchProb* P, const BatchItem* it, int n) {

@@ -505,6 +505,7 @@ size_t coarse_factor_smem_bytes(int n, int bw, bool fp64);
 size_t coarse_solve_smem_bytes(int n, int bw, bool fp64);
 int coarse_dinv_size(int n);
 size_t coarse_slots_smem(const LatView& lv);
+size_t coarse_slots_it_smem(const LatView& lv, bool fp32);
 // one-time function attributes (max dynamic shared memory), per device
 cudaError_t configure_setup(int max_smem);
 cudaError_t configure_relax(int max_smem);
