@@ -312,7 +312,7 @@ struct RtShape {
   const RtNode* nodes;            // children first
   const unsigned short* front;    // per node: region nodes of S, then B
   const short* cmap;
-  const int* place;               // per tree node and front unknown: matrix column 32 + lane of its row's start
+  const int* place;               // per tree node, row and group of four columns: matrix column 32 + lane
 };
 struct RtView {
   const RtShape* shapes = nullptr;

@@ -32,14 +32,17 @@
 // only.
 //
 // Measured per launch, row substitution -> this (FP64, FP32; us): 16 sets of
-// 16 x 16 nodes 73 -> 34 and 61 -> 22; 70 of 32 x 32 (4 nodes overlap) 390 -> 271
-// and 195 -> 105; 72 of 64 x 64 726 -> 415 and 343 -> 157; 256 of 64 x 64 (1024^2
-// lattice) 1191 (its balanced schedule) -> 706 and 448 -> 261.  Bound by: FP64,
+// 16 x 16 nodes 73 -> 28 and 61 -> 22; 70 of 32 x 32 (4 nodes overlap) 390 -> 271
+// and 195 -> 105; 72 of 64 x 64 726 -> 394 and 343 -> 156; 256 of 64 x 64 (1024^2
+// lattice) 1191 (its balanced schedule) -> 710 and 448 -> 263.  Bound by: FP64,
 // the FP64 units of the SMs that hold sets (1203 K fused multiply-adds of a set
-// take 300 us at two per clock and SM, and 104 SMs hold two of the 256); FP32, the issue and shared-memory loads of the dot products
-// (1.23 GB of factor in 261 us: 4.7 TB/s); on few or small sets, the chain of
-// phases, 1 to 2 us each.  A deeper ring, bulk copies by one elected lane and
-// prefetches into the L2 measured the same.
+// take 300 us at two per clock and SM, and 104 SMs hold two of the 256); FP32, the
+// issue and shared-memory loads of the dot products (1.23 GB of factor in 263 us:
+// 4.7 TB/s); on few or small sets, the chain of phases, 1 to 2 us each.  A deeper
+// ring, bulk copies by one elected lane and prefetches into the L2 measured the
+// same.  Panels of phases too short for eight streams are split by columns: FP64
+// 16 x 16 nodes 34 -> 28, 32 x 32 110 -> 94, 24 x 20 87 -> 82 (whole panels left
+// the longest stream 1.5 to 2.5 times the mean).
 #include <algorithm>
 #include <array>
 #include <cmath>
@@ -214,7 +217,7 @@ __device__ __forceinline__ void rtree_body(const LatView& lv, const RtView& rt, 
   }
   for (int ph = 0; ph < nphase; ++ph) {
     const bool down = ph >= nup;
-    const int2 df = defer[ph];  // deferred outputs of the phase: first entry of dlist, count
+    const int2 df = defer[ph];  // deferred outputs of the phase: first entry of dlist; count, parts of each
     for (int q = 0; q < PER; ++q) {
       const int v = warp + q * NW;
       const int p0 = vp[ph * NV + v], p1 = vp[ph * NV + v + 1];
@@ -305,7 +308,13 @@ __device__ __forceinline__ void rtree_body(const LatView& lv, const RtView& rt, 
     }
     __syncthreads();
     if (df.y > 0) {
-      for (int k = tid; k < df.y; k += NT) z[dlist[df.x + k]] = xs[k];
+      const int cnt = df.y & 0xffff, parts = df.y >> 16;
+      for (int k = tid; k < cnt; k += NT) {
+        T s = xs[k];
+        for (int j = 1; j < parts; ++j) s += xs[j * cnt + k];
+        T* o = z + dlist[df.x + k];
+        *o = down ? s : *o + s;
+      }
       __syncthreads();
     }
   }
@@ -479,8 +488,9 @@ __global__ void __launch_bounds__(FTH) k_rtree_factor(LatView lv, RtView rt, dou
     const RtShape& sh = rt.shapes[rt.sid[I]];
     const Region R = relax_region(lv, I);
     const long long base = rt.off[I];
-    auto put = [&](int place, int k, double v) {  // column k of the row whose matrix starts at `place`
-      const long long rr = (place >> 5) + k;
+    auto put = [&](int row, int k, double v) {  // column k of a row; row: its first entry in place
+      const int place = sh.place[row + (k >> 2)];
+      const long long rr = (place >> 5) + (k & 3);
       if (f64) f64[base + rt_elem<double>(rr, place & 31)] = v;
       if (f32) f32[base + rt_elem<float>(rr, place & 31)] = (float)v;
     };
@@ -488,6 +498,7 @@ __global__ void __launch_bounds__(FTH) k_rtree_factor(LatView lv, RtView rt, dou
     for (int q = 0; q < sh.nnode; ++q) {
       const RtNode nd = sh.nodes[q];
       const int ns = 2 * nd.ns, nb = 2 * nd.nb, nf = ns + nb;
+      const int gu = (ns + 3) >> 2, gd = gu + ((nb + 3) >> 2);  // groups of an up row, of a down row
       const unsigned short* fr = sh.front + nd.f_off;  // region nodes of S, then B
       double* col = S + pk(ns - 1, ns - 1) + 1;        // pivot column, and A_SS's own diagonal
       double* dia = col + ns;
@@ -546,13 +557,13 @@ __global__ void __launch_bounds__(FTH) k_rtree_factor(LatView lv, RtView rt, dou
           for (int k = 0; k < j; ++k) acc = fma(-ar[k], S[pk(j, k)], acc);
           for (int k = j; k < ns; ++k) acc = fma(-ar[k], S[pk(k, j)], acc);
           G[(size_t)i * ns + j] = acc;
-          put(sh.place[nd.p_off + ns + i], j, -acc);
-          put(sh.place[nd.p_off + j], ((ns + 3) & ~3) + i, -acc);
+          put(nd.p_off + ns * gd + i * gu, j, -acc);
+          put(nd.p_off + j * gd, 4 * gu + i, -acc);
         }
       }
       for (int i = warp; i < ns; i += FTH / 32)
         for (int j = lane; j < ns; j += 32)
-          put(sh.place[nd.p_off + i], j, j <= i ? -S[pk(i, j)] : -S[pk(j, i)]);
+          put(nd.p_off + i * gd, j, j <= i ? -S[pk(i, j)] : -S[pk(j, i)]);
       __syncthreads();
       // the parent's update A_BB - G A_BS^T
       for (int i = warp; i < nb; i += FTH / 32) {
@@ -612,7 +623,7 @@ struct Panel {
   bool more = false, cont = false;  // its node's panels stay together; not the first of them
   int base[32][4] = {}, out[32] = {}, xs[32] = {};
   std::vector<int> in;  // none: the panel before's (of the same node)
-  std::vector<std::array<int, 3>> note;  // index into place, segment, lane
+  std::vector<std::array<int, 5>> note;  // row's first entry in place, segment, lane, its first group here, groups in all
 };
 
 }  // namespace
@@ -683,7 +694,7 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
     for (int s : v.S) P->front.push_back((unsigned short)s);
     for (int s : v.B) P->front.push_back((unsigned short)s);
     d.p_off = places;
-    places += 2 * (d.ns + d.nb);
+    places += 2 * d.ns * (ns4 + nb4) / 4 + 2 * d.nb * (ns4 / 4);
     d.u_off = (int)take(4LL * d.nb * d.nb);
     d.nchild = (int)v.child.size();
     for (int c = 0; c < d.nchild; ++c) {
@@ -719,6 +730,13 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
   };
   std::vector<Around> around(2 * (size_t)nn);
   std::vector<int> at(nnode, -1), open;  // start of a node's z_S in the open panel's inputs
+  auto groups = [&](int k, bool down) {  // of a row of node k
+    const int gu = (2 * (int)hn[k].S.size() + 3) / 4;
+    return down ? gu + (2 * (int)hn[k].B.size() + 3) / 4 : gu;
+  };
+  auto up_row = [&](int k, int b) {
+    return P->nodes[k].p_off + 2 * (int)hn[k].S.size() * groups(k, true) + b * groups(k, false);
+  };
   for (int hgt = 0; hgt < top; ++hgt) {
     std::vector<int> order;
     for (int k : byh[hgt])
@@ -778,7 +796,7 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
           p.base[l][q] = at[k];
           p.maxb[q] = std::max(p.maxb[q], at[k]);
           p.seg4[q] = std::max(p.seg4[q], ns4_of(k) / 4);
-          p.note.push_back({P->nodes[k].p_off + 2 * (int)hn[k].S.size() + rw.row[q], q, l});
+          p.note.push_back({up_row(k, rw.row[q]), q, l, 0, ns4_of(k) / 4});
         }
         break;
       }
@@ -834,7 +852,7 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
             p.xs[l] = (int)dl.size();
             dl.push_back(p.out[l]);
           }
-          p.note.push_back({P->nodes[k].p_off + s, 0, l});
+          p.note.push_back({P->nodes[k].p_off + s * groups(k, true), 0, l, 0, groups(k, true)});
         }
       }
     }
@@ -843,11 +861,13 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
   }
   P->nphase = (int)phases.size();
   // ---- deal the panels to the streams: longest first, to the least loaded
-  // stream of the phase ----
-  std::vector<std::array<std::vector<int>, NV>> deal(P->nphase);
-  for (int ph = 0; ph < P->nphase; ++ph) {
-    auto& ps = phases[ph];
-    auto rows_of = [&](const Panel& p) { return 4 * (p.seg4[0] + p.seg4[1] + p.seg4[2] + p.seg4[3]); };
+  // stream of the phase.  Phases with few panels for eight streams (the top of the
+  // tree, all of a small set's) have each panel's columns split in two or four
+  // parts, dealt apart, their sums added when the phase ends ----
+  using Deal = std::array<std::vector<int>, NV>;
+  constexpr int FIXED = 12, HELD = 10;  // a panel's and a deferred phase's fixed parts, in columns
+  auto rows_of = [](const Panel& p) { return 4 * (p.seg4[0] + p.seg4[1] + p.seg4[2] + p.seg4[3]); };
+  auto deal_out = [&](const std::vector<Panel>& ps, Deal* out) {  // the longest stream's load
     std::vector<std::vector<int>> units;  // panels that stay together
     for (int q = 0; q < (int)ps.size(); ++q) {
       if (!ps[q].cont) units.emplace_back();
@@ -867,11 +887,81 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
       for (int v = 1; v < NV; ++v)
         if (load[v] < load[best]) best = v;
       for (int q : u) {
-        load[best] += rows_of(ps[q]) + 8;  // a panel's fixed part
-        deal[ph][best].push_back(q);
-        vrows[best] += rows_of(ps[q]);
+        load[best] += rows_of(ps[q]) + FIXED;
+        (*out)[best].push_back(q);
       }
     }
+    return *std::max_element(load.begin(), load.end());
+  };
+  // part j of np of every panel; outs: the phase's outputs in the order of their places
+  auto split = [&](const std::vector<Panel>& ps, int np, std::vector<int>* outs) {
+    std::vector<Panel> r;
+    outs->clear();
+    const std::vector<int>* in = nullptr;
+    for (const Panel& p : ps) {
+      if (!p.cont) in = &p.in;
+      const int g = rows_of(p) / 4, first = (int)outs->size();
+      for (int l = 0; l < p.nlane; ++l) outs->push_back(p.out[l]);
+      for (int j = 0; j < np; ++j) {
+        const int ga = g * j / np, gb = g * (j + 1) / np;
+        Panel n;
+        n.nlane = p.nlane;
+        for (int l = 0; l < p.nlane; ++l) {
+          n.out[l] = p.out[l];
+          n.xs[l] = (j << 16) | (first + l);
+        }
+        int at = 0;
+        std::array<int, 4> seg{-1, -1, -1, -1}, skip{};
+        for (int q = 0; q < p.nseg; ++q) {
+          const int a = std::max(ga - at, 0), b = std::min(gb - at, p.seg4[q]);
+          at += p.seg4[q];
+          if (b <= a) continue;
+          seg[q] = n.nseg;
+          skip[q] = a;
+          n.seg4[n.nseg] = b - a;
+          n.maxb[n.nseg] = p.maxb[q] + 4 * a;
+          for (int l = 0; l < p.nlane; ++l) n.base[l][n.nseg] = p.base[l][q] + 4 * a;
+          ++n.nseg;
+        }
+        for (const auto& t : p.note)
+          if (seg[t[1]] >= 0) n.note.push_back({t[0], seg[t[1]], t[2], t[3] + skip[t[1]], t[4]});
+        if (n.nseg > 0) n.in = *in;
+        bool one = n.nseg == 1;  // one input range for all lanes: gather no more than that
+        for (int l = 1; l < p.nlane; ++l) one = one && n.base[l][0] == n.base[0][0];
+        if (one) {
+          const int b0 = n.base[0][0], e0 = std::min(b0 + 4 * n.seg4[0], (int)n.in.size());
+          n.in = std::vector<int>(n.in.begin() + b0, n.in.begin() + e0);
+          n.maxb[0] = 0;
+          for (int l = 0; l < p.nlane; ++l) n.base[l][0] = 0;
+        }
+        r.push_back(std::move(n));
+      }
+    }
+    const int cnt = (int)outs->size();
+    for (Panel& n : r)
+      for (int l = 0; l < n.nlane; ++l) n.xs[l] = (n.xs[l] >> 16) * cnt + (n.xs[l] & 0xffff);
+    return r;
+  };
+  std::vector<Deal> deal(P->nphase);
+  std::vector<int> parts(P->nphase, 1);
+  for (int ph = 0; ph < P->nphase; ++ph) {
+    int best = deal_out(phases[ph], &deal[ph]) + (dls[ph].empty() ? 0 : HELD);
+    const std::vector<Panel> whole = phases[ph];
+    for (int np = 2; np <= 4; np += 2) {
+      std::vector<int> outs;
+      std::vector<Panel> ps = split(whole, np, &outs);
+      if (np * (int)outs.size() > 256) continue;
+      Deal d;
+      const int cost = deal_out(ps, &d) + HELD;
+      if (100 * cost > 92 * best) continue;
+      best = cost;
+      phases[ph] = std::move(ps);
+      dls[ph] = std::move(outs);
+      deal[ph] = std::move(d);
+      parts[ph] = np;
+    }
+    for (int v = 0; v < NV; ++v)
+      for (int q : deal[ph][v]) vrows[v] += rows_of(phases[ph][q]);
   }
   P->vrow[0] = 0;
   for (int v = 0; v < NV; ++v) P->vrow[v + 1] = P->vrow[v] + (vrows[v] + 15) / 16 * 16;  // whole chunks
@@ -892,7 +982,9 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
           if (p.seg4[s] > 255) return false;
           packed |= p.seg4[s] << (8 * s);
         }
-        for (auto& nt : p.note) P->place[nt[0]] = start[nt[1]] * 32 + nt[2];
+        for (auto& nt : p.note)
+          for (int t = 0; t < p.seg4[nt[1]] && nt[3] + t < nt[4]; ++t)
+            P->place[nt[0] + nt[3] + t] = (start[nt[1]] + 4 * t) * 32 + nt[2];
         row[v] = r0;
         P->desc.push_back(packed);
         P->desc.push_back((int)p.in.size() | (p.nseg << 16));
@@ -915,9 +1007,10 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
       }
     }
     P->defer.push_back((int)P->dlist.size());
-    P->defer.push_back((int)dls[ph].size());
+    P->defer.push_back((int)dls[ph].size() | (parts[ph] << 16));
+    if (dls[ph].empty()) P->defer.back() = 0;
     for (int zi : dls[ph]) P->dlist.push_back((unsigned short)zi);
-    xsmax = std::max(xsmax, (int)dls[ph].size());
+    xsmax = std::max(xsmax, parts[ph] * (int)dls[ph].size());
   }
   P->vp.push_back((int)P->desc.size() / 2);
   P->npanel = (int)P->desc.size() / 2;
