@@ -635,7 +635,7 @@ size_t rt_list_bytes(const RtShapeHost& P) { return P.desc.size() * 4; }
 bool rt_shape_build(int W, int H, RtShapeHost* P) {
   *P = RtShapeHost();
   const int nn = W * H;
-  if (2 * nn + 4 > 0xffff) return false;
+  if (2 * nn + 4 > 0xffff) return false;  // and fewer than 2^15 tree nodes
   P->w = W, P->h = H, P->nn = nn;
   std::vector<HNode> hn;
   rt_cut(hn, W, H, 0, 0, W, H);
@@ -668,8 +668,8 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
   };
   auto give = [&](long long off, long long len) {
     if (len == 0) return;
-    size_t k = 0;
-    while (k < freed.size() && freed[k].off < off) ++k;
+    size_t k = std::lower_bound(freed.begin(), freed.end(), off,
+                                [](const Span& a, long long o) { return a.off < o; }) - freed.begin();
     freed.insert(freed.begin() + k, Span{off, len});
     if (k + 1 < freed.size() && freed[k].off + freed[k].len == freed[k + 1].off) {
       freed[k].len += freed[k + 1].len;
@@ -749,13 +749,15 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
         a.row[a.n++] = b;
       }
     // rows with the same nodes side by side, most segments first
-    std::sort(order.begin(), order.end(), [&](int x, int y) {
-      const Around &a = around[x], &b = around[y];
-      if (a.n != b.n) return a.n > b.n;
-      for (int q = 0; q < a.n; ++q)
-        if (a.node[q] != b.node[q]) return a.node[q] < b.node[q];
-      return x < y;
-    });
+    std::vector<std::pair<unsigned long long, int>> keyed(order.size());
+    for (size_t k = 0; k < order.size(); ++k) {
+      const Around& a = around[order[k]];
+      unsigned long long key = 4 - a.n;
+      for (int q = 0; q < 4; ++q) key = (key << 15) | (unsigned long long)(q < a.n ? a.node[q] : 0);
+      keyed[k] = {key, order[k]};
+    }
+    std::sort(keyed.begin(), keyed.end());
+    for (size_t k = 0; k < order.size(); ++k) order[k] = keyed[k].second;
     std::vector<Panel> ps;
     auto ns4_of = [&](int k) { return (2 * (int)hn[k].S.size() + 3) & ~3; };
     for (int zi : order) {
@@ -923,6 +925,7 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
           for (int l = 0; l < p.nlane; ++l) n.base[l][n.nseg] = p.base[l][q] + 4 * a;
           ++n.nseg;
         }
+        n.note.reserve(p.note.size());
         for (const auto& t : p.note)
           if (seg[t[1]] >= 0) n.note.push_back({t[0], seg[t[1]], t[2], t[3] + skip[t[1]], t[4]});
         if (n.nseg > 0) n.in = *in;
@@ -946,6 +949,9 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
   std::vector<int> parts(P->nphase, 1);
   for (int ph = 0; ph < P->nphase; ++ph) {
     int best = deal_out(phases[ph], &deal[ph]) + (dls[ph].empty() ? 0 : HELD);
+    int total = 0;
+    for (const Panel& p : phases[ph]) total += rows_of(p) + FIXED;
+    if (best * NV <= total + total / 10) continue;  // dealt evenly as they are
     const std::vector<Panel> whole = phases[ph];
     for (int np = 2; np <= 4; np += 2) {
       std::vector<int> outs;
@@ -960,9 +966,10 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
       deal[ph] = std::move(d);
       parts[ph] = np;
     }
+  }
+  for (int ph = 0; ph < P->nphase; ++ph)
     for (int v = 0; v < NV; ++v)
       for (int q : deal[ph][v]) vrows[v] += rows_of(phases[ph][q]);
-  }
   P->vrow[0] = 0;
   for (int v = 0; v < NV; ++v) P->vrow[v + 1] = P->vrow[v] + (vrows[v] + 15) / 16 * 16;  // whole chunks
   if ((long long)P->vrow[NV] * 32 > 0x3fffffffLL) return false;
@@ -990,20 +997,16 @@ bool rt_shape_build(int W, int H, RtShapeHost* P) {
         P->desc.push_back((int)p.in.size() | (p.nseg << 16));
         for (int t = 0; t < 4; ++t) P->stg = std::max(P->stg, p.maxb[t] + 4 * p.seg4[t]);
         P->stg = std::max(P->stg, ((int)p.in.size() + 31) / 32 * 32);
-        for (int l = 0; l < 32; ++l) {
-          unsigned short u[8] = {0, 0, 0, 0, 0xffff, 0, 0, 0};
-          if (l < p.nlane) {
-            for (int s = 0; s < 4; ++s) u[s] = (unsigned short)p.base[l][s];
-            u[4] = (unsigned short)p.out[l];
-            u[5] = (unsigned short)p.xs[l];
-          }
-          P->lane.insert(P->lane.end(), u, u + 8);
+        const size_t at = P->lane.size();
+        P->lane.resize(at + 512, (unsigned short)(2 * nn));
+        unsigned short* u = P->lane.data() + at;
+        for (int l = 0; l < 32; ++l, u += 8) {
+          for (int s = 0; s < 4; ++s) u[s] = (unsigned short)(l < p.nlane ? p.base[l][s] : 0);
+          u[4] = (unsigned short)(l < p.nlane ? p.out[l] : 0xffff);
+          u[5] = (unsigned short)(l < p.nlane ? p.xs[l] : 0);
+          u[6] = u[7] = 0;
         }
-        for (int l = 0; l < 32; ++l)
-          for (int t = 0; t < 8; ++t) {
-            const int e = l + 32 * t;
-            P->lane.push_back((unsigned short)(e < (int)p.in.size() ? p.in[e] : 2 * nn));
-          }
+        for (int e = 0; e < (int)p.in.size(); ++e) u[8 * (e & 31) + (e >> 5)] = (unsigned short)p.in[e];
       }
     }
     P->defer.push_back((int)P->dlist.size());
