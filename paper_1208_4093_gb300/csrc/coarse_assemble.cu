@@ -21,6 +21,7 @@
 
 #include <type_traits>
 
+#include "coarse_blocks.cuh"
 #include "hms_internal.cuh"
 #include "ptx.cuh"
 
@@ -681,7 +682,7 @@ __global__ void kb_coarse_diag(const BatchProb* __restrict__ Pb, const BatchItem
 
 // Modes that depend on earlier modes of the same set get a = 0.  Sets have
 // disjoint supports, so the columns of V can only be dependent within a set:
-// the Jacobi-scaled 9 x 9 diagonal block of every set is factored in FP64 in
+// the Jacobi-scaled 9 x 9 diagonal block of every set is eliminated in FP64 in
 // mode order, and a mode whose pivot is <= 1e-14 is dropped (the rule of the
 // full upper-level system, decided where FP64 resolves it).
 template <int Q = NMODES>
@@ -689,46 +690,17 @@ __device__ __forceinline__ void set_drops_body(int nsets, int bw, const double* 
                                                const double* __restrict__ scale, int* __restrict__ dropped,
                                                const IterCtl* ctl, int bx, int gx) {
   if (ctl && *(volatile const int*)&ctl->done) return;
-  const int I = bx * blockDim.x + threadIdx.x;
+  const int I = bx * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (I >= nsets) return;
-  constexpr int NMODES = Q;  // modes per set (shadows the 9 of the displacement-controlled form)
-  double A[NMODES][NMODES];
-  bool dr[NMODES];
+  const int row = lane < Q ? lane : Q - 1;
+  double A[Q];
 #pragma unroll
-  for (int m = 0; m < NMODES; ++m) {
-    dr[m] = dropped[NMODES * I + m] != 0;
-#pragma unroll
-    for (int l = 0; l < NMODES; ++l) {
-      const int lo = l < m ? l : m, hi = l < m ? m : l;
-      const int c = NMODES * I + lo;
-      A[m][l] = scale[NMODES * I + m] * band[(size_t)c * (bw + 1) + (hi - lo)] * scale[NMODES * I + l];
-    }
+  for (int l = 0; l < Q; ++l) {
+    const int lo = l < row ? l : row, hi = l < row ? row : l;
+    A[l] = scale[Q * I + row] * band[(size_t)(Q * I + lo) * (bw + 1) + (hi - lo)] * scale[Q * I + l];
   }
-#pragma unroll
-  for (int m = 0; m < NMODES; ++m) {
-    if (dr[m]) continue;
-    double piv = A[m][m];
-#pragma unroll
-    for (int k = 0; k < m; ++k) piv -= A[m][k] * A[m][k];
-    if (!(piv > 1e-14)) {
-      dr[m] = true;  // its column of L is zero
-#pragma unroll
-      for (int l = m + 1; l < NMODES; ++l) A[l][m] = 0.0;
-      continue;
-    }
-    const double d = sqrt(piv);
-    A[m][m] = d;
-#pragma unroll
-    for (int l = m + 1; l < NMODES; ++l) {
-      if (dr[l]) continue;
-      double v = A[l][m];
-#pragma unroll
-      for (int k = 0; k < m; ++k) v -= A[l][k] * A[m][k];
-      A[l][m] = v / d;
-    }
-  }
-#pragma unroll
-  for (int m = 0; m < NMODES; ++m) dropped[NMODES * I + m] = dr[m] ? 1 : 0;
+  const bool dr = drop_pivots<Q>(A, dropped[Q * I + row] != 0, lane);
+  if (lane < Q) dropped[Q * I + lane] = dr ? 1 : 0;
 }
 
 template <int Q>
@@ -850,7 +822,7 @@ static int grid_for(size_t total) {
 }
 
 int coarse_grid_for(size_t n) { return grid_for(n); }
-int set_drops_blocks(int nsets) { return (nsets + 127) / 128; }
+int set_drops_blocks(int nsets) { return (nsets + 3) / 4; }  // a warp per set
 
 cudaError_t launch_batch_slots(cudaStream_t s, bool fp32, size_t smem, const BatchProb* P, const BatchItem* it,
                                int n) {
@@ -908,9 +880,9 @@ cudaError_t launch_coarse_scale(cudaStream_t s, int n, int bw, bool fp64, const 
   if (e != cudaSuccess) return e;
   const int nsets = n / nm;
   if (nm == NMODES_RF)
-    k_coarse_set_drops<NMODES_RF><<<(nsets + 127) / 128, 128, 0, s>>>(nsets, bw, band, scale, dropped, ctl);
+    k_coarse_set_drops<NMODES_RF><<<set_drops_blocks(nsets), 128, 0, s>>>(nsets, bw, band, scale, dropped, ctl);
   else
-    k_coarse_set_drops<NMODES><<<(nsets + 127) / 128, 128, 0, s>>>(nsets, bw, band, scale, dropped, ctl);
+    k_coarse_set_drops<NMODES><<<set_drops_blocks(nsets), 128, 0, s>>>(nsets, bw, band, scale, dropped, ctl);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   double* sbandR = sband + (size_t)n * (bw + 1);

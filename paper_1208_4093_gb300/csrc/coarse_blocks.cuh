@@ -39,4 +39,33 @@ __device__ inline double blk_entry(const LatView& lv, const double* base, const 
   return slot_val(base, it, nm, I, SLOT_NW, nm + l, m);
 }
 
+// The modes of a set left out by the FP64 elimination of its scaled diagonal block in
+// mode order, by one warp: lane = row, A[l] = entry (row, l), dr = left out
+// beforehand.  A pivot <= 1e-14 leaves its mode out.  L D L^T with 1 / piv by two
+// Newton steps from FP32: an FP64 operation of one warp takes 64 clocks, a square
+// root or a division a dozen of them.
+template <int Q>
+__device__ __forceinline__ bool drop_pivots(double (&A)[Q], bool dr, int lane) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const unsigned dr0 = __ballot_sync(FULL, dr);
+#pragma unroll
+  for (int m = 0; m < Q; ++m) {
+    const double piv = __shfl_sync(FULL, A[m], m);
+    const bool out = (dr0 >> m) & 1u;  // its row and column count as zero
+    const bool low = !out && !(piv > 1e-14);
+    if (low && lane == m) dr = true;
+    // FP32, then 24 -> 48 -> 53 bits (piv <= 1 but for rounding, > 1e-14)
+    double ri = (double)__frcp_rn((float)piv);
+    ri = fma(ri, fma(-piv, ri, 1.0), ri);
+    ri = fma(ri, fma(-piv, ri, 1.0), ri);
+    const double t = out || low ? 0.0 : A[m] * ri;
+#pragma unroll
+    for (int l = m + 1; l < Q; ++l) {
+      const double al = __shfl_sync(FULL, A[m], l);
+      A[l] = out || low ? A[l] : fma(-t, al, A[l]);
+    }
+  }
+  return dr;
+}
+
 }  // namespace hms

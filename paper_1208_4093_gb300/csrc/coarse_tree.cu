@@ -127,24 +127,7 @@ __global__ void __launch_bounds__(DIAG_T<Q>) k_tree_diag(const TreeProb* __restr
     const int lo = l < row ? l : row, hi = l < row ? row : l;
     A[l] = sc * S[hi * Q + lo] * __shfl_sync(FULL, sc, l);
   }
-  const unsigned dr0 = __ballot_sync(FULL, dr);
-#pragma unroll
-  for (int m = 0; m < Q; ++m) {
-    const double piv = __shfl_sync(FULL, A[m], m);
-    const bool out = (dr0 >> m) & 1u;  // left out beforehand: its row and column are zero
-    const bool low = !out && !(piv > 1e-14);
-    if (low && lane == m) dr = true;
-    // 1 / piv: FP32, then 24 -> 48 -> 53 bits (piv <= 1 but for rounding, > 1e-14)
-    double ri = (double)__frcp_rn((float)piv);
-    ri = fma(ri, fma(-piv, ri, 1.0), ri);
-    ri = fma(ri, fma(-piv, ri, 1.0), ri);
-    const double t = out || low ? 0.0 : A[m] * ri;
-#pragma unroll
-    for (int l = m + 1; l < Q; ++l) {
-      const double al = __shfl_sync(FULL, A[m], l);
-      A[l] = out || low ? A[l] : fma(-t, al, A[l]);
-    }
-  }
+  dr = drop_pivots<Q>(A, dr, lane);
   if (lane < Q) {
     const int i = Q * I + lane;
     scale[i] = sc;
