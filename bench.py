@@ -976,10 +976,10 @@ def run_ours(args, rank, world, local_rank):
         rooflines[name] = roof
 
     # kernels launched per solve: graph batches of 16 iterations, each iteration
-    # 10 kernels (residual, relaxation, assembly, the scaled system's diagonal and
-    # rows, four levels of fronts, all solves), plus 1 load-norm kernel
+    # 9 kernels (residual, relaxation, assembly, the scaled system's diagonal and
+    # rows, three levels of fronts, all solves), plus 1 load-norm kernel
     batches = math.ceil((nit64 + 1) / 16)
-    per_iter = 10
+    per_iter = 9
     launches = args.steps * (batches * 16 * per_iter + 1)
 
     # ---- serving (continuous batching under the HBM budget), a bounded run ----
@@ -1027,7 +1027,7 @@ def run_ours(args, rank, world, local_rank):
         "dtype": "f64", "data": "synthetic",
         "config": {**workload_config(c),
                    "iterations": nit64, "setup_ms": setup64, "relax_launch": shape64,
-                   "l2": "working set > L2 (FP64 factors 2.2 GB streamed every iteration); no flush",
+                   "l2": "working set > L2 (FP64 factors 2.5 GB streamed every iteration); no flush",
                    "parallelism": "replicas" if world > 1 else "single GPU"},
         "err_vs_oracle_sampled": err_vs_oracle(u64),
         "err_vs_tight_solve": {"value": err_tight, "tight_tol": 1e-12, "tight_iterations": tight_its,

@@ -125,7 +125,7 @@ __device__ inline double bar_k(const LatView& lv, int i, int j, int d) {
 // which lets the next kernel's CTAs in as soon as an SM has room: with it in the
 // residual and the relaxation the FP64 kernels after them piled up on the SMs that
 // came free first (256^2 nodes FP64 373 -> 425 us per update, 327 without).  An
-// update of 10 kernels: 64^2 nodes FP64 167 -> 151 us, mixed 124 -> 112; 333 x 250
+// update of 7 to 12 kernels: 64^2 nodes FP64 167 -> 151 us, mixed 124 -> 112; 333 x 250
 // mixed 263 -> 256.  cl: CTAs per cluster, 0 = no cluster launch.
 template <typename... KA, typename... A>
 inline cudaError_t launch_dep(void (*k)(KA...), cudaStream_t s, dim3 grid, int threads, size_t smem, int cl,
