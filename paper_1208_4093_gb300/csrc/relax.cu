@@ -1,5 +1,7 @@
 // K2: displacement-controlled local relaxation of every set (Eqs. 11-13) and
-// the upper-level force P = V^T r (Eq. 7).
+// the upper-level force P = V^T r (Eq. 7), by substitution row by row of the
+// lattice: for set tiles of up to 64 nodes and with relax_balance = 1 or 2; else
+// relax_tree.cu.
 //
 // Eq. 12 fixes the outer displacements at their old values and solves
 //   k^Inner u^RD = p^Inner - k^Outer u^Outer-old.
