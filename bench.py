@@ -185,7 +185,7 @@ def traffic_for(kernel, workload, src):
     """DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum of one
     ncu capture) from the TRAFFIC lines of the committed kernel summary, or
     None if the kernel's source changed since the capture."""
-    p = os.path.join(ROOT, "profiles", "kernels_lattice1024_lognormal.md")
+    p = os.path.join(ROOT, "profiles", "launches_update_paths.md")
     try:
         for line in open(p):
             m = re.match(r"TRAFFIC (\S+) workload=(\S+) src_sha=(\S+) bytes_per_launch=(\d+)", line.strip())

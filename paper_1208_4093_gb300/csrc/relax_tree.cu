@@ -37,8 +37,8 @@
 // lattice) 1191 (its balanced schedule) -> 710 and 448 -> 263.  Bound by: FP64,
 // the FP64 units of the SMs that hold sets (1203 K fused multiply-adds of a set
 // take 300 us at two per clock and SM, and 104 SMs hold two of the 256); FP32, the
-// issue and shared-memory loads of the dot products (1.23 GB of factor in 263 us:
-// 4.7 TB/s); on few or small sets, the chain of phases, 1 to 2 us each.  A deeper
+// latency of the dot products' chains in eight warps per set (1.28 GB from HBM in
+// 254 us: 5.0 TB/s; issue slots 31 %, shared-memory pipe 27 % busy); on few or small sets, the chain of phases, 1 to 2 us each.  A deeper
 // ring, bulk copies by one elected lane and prefetches into the L2 measured the
 // same.  Panels of phases too short for eight streams are split by columns: FP64
 // 16 x 16 nodes 34 -> 28, 32 x 32 110 -> 94, 24 x 20 87 -> 82 (whole panels left
