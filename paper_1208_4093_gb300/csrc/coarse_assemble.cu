@@ -310,6 +310,7 @@ __device__ __forceinline__ void slots_it_body(const LatView& lv, const DT* __res
   cg::cluster_group cluster = cg::this_cluster();
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
+  if (C > 1) cluster_arrive();
   const int Ix = I % lv.Mx, Iy = I / lv.Mx;
   const int i0 = Ix * lv.sx, j0 = Iy * lv.sy;
   const int w = min(lv.sx, lv.nx - i0), h = min(lv.sy, lv.ny - j0);
@@ -375,6 +376,7 @@ __device__ __forceinline__ void slots_it_body(const LatView& lv, const DT* __res
   }
 
   // ---- bars inside the set ----
+  if (C > 1) cluster_wait();  // rank 0 runs: its shared memory may be written
   double* part0 = cluster.map_shared_rank(part, 0);
   const PT LA = (PT)lv.L, LyA = (PT)(lv.L * SQ3_2);
   const PT c0x = (PT)fma(lv.L, (double)i0, -repI.x), c0y = (PT)fma(lv.L * SQ3_2, (double)j0, -repI.y);

@@ -703,6 +703,7 @@ __global__ void __launch_bounds__(ST, 1) k_tree_solve(const TreeProb* __restrict
   const int gl = tid & 7;  // lane of a row group
   const int grp = tid >> 3;
   constexpr int ngrp = ST / 8;
+  cluster_arrive();
   const int nphase = pb.nphase;
   const int4 *gath = pb.gath, *rows = pb.rows, *phase = pb.phase;
   const float4* M4 = reinterpret_cast<const float4*>(pb.M);
@@ -710,6 +711,7 @@ __global__ void __launch_bounds__(ST, 1) k_tree_solve(const TreeProb* __restrict
   const int ub = (int)((long long)n * rank / cl), ue = (int)((long long)n * (rank + 1) / cl);
   for (int ph = tid; ph < nphase; ph += ST) span[ph] = phase[ph * cl + rank];
   dep_wait();
+  cluster_wait();  // the other CTAs run: their cred may be written
   if (use_ctl && tree_done(pb.ctl)) return;
   double bm = 0.0;
   for (int i = ub + tid; i < ue; i += ST) {

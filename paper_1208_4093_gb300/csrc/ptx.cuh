@@ -14,6 +14,12 @@ namespace hms {
 __device__ inline void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ inline void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Cluster barrier in two halves, for the start of a kernel: a CTA may touch another
+// one's shared memory only once that one runs, which is known when cluster_wait
+// returns.  Every thread of the cluster calls both, cluster_arrive as early as it
+// likes.  Orders no memory accesses.
+__device__ inline void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+__device__ inline void cluster_wait() { asm volatile("barrier.cluster.wait;" ::: "memory"); }
 
 __device__ inline uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
