@@ -232,12 +232,13 @@ __device__ inline void mode_proj12(double ex, double ey, double xi, double eta, 
 // direction) and k s_m s_l to the products', 50 FP64 operations per node for Q = 9
 // and 8 for its three bars' projections; bars at constrained DOFs take the general
 // form in a second pass of the warps that have any.  PT: arithmetic of the
-// projections, AT: of the products (the mixed form's: PT FP64 with the
-// force-controlled modes, else FP32).
+// projections, AT: of the products and of a lane's sums, ST: of the sums over lanes (the
+// mixed form's: PT and ST FP64 with the force-controlled modes, else FP32).
 //
 // Measured (us, before: one CTA of 256 threads per set, with Q = 12 every bar in
 // the general form): FP64, 16 sets of 16 x 16 nodes 28 -> 23, 256 of 64 x 64 250
-// -> 190; mixed 52 -> 43; Q = 12, 48 of 32 x 32 115 -> 65, mixed 98 -> 48.
+// -> 190; mixed 52 -> 43; Q = 12, 48 of 32 x 32 115 -> 65, mixed 98 -> 62 (48 with the
+// sums over lanes in FP32).
 constexpr int SP = 16;
 template <int Q>
 struct SlotSums {
@@ -267,16 +268,16 @@ constexpr SlotPairs<Q> slot_pairs() {
 __device__ const SlotPairs<NMODES> PAIRS9 = slot_pairs<NMODES>();
 __device__ const SlotPairs<NMODES_RF> PAIRS12 = slot_pairs<NMODES_RF>();
 
-// Sums over a warp of N values per lane, N adds and a few: value k's sum ends in
-// lane k (k < 32) and, of values 32.., in lane k - 32, and is stored at dst[k].
-template <int N, typename AT>
+// Sums over a warp of N values per lane, N adds and a few, in ST: value k's sum ends
+// in lane k (k < 32) and, of values 32.., in lane k - 32, and is stored at dst[k].
+template <typename ST, int N, typename AT>
 __device__ __forceinline__ void warp_sums(AT (&v)[N], double* dst) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int b = 0; b < N; b += 32) {
-    AT x[32];
+    ST x[32];
 #pragma unroll
-    for (int k = 0; k < 32; ++k) x[k] = b + k < N ? v[b + k < N ? b + k : 0] : AT(0);
+    for (int k = 0; k < 32; ++k) x[k] = b + k < N ? (ST)v[b + k < N ? b + k : 0] : ST(0);
     // halve the values, not the lanes: after step m a lane holds those whose number
     // agrees with its own in the bits seen
 #pragma unroll
@@ -285,7 +286,7 @@ __device__ __forceinline__ void warp_sums(AT (&v)[N], double* dst) {
 #pragma unroll
       for (int k = 0; k < m; ++k) {
         if (b + k >= N) continue;  // neither half holds a value
-        const AT give = up ? x[k] : x[k + m], keep = up ? x[k + m] : x[k];
+        const ST give = up ? x[k] : x[k + m], keep = up ? x[k + m] : x[k];
         x[k] = keep + __shfl_xor_sync(0xffffffffu, give, m);
       }
     }
@@ -305,6 +306,7 @@ __device__ __forceinline__ void slots_it_body(const LatView& lv, const DT* __res
   using SS = SlotSums<Q>;
   using LT = typename std::conditional<Q == NMODES_RF, double, AT>::type;  // of the lists
   using PT = LT;
+  using ST = LT;
   constexpr int NS = SS::NS, NF = NS / 3, LST = 4 * Q, SD = 2 * Q, SZ = SD * SD;
   extern __shared__ double lists[];
   cg::cluster_group cluster = cg::this_cluster();
@@ -432,7 +434,7 @@ __device__ __forceinline__ void slots_it_body(const LatView& lv, const DT* __res
       }
     }
     double* dst = part0 + (size_t)pt * SS::NACC;
-    warp_sums(acc, dst);
+    warp_sums<ST>(acc, dst);
     dst += SS::NLIN + SS::NQUAD;
     if (!__any_sync(0xffffffffu, special)) {
       for (int k = lane; k < SS::NGEN; k += 32) dst[k] = 0.0;
@@ -479,7 +481,7 @@ __device__ __forceinline__ void slots_it_body(const LatView& lv, const DT* __res
           }
       }
     }
-    warp_sums(gen, dst);
+    warp_sums<ST>(gen, dst);
   }
   __syncthreads();
 
