@@ -119,9 +119,10 @@ typedef struct {
   int32_t relax_threads;     /* compute threads per CTA of the relaxation (Eqs. 11-13; the row
                                 substitution has one more warp that issues its copies): 64,
                                 128 or 256, or
-                                0 = autotuned: the first problem of a set-tile shape and
-                                precision on a context times each size on its own factors
-                                and the context keeps the fastest for that shape.  Results
+                                0 = autotuned: the first problem of a set-tile shape,
+                                precision and load of the SMs (CTAs per SM, up to four) on
+                                a context times each size on its own factors and the
+                                context keeps the fastest for that shape.  Results
                                 are bitwise the same for every size */
   int32_t relax_copies;      /* shared memory per CTA of the FP64 relaxation: 1 or 2.  Row
                                 substitution: 1 or 2 bulk copies per factor matrix (2: the
@@ -224,6 +225,8 @@ double hms_problem_setup_ms(const hms_problem* pr);
  * or the autotuned choice). */
 int32_t hms_problem_relax_threads(const hms_problem* pr);
 int32_t hms_problem_relax_copies(const hms_problem* pr);
+/* Number of relaxation launch shapes that ctx has picked by timing and keeps. */
+int32_t hms_context_tuned_shapes(const hms_context* ctx);
 /* 1 if the relaxation of pr runs on the balanced schedule (relax_balance). */
 int32_t hms_problem_relax_balanced(const hms_problem* pr);
 /* No counterpart in the paper (a launch plan of the relaxation of Eqs. 12-13):

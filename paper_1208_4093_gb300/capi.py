@@ -104,6 +104,7 @@ def lib():
         "hms_residual_noalloc": (ctypes.c_int32, [_P, _P, _P, _P, _P]),
         "hms_solve_batch": (ctypes.c_int32, [_P, ctypes.c_int32, _P, _P, _P, _P, _P, ctypes.c_int32]),
         "hms_context_set_batch_mode": (ctypes.c_int32, [_P, ctypes.c_int32]),
+        "hms_context_tuned_shapes": (ctypes.c_int32, [_P]),
         "hms_problem_estimate_bytes": (ctypes.c_size_t, [_P, ctypes.POINTER(LatticeDesc), ctypes.POINTER(Options)]),
         "hms_server_create": (ctypes.c_int32, [_P, ctypes.c_uint64, ctypes.c_int32, ctypes.POINTER(_P)]),
         "hms_server_destroy": (None, [_P]),
@@ -137,7 +138,7 @@ def exported_symbols():
             "hms_problem_relax_threads", "hms_context_set_batch_mode", "hms_problem_relax_copies",
             "hms_reactions", "hms_problem_refine_cap_hits", "hms_problem_set_relax_wait_limit",
             "hms_measure_fp64_rate", "hms_relax_force", "hms_problem_relax_balanced", "hms_relax_schedule",
-            "hms_set_classes", "hms_nd_plan"]
+            "hms_set_classes", "hms_nd_plan", "hms_context_tuned_shapes"]
 
 
 # ---------------------------------------------------------------- marshalling
@@ -333,6 +334,10 @@ def hms_solve(ctx, pr, loads, u_out, u0=None, hist=None, iters=None, allow_no_co
 
 def hms_context_set_batch_mode(ctx, mode):
     _check(ctx, lib().hms_context_set_batch_mode(ctx, int(mode)))
+
+
+def hms_context_tuned_shapes(ctx) -> int:
+    return int(lib().hms_context_tuned_shapes(ctx))
 
 
 def hms_solve_batch(ctx, problems, loads, u_out, iters=None, allow_no_convergence=False):

@@ -25,8 +25,8 @@ struct hms_context {
   cudaStream_t stream = nullptr;
   std::vector<cudaStream_t> pool;  // streams of hms_solve_batch, created on first use
   std::string err;
-  // relaxation launch shape picked by timing, per (set width, set height,
-  // precision and copies, overlap, set count where the balanced schedule applies)
+  // relaxation launch shape picked by timing, per (set width, set height, precision,
+  // copies asked for and possible, overlap, set count: see autotune_relax)
   std::map<std::tuple<int, int, int, int, int>, int> relax_tuned;
   int batch_mode = HMS_BATCH_AUTO;
 };
@@ -1130,10 +1130,10 @@ static cudaError_t setup_relax_sched(hms_problem* pr, bool* ok) {
 }
 
 // Relaxation launch shape by timing: the first problem of a (set width, set
-// height, precision) on a context times one warm-up and three timed launches
-// of each CTA size, copies per matrix and, where it applies, the balanced
-// schedule on its own factors (r = 0; the kernel's time does not depend on the
-// values) and the context keeps the fastest for that shape.  All candidates
+// height, precision, load of the SMs) on a context times one warm-up and three
+// timed launches of each CTA size, copies per matrix and, where it applies, the
+// balanced schedule on its own factors (r = 0; the kernel's time does not depend
+// on the values) and the context keeps the fastest for that shape.  All candidates
 // give bitwise the same results, so the choice only changes the time.
 static cudaError_t autotune_relax(hms_problem* pr, int copies, bool try_sched) {
   hms_context* c = pr->ctx;
@@ -1143,12 +1143,18 @@ static cudaError_t autotune_relax(hms_problem* pr, int copies, bool try_sched) {
     cudaError_t e = setup_relax_sched(pr, &sched_ok);
     if (e != cudaSuccess) return e;
   }
-  // the relaxation region's overlap changes the factors' shapes and rules out
-  // two copies per matrix, so it is part of the key; so is the set count
-  // where the balanced schedule applies (its gain depends on it)
+  // The relaxation region's overlap changes the factors' shapes, so it is part of
+  // the key; so is whether two copies are possible (the last column of sets may be
+  // too narrow), and the set count where the balanced schedule applies (its gain
+  // depends on it).  By nested dissection the CTAs per SM are (up to four; both
+  // relaxations of twelve modes share a launch): a smaller ring lets two CTAs
+  // share an SM, which is worth nothing to sets that have one each.
+  const int max_nc = copies != 0 ? copies : (relax_chunks_possible(lv, fp32(pr)) ? 2 : 1);
+  const bool cut = pr->rtree && lv.q == NMODES_RF;
+  const int per_sm = std::min(((cut ? 2 : 1) * lv.M + c->nsm - 1) / c->nsm, 4);
   const auto key = std::make_tuple(std::min(lv.sx, lv.nx), std::min(lv.sy, lv.ny),
-                                   pr->precision * 10 + copies + (pr->rtree ? 100 : 0),
-                                   lv.ov, sched_ok ? lv.M : 0);
+                                   pr->precision * 10 + copies + (pr->rtree ? 100 : 0) + (max_nc == 2 ? 1000 : 0),
+                                   lv.ov, pr->rtree ? per_sm : (sched_ok ? lv.M : 0));
   const auto it = c->relax_tuned.find(key);
   if (it != c->relax_tuned.end()) {
     pr->relax_threads = (it->second % 10000) / 10;
@@ -1158,6 +1164,7 @@ static cudaError_t autotune_relax(hms_problem* pr, int copies, bool try_sched) {
   }
   cudaStream_t s = c->stream;
   cudaError_t e = cudaMemsetAsync(pr->r, 0, nnodes(pr) * sizeof(double2), s);
+  if (e == cudaSuccess && cut) e = cudaMemsetAsync(pr->rproj, 0, nnodes(pr) * sizeof(double2), s);
   if (e != cudaSuccess) return e;
   cudaEvent_t e0, e1;
   if ((e = cudaEventCreate(&e0)) != cudaSuccess) return e;
@@ -1169,7 +1176,6 @@ static cudaError_t autotune_relax(hms_problem* pr, int copies, bool try_sched) {
   // warm-up, so that clocks ramping up from idle do not favour later ones
   // (threads, copies); copies 0 = the balanced schedule (256 threads, one copy)
   std::vector<std::pair<int, int>> cand;
-  const int max_nc = copies != 0 ? copies : (relax_chunks_possible(lv, fp32(pr)) ? 2 : 1);
   for (int nc = copies != 0 ? copies : 1; nc <= max_nc; ++nc)
     for (int nt : {64, 128, 256}) cand.push_back({nt, nc});
   if (sched_ok) cand.push_back({256, 0});
@@ -1178,9 +1184,11 @@ static cudaError_t autotune_relax(hms_problem* pr, int copies, bool try_sched) {
     if (nc == 0)
       return launch_relax_sched(s, lv, pr->set_off, pr->f64, pr->f32, pr->r, pr->delta, pr->P, pr->yscratch,
                                 nullptr, pr->err, pr->sched_segs, pr->sched_cta, pr->sched_flags, pr->sched_grid);
-    if (pr->rtree)
-      return launch_rtree(s, lv, pr->rt, fp32(pr) ? (const void*)pr->f32 : pr->f64, fp32(pr), pr->r, pr->delta, pr->P,
-                          nullptr, pr->err, nt, nc, pr->rt_smem[nc], -1);
+    if (pr->rtree) {
+      pr->relax_threads = nt;
+      pr->relax_chunks = nc;
+      return launch_relax_tree(pr, s, nullptr, true, cut);
+    }
     return launch_relax(s, lv, pr->set_off, pr->f64, pr->f32, pr->r, pr->delta, pr->P, pr->yscratch, nullptr,
                         pr->err, nt, nc);
   };
@@ -1755,6 +1763,8 @@ static hms_status solve_batch_streams(hms_context* c, int32_t count, hms_problem
 static hms_status solve_batch_lockstep(hms_context* c, int32_t count, hms_problem* const* problems,
                                        const int32_t* nrhs, const double* const* loads, double* const* u_out,
                                        int32_t* iters, int32_t mem_kind);
+
+int32_t hms_context_tuned_shapes(const hms_context* c) { return c ? (int32_t)c->relax_tuned.size() : 0; }
 
 hms_status hms_context_set_batch_mode(hms_context* c, int32_t mode) {
   if (!c || mode < HMS_BATCH_AUTO || mode > HMS_BATCH_LOCKSTEP) return HMS_ERR_ARG;
