@@ -225,6 +225,23 @@ double hms_problem_setup_ms(const hms_problem* pr);
  * or the autotuned choice). */
 int32_t hms_problem_relax_threads(const hms_problem* pr);
 int32_t hms_problem_relax_copies(const hms_problem* pr);
+/* The factor of Eq. 8 that pr runs with (numbered as options.coarse_factor where
+ * that names it alone), and the CTAs of the cluster that its solves run on
+ * (solve_ctas, nullable: 1 to 16 for the tree of fronts, else 0).  0 for NULL. */
+#define HMS_COARSE_BAND_CLUSTER 1   /* FP32 band on a cluster of 4 SMs */
+#define HMS_COARSE_BAND_FP64 2
+#define HMS_COARSE_BAND_ROWS 3      /* FP32 band on one SM, solved in 16-row steps */
+#define HMS_COARSE_BAND 4           /* FP32 band on one SM */
+#define HMS_COARSE_BAND_TWO_SIDED 5
+#define HMS_COARSE_TREE 6           /* tree of fronts in shared memory */
+#define HMS_COARSE_PANELS 7         /* fronts panel by panel from device memory */
+int32_t hms_problem_coarse_form(const hms_problem* pr, int32_t* solve_ctas);
+/* Problems created on ctx from now on run the solves of the tree of fronts on
+ * clusters of at most `ctas` CTAs: 16 (the default), 8, 4, 2 or 1; in any case no
+ * more than the device can place.  0: they take no tree of fronts, but what they
+ * would take if its fronts did not fit.  The cluster's size does not change
+ * results. */
+hms_status hms_context_set_tree_cluster(hms_context* ctx, int32_t ctas);
 /* Number of relaxation launch shapes that ctx has picked by timing and keeps. */
 int32_t hms_context_tuned_shapes(const hms_context* ctx);
 /* 1 if the relaxation of pr runs on the balanced schedule (relax_balance). */

@@ -30,6 +30,8 @@ HMS_MIXED = 1
 HMS_BATCH_AUTO = 0
 HMS_BATCH_STREAMS = 1
 HMS_BATCH_LOCKSTEP = 2
+HMS_COARSE_BAND_CLUSTER, HMS_COARSE_BAND_FP64, HMS_COARSE_BAND_ROWS, HMS_COARSE_BAND = 1, 2, 3, 4
+HMS_COARSE_BAND_TWO_SIDED, HMS_COARSE_TREE, HMS_COARSE_PANELS = 5, 6, 7
 
 KERNEL_NAMES = ("update_residual", "relax", "coarse_assemble", "coarse_band", "coarse_factor",
                 "coarse_residual", "coarse_solve")
@@ -105,6 +107,8 @@ def lib():
         "hms_solve_batch": (ctypes.c_int32, [_P, ctypes.c_int32, _P, _P, _P, _P, _P, ctypes.c_int32]),
         "hms_context_set_batch_mode": (ctypes.c_int32, [_P, ctypes.c_int32]),
         "hms_context_tuned_shapes": (ctypes.c_int32, [_P]),
+        "hms_problem_coarse_form": (ctypes.c_int32, [_P, ctypes.POINTER(ctypes.c_int32)]),
+        "hms_context_set_tree_cluster": (ctypes.c_int32, [_P, ctypes.c_int32]),
         "hms_problem_estimate_bytes": (ctypes.c_size_t, [_P, ctypes.POINTER(LatticeDesc), ctypes.POINTER(Options)]),
         "hms_server_create": (ctypes.c_int32, [_P, ctypes.c_uint64, ctypes.c_int32, ctypes.POINTER(_P)]),
         "hms_server_destroy": (None, [_P]),
@@ -138,7 +142,8 @@ def exported_symbols():
             "hms_problem_relax_threads", "hms_context_set_batch_mode", "hms_problem_relax_copies",
             "hms_reactions", "hms_problem_refine_cap_hits", "hms_problem_set_relax_wait_limit",
             "hms_measure_fp64_rate", "hms_relax_force", "hms_problem_relax_balanced", "hms_relax_schedule",
-            "hms_set_classes", "hms_nd_plan", "hms_context_tuned_shapes"]
+            "hms_set_classes", "hms_nd_plan", "hms_context_tuned_shapes", "hms_problem_coarse_form",
+            "hms_context_set_tree_cluster"]
 
 
 # ---------------------------------------------------------------- marshalling
@@ -334,6 +339,17 @@ def hms_solve(ctx, pr, loads, u_out, u0=None, hist=None, iters=None, allow_no_co
 
 def hms_context_set_batch_mode(ctx, mode):
     _check(ctx, lib().hms_context_set_batch_mode(ctx, int(mode)))
+
+
+def hms_context_set_tree_cluster(ctx, ctas):
+    _check(ctx, lib().hms_context_set_tree_cluster(ctx, int(ctas)))
+
+
+def hms_problem_coarse_form(pr):
+    """(form, CTAs of the solves' cluster)"""
+    n = ctypes.c_int32(0)
+    form = int(lib().hms_problem_coarse_form(pr, ctypes.byref(n)))
+    return form, n.value
 
 
 def hms_context_tuned_shapes(ctx) -> int:

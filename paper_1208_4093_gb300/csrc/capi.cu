@@ -29,6 +29,7 @@ struct hms_context {
   // copies asked for and possible, overlap, set count: see autotune_relax)
   std::map<std::tuple<int, int, int, int, int>, int> relax_tuned;
   int batch_mode = HMS_BATCH_AUTO;
+  int tree_cluster = TREE_SCL;  // largest cluster of the solves by the tree of fronts (0: no tree)
 };
 
 // Buffers that stay read-only after setup (lattice description, set
@@ -658,17 +659,17 @@ RtSetup rt_setup(const RtPlanHost& P, int M, int nsm) {
 // memory of one cluster each (coarse_tree.cu) where they fit, else panel by
 // panel from device memory (coarse_nd.cu), if every front fits the factor
 // kernel's shared memory.
-bool choose_tree(hms_problem* pr, int maxsm) {
+bool choose_tree(hms_problem* pr, int maxsm, int max_cl) {
   pr->coarse_fp64 = false;
   pr->two_sided = false;
   pr->cluster_factor = false;
   pr->big_stages = 0;
   pr->nd = false;
-  pr->tree = tree_plan_build(pr->lv, maxsm, &pr->tph);
+  pr->tree = tree_plan_build(pr->lv, maxsm, max_cl, &pr->tph);
   return pr->tree;
 }
-bool choose_nd(hms_problem* pr, int maxsm) {
-  if (choose_tree(pr, maxsm)) return true;
+bool choose_nd(hms_problem* pr, int maxsm, int max_cl) {
+  if (choose_tree(pr, maxsm, max_cl)) return true;
   if (!nd_plan_build(pr->lv, &pr->ndp) || !nd_plan_smem(&pr->ndp, maxsm)) return false;
   pr->nd = true;
   return true;
@@ -680,13 +681,13 @@ bool choose_nd(hms_problem* pr, int maxsm) {
 // and solves of an update took 105 us against 183 for the one-SM band on 4 x 4
 // sets (FP64 form), 172 against 336 for the two-sided band on 8 x 8, 271 against
 // 863 on 16 x 16; then a band factor, then the panel-by-panel fronts.
-bool choose_coarse(hms_problem* pr, const hms_options* o, int maxsm) {
+bool choose_coarse(hms_problem* pr, const hms_options* o, int maxsm, int max_cl) {
   pr->nd = pr->tree = false;
-  if (o->coarse_factor == 6) return choose_nd(pr, maxsm);
+  if (o->coarse_factor == 6) return choose_nd(pr, maxsm, max_cl);
   const bool band = choose_band(pr, o, maxsm);
   if (o->coarse_factor != 0 || (band && pr->coarse_fp64)) return band;
-  if (choose_tree(pr, maxsm)) return true;
-  return choose_band(pr, o, maxsm) || choose_nd(pr, maxsm);
+  if (choose_tree(pr, maxsm, max_cl)) return true;
+  return choose_band(pr, o, maxsm) || choose_nd(pr, maxsm, max_cl);
 }
 
 }  // namespace
@@ -1296,7 +1297,7 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
     delete pr;
     return fail(c, HMS_ERR_ARG, "set tile too large for the relaxation kernel's shared memory");
   }
-  if (!choose_coarse(pr, o, maxsm)) {
+  if (!choose_coarse(pr, o, maxsm, c->tree_cluster)) {
     delete pr;
     return fail(c, HMS_ERR_ARG, "set grid too wide for the upper-level factorisations");
   }
@@ -1763,6 +1764,23 @@ static hms_status solve_batch_streams(hms_context* c, int32_t count, hms_problem
 static hms_status solve_batch_lockstep(hms_context* c, int32_t count, hms_problem* const* problems,
                                        const int32_t* nrhs, const double* const* loads, double* const* u_out,
                                        int32_t* iters, int32_t mem_kind);
+
+hms_status hms_context_set_tree_cluster(hms_context* c, int32_t ctas) {
+  if (!c || ctas < 0 || ctas > TREE_SCL || (ctas & (ctas - 1)) != 0) return HMS_ERR_ARG;
+  c->tree_cluster = ctas;
+  return HMS_OK;
+}
+
+int32_t hms_problem_coarse_form(const hms_problem* pr, int32_t* solve_ctas) {
+  if (!pr) return 0;
+  if (solve_ctas) *solve_ctas = pr->tree ? pr->tph.scl : 0;
+  if (pr->tree) return HMS_COARSE_TREE;
+  if (pr->nd) return HMS_COARSE_PANELS;
+  if (pr->coarse_fp64) return HMS_COARSE_BAND_FP64;
+  if (pr->two_sided) return HMS_COARSE_BAND_TWO_SIDED;
+  if (pr->cluster_factor) return HMS_COARSE_BAND_CLUSTER;
+  return pr->big_stages > 0 ? HMS_COARSE_BAND : HMS_COARSE_BAND_ROWS;
+}
 
 int32_t hms_context_tuned_shapes(const hms_context* c) { return c ? (int32_t)c->relax_tuned.size() : 0; }
 
@@ -2590,6 +2608,7 @@ bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options
         o->relax_overlap != 0)
       return false;
   }
+  if (cudaSetDevice(c->device) != cudaSuccess) return false;
   hms_problem pr;
   LatView& lv = pr.lv;
   lv.nx = d->nx;
@@ -2606,7 +2625,7 @@ bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options
   pr.bw = coarse_bw(lv);
   int maxsm = 0;
   cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
-  if (relax_smem_bytes(lv, fp32(&pr)) + 2048 > (size_t)maxsm || !choose_coarse(&pr, o, maxsm) ||
+  if (relax_smem_bytes(lv, fp32(&pr)) + 2048 > (size_t)maxsm || !choose_coarse(&pr, o, maxsm, c->tree_cluster) ||
       coarse_slots_smem(lv) > (size_t)maxsm)
     return false;
   const size_t nn = (size_t)lv.nx * lv.ny, M = (size_t)lv.M, n_c = (size_t)pr.n_c;

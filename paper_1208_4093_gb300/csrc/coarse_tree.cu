@@ -925,8 +925,8 @@ namespace {
 // (35 x 29 sets: 637, 652, 710, 725).
 constexpr int TREE_LEAF = 4, TREE_ROOT = 256;
 constexpr int TREE_FILL = 148;  // CTAs a level is spread over, if its fronts allow (152 SMs)
-constexpr int TREE_SCL = 16;    // CTAs of a solve, one per TREE_SROWS unknowns at most
-constexpr int TREE_SROWS = 16;
+constexpr int TREE_SROWS = 16;  // unknowns of a CTA of a solve, at least
+constexpr int TREE_PORTABLE = 8;  // a cluster size that every part can place
 }  // namespace
 
 // bytes of shared memory of the largest CTA of a front of T block rows
@@ -955,8 +955,32 @@ TreeLaunch tree_level_launch(int n, int T, int max_smem) {
   return L;
 }
 
-bool tree_plan_build(const LatView& lv, int max_smem, TreePlanHost* P) {
+// Whether the device can place a cluster of scl CTAs of the solves: above the
+// portable size that depends on the part (its SMs per processing cluster).
+static bool tree_solve_fits(int q, int scl, size_t smem) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)scl);
+  cfg.blockDim = dim3(ST);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)scl;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  const cudaError_t e = q == NMODES_RF ? cudaOccupancyMaxActiveClusters(&n, k_tree_solve<NMODES_RF>, &cfg)
+                                       : cudaOccupancyMaxActiveClusters(&n, k_tree_solve<NMODES>, &cfg);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return n >= 1;
+}
+
+bool tree_plan_build(const LatView& lv, int max_smem, int max_cl, TreePlanHost* P) {
   *P = TreePlanHost();
+  if (max_cl < 1) return false;
   const int nm = lv.q, n = nm * lv.M;
   if (n > (1 << 20) || std::max(lv.Mx, lv.My) > 8000) return false;
   const size_t cap = (size_t)max_smem - 2048;
@@ -1041,7 +1065,7 @@ bool tree_plan_build(const LatView& lv, int max_smem, TreePlanHost* P) {
   }
   P->level_begin[H + 1] = (int)P->items.size();
   // ---- solve schedule ----
-  int scl = TREE_SCL;
+  int scl = max_cl;
   while (scl > 1 && n < TREE_SROWS * scl) scl /= 2;
   P->scl = scl;
   P->nphase = 0;
@@ -1122,8 +1146,9 @@ bool tree_plan_build(const LatView& lv, int max_smem, TreePlanHost* P) {
       ++P->nphase;
     }
   P->solve_smem = (size_t)smax * sizeof(float);
-  if (P->nphase > 64) return false;
-  return P->solve_smem + 4096 <= (size_t)max_smem;
+  if (P->nphase > TREE_MAXPH || P->solve_smem + 4096 > (size_t)max_smem) return false;
+  if (scl <= TREE_PORTABLE || tree_solve_fits(nm, scl, P->solve_smem)) return true;
+  return tree_plan_build(lv, max_smem, scl / 2, P);
 }
 
 size_t tree_arow_elems(const LatView& lv) { return (size_t)lv.q * lv.M * 9 * lv.q; }

@@ -625,8 +625,10 @@ struct TreePlanHost {
   int n = 0, nm = 9, nlev = 0, scl = 1, nphase = 0, v_rhs = 0, v_x = 0;
   size_t m_elems = 0, u_elems = 0, v_elems = 0, x_elems = 0, solve_smem = 0;
 };
-// The plan of a set grid; false if a front does not fit (coarse_nd.cu takes it).
-bool tree_plan_build(const LatView& lv, int max_smem, TreePlanHost* P);
+constexpr int TREE_SCL = 16;  // CTAs of a solve's cluster, at most
+// The plan of a set grid, its solves on a cluster of at most max_cl CTAs (a power of
+// two); false if a front does not fit (coarse_nd.cu takes it) or max_cl is 0.
+bool tree_plan_build(const LatView& lv, int max_smem, int max_cl, TreePlanHost* P);
 size_t tree_arow_elems(const LatView& lv);
 cudaError_t configure_coarse_tree(int max_smem);
 TreeLaunch tree_level_launch(int n, int T, int max_smem);
