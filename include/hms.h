@@ -246,6 +246,12 @@ hms_status hms_context_set_tree_cluster(hms_context* ctx, int32_t ctas);
 int32_t hms_context_tuned_shapes(const hms_context* ctx);
 /* 1 if the relaxation of pr runs on the balanced schedule (relax_balance). */
 int32_t hms_problem_relax_balanced(const hms_problem* pr);
+/* The relaxation that pr runs with; -1 for NULL. */
+#define HMS_RELAX_DISSECTED 0       /* nested dissection of every set */
+#define HMS_RELAX_ROWS 1            /* row substitution, one CTA per set */
+#define HMS_RELAX_BALANCED 2        /* row substitution, balanced */
+#define HMS_RELAX_CLASS_BATCHES 3   /* class factors, many right-hand sides per CTA */
+int32_t hms_problem_relax_form(const hms_problem* pr);
 /* No counterpart in the paper (a launch plan of the relaxation of Eqs. 12-13):
  * the balanced relaxation schedule (relax_balance) of a lattice's sets over
  * `ctas` persistent CTAs (one per SM), computed on the host; no device is

@@ -31,6 +31,7 @@ HMS_BATCH_AUTO = 0
 HMS_BATCH_STREAMS = 1
 HMS_BATCH_LOCKSTEP = 2
 HMS_COARSE_BAND_CLUSTER, HMS_COARSE_BAND_FP64, HMS_COARSE_BAND_ROWS, HMS_COARSE_BAND = 1, 2, 3, 4
+HMS_RELAX_DISSECTED, HMS_RELAX_ROWS, HMS_RELAX_BALANCED, HMS_RELAX_CLASS_BATCHES = 0, 1, 2, 3
 HMS_COARSE_BAND_TWO_SIDED, HMS_COARSE_TREE, HMS_COARSE_PANELS = 5, 6, 7
 
 KERNEL_NAMES = ("update_residual", "relax", "coarse_assemble", "coarse_band", "coarse_factor",
@@ -107,6 +108,7 @@ def lib():
         "hms_solve_batch": (ctypes.c_int32, [_P, ctypes.c_int32, _P, _P, _P, _P, _P, ctypes.c_int32]),
         "hms_context_set_batch_mode": (ctypes.c_int32, [_P, ctypes.c_int32]),
         "hms_context_tuned_shapes": (ctypes.c_int32, [_P]),
+        "hms_problem_relax_form": (ctypes.c_int32, [_P]),
         "hms_problem_coarse_form": (ctypes.c_int32, [_P, ctypes.POINTER(ctypes.c_int32)]),
         "hms_context_set_tree_cluster": (ctypes.c_int32, [_P, ctypes.c_int32]),
         "hms_problem_estimate_bytes": (ctypes.c_size_t, [_P, ctypes.POINTER(LatticeDesc), ctypes.POINTER(Options)]),
@@ -143,7 +145,7 @@ def exported_symbols():
             "hms_reactions", "hms_problem_refine_cap_hits", "hms_problem_set_relax_wait_limit",
             "hms_measure_fp64_rate", "hms_relax_force", "hms_problem_relax_balanced", "hms_relax_schedule",
             "hms_set_classes", "hms_nd_plan", "hms_context_tuned_shapes", "hms_problem_coarse_form",
-            "hms_context_set_tree_cluster"]
+            "hms_context_set_tree_cluster", "hms_problem_relax_form"]
 
 
 # ---------------------------------------------------------------- marshalling
@@ -272,6 +274,10 @@ def hms_problem_relax_threads(pr) -> int:
 
 def hms_problem_relax_copies(pr) -> int:
     return int(lib().hms_problem_relax_copies(pr))
+
+
+def hms_problem_relax_form(pr) -> int:
+    return int(lib().hms_problem_relax_form(pr))
 
 
 def hms_problem_relax_balanced(pr) -> int:

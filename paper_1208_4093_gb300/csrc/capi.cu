@@ -1782,6 +1782,13 @@ int32_t hms_problem_coarse_form(const hms_problem* pr, int32_t* solve_ctas) {
   return pr->big_stages > 0 ? HMS_COARSE_BAND : HMS_COARSE_BAND_ROWS;
 }
 
+int32_t hms_problem_relax_form(const hms_problem* pr) {
+  if (!pr) return -1;
+  if (pr->cls) return HMS_RELAX_CLASS_BATCHES;
+  if (pr->rtree) return HMS_RELAX_DISSECTED;
+  return pr->relax_sched ? HMS_RELAX_BALANCED : HMS_RELAX_ROWS;
+}
+
 int32_t hms_context_tuned_shapes(const hms_context* c) { return c ? (int32_t)c->relax_tuned.size() : 0; }
 
 hms_status hms_context_set_batch_mode(hms_context* c, int32_t mode) {
