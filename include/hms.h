@@ -172,8 +172,9 @@ typedef struct {
   int32_t relax_balance;     /* schedule of the relaxation with per-set factors:
                                 0 = one CTA per set (sets in waves of the SM count), its
                                 nodes ordered by nested dissection: for set tiles of more
-                                than 64 nodes, unless its padded factors take 4 GB more
-                                than those of the row substitution; else, with
+                                than 64 nodes, unless its padded factors take more
+                                memory than those of the row substitution and that is
+                                more than 4 GB or more than is free; else, with
                                 relax_threads = 0, the faster of 1 and 2 by timing where
                                 both apply, else 1;
                                 1 = substitution row by row of the lattice, one CTA per
@@ -485,7 +486,8 @@ hms_status hms_residual_noalloc(hms_problem* pr, const double* p, const double* 
 /* Device bytes hms_problem_create would allocate for (d, o), counted
  * allocation by allocation as the library makes them, including the scratch
  * held while the set factors are computed; 0 if the problem would be
- * rejected (bad arguments, set tile or set grid too large). */
+ * rejected (bad arguments, set tile or set grid too large).  Where the memory
+ * that is free decides the relaxation's form (relax_balance = 0), that of now. */
 size_t hms_problem_estimate_bytes(hms_context* c, const hms_lattice_desc* d, const hms_options* o);
 
 /* A request server on one context: requests (lattice, options, nrhs load
@@ -509,7 +511,8 @@ void hms_server_destroy(hms_server* s);
 /* Queue a request; d, its ea / fixed arrays (host) and the nrhs load vectors
  * loads [nrhs][2*nx*ny] (host) are copied.  *id receives its id.  A request
  * whose problem would be rejected gives HMS_ERR_ARG, one larger than the
- * whole budget HMS_ERR_OOM. */
+ * whole budget HMS_ERR_OOM; with relax_balance = 0, one that is so only with
+ * the dissected sets' factors runs the row substitution. */
 hms_status hms_server_submit(hms_server* s, const hms_lattice_desc* d, const hms_options* o,
                              int32_t nrhs, const double* loads, int64_t* id);
 /* One scheduling pass, asynchronous: admit what fits; for every instance

@@ -567,6 +567,7 @@ struct RtPlanHost {
   std::vector<int> sid;
   std::vector<long long> off;   // per set; sets of one class share a factor
   long long elems = 0;          // of all factors
+  long long more = 0;           // bytes beyond the row substitution's factors (of one kind)
   long long scratch = 0;        // doubles per CTA of the factorisation
   int smax = 0;
   size_t smem[3] = {0, 0, 0};   // of the relaxation, by copies per matrix
@@ -577,9 +578,10 @@ struct RtPlanHost {
 // 8 x 8 nodes take the row substitution (30 dependent steps of 16 unknowns, in a
 // few KB): at 9 x 8 nodes nested dissection takes 24 us for 41 (FP64, 18 x 15
 // sets).  Padding to 32 lanes makes small tiles' factors larger than the
-// substitution's (9 x 8 nodes: 8 K entries for 6 K; 64 x 64: 1.2 M for 2.1 M);
+// substitution's (9 x 8 nodes: 9 K entries for 6 K; 64 x 64: 1.2 M for 2.1 M);
 // where that would cost more than RT_MORE_BYTES in all, a lattice of millions of
-// nodes, the smaller form stays, so that what fits the device still does.
+// nodes, or more than there is (rt_has_room), the smaller form stays, so that what
+// fits the device still does.
 constexpr long long RT_MORE_BYTES = 4LL << 30;
 // With class factors (cph) a class's sets read one factor, mostly from the L2; in
 // FP32 up to RT_CLASS_SETS sets per SM, beyond which relax_class.cu's batches of
@@ -634,7 +636,8 @@ bool rt_plan(const LatView& lv, const hms_options* o, bool f32, int maxsm, int n
     P->off[I] = at[cls[I]];
   }
   P->off[lv.M] = P->elems;
-  return (P->elems - rows) * (f32 ? 4 : 8) <= RT_MORE_BYTES;
+  P->more = (P->elems - rows) * (f32 ? 4 : 8);
+  return P->more <= RT_MORE_BYTES;
 }
 
 // CTAs of the sets' factorisation by nested dissection, those of them that work
@@ -1219,8 +1222,34 @@ static cudaError_t autotune_relax(hms_problem* pr, int copies, bool try_sched) {
   return cudaSuccess;
 }
 
-hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const hms_options* o,
-                              hms_problem** out) {
+namespace {
+bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options* o, bool rows, size_t* shared,
+                    size_t* inst, size_t* scratch, long long* more = nullptr);
+
+size_t free_bytes() {
+  size_t f = 0, t = 0;
+  if (cudaMemGetInfo(&f, &t) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return f;
+}
+
+// Whether a problem whose dissected factors take more memory than the row
+// substitution's fits into `room` bytes with them, RT_SLACK left for what the
+// estimate does not count (the CUDA graph, allocation granularity).  A few KB per
+// node beside the factors are room enough without a closer look.
+constexpr size_t RT_SLACK = (size_t)256 << 20;
+bool rt_has_room(hms_context* c, const hms_lattice_desc* d, const hms_options* o, const RtPlanHost& P, size_t room) {
+  if (RT_SLACK + 32 * (size_t)P.elems + 4096 * (size_t)d->nx * d->ny <= room) return true;
+  size_t sh = 0, in = 0, sc = 0;
+  return estimate_parts(c, d, o, false, &sh, &in, &sc) && sh + in + sc + RT_SLACK <= room;
+}
+}  // namespace
+
+// rows: the relaxation without nested dissection.
+static hms_status problem_create(hms_context* c, const hms_lattice_desc* d, const hms_options* o, bool rows,
+                                 hms_problem** out) {
   if (!c || !d || !o || !out) return HMS_ERR_ARG;
   *out = nullptr;
   if (d->nx < 2 || d->ny < 2) return fail(c, HMS_ERR_ARG, "nx, ny must be >= 2");
@@ -1364,7 +1393,8 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
       return fail(c, HMS_ERR_ARG, "set tile too large for the class-factor relaxation's shared memory");
     }
   }
-  pr->rtree = rt_plan(lv, o, fp32(pr), maxsm, c->nsm, o->class_factors ? &cph : nullptr, &rtp);
+  pr->rtree = !rows && rt_plan(lv, o, fp32(pr), maxsm, c->nsm, o->class_factors ? &cph : nullptr, &rtp) &&
+              (rtp.more <= 0 || rt_has_room(c, d, o, rtp, free_bytes() + pr->bytes));
   RtSetup rtsu;
   double* rtwork = nullptr;
   {
@@ -1630,6 +1660,10 @@ hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const h
 #undef CKP
   *out = pr;
   return HMS_OK;
+}
+
+hms_status hms_problem_create(hms_context* c, const hms_lattice_desc* d, const hms_options* o, hms_problem** out) {
+  return problem_create(c, d, o, false, out);
 }
 
 hms_status hms_solve(hms_problem* pr, int32_t nrhs, const double* loads, const double* u0, double* u_out,
@@ -2594,10 +2628,11 @@ hms_status hms_residual_noalloc(hms_problem* pr, const double* p, const double* 
 namespace {
 // Device bytes of a problem for (d, o), following hms_problem_create's
 // allocations one by one: the shared setup buffers, one instance's buffers
-// and the scratch held while the set factors are computed.  False if the
-// problem would be rejected.
-bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options* o, size_t* shared, size_t* inst,
-                    size_t* scratch) {
+// and the scratch held while the set factors are computed (rows: without nested
+// dissection; more: RtPlanHost::more, 0 without it).  False if the problem would
+// be rejected.
+bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options* o, bool rows, size_t* shared,
+                    size_t* inst, size_t* scratch, long long* more) {
   if (!c || !d || !o || d->nx < 2 || d->ny < 2 || d->set_sx < 1 || d->set_sx > MAX_SX || d->set_sy < 1) return false;
   if (o->precision != HMS_FP64 && o->precision != HMS_MIXED) return false;
   const long long rw = std::min((long long)d->nx, (long long)d->set_sx + 2LL * (long long)o->relax_overlap);
@@ -2646,7 +2681,8 @@ bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options
     if (relax_class_smem(cph.slot_elems, cph.nb8max, fp32(&pr)) + 1024 > (size_t)maxsm) return false;
   }
   const size_t nc = cph.rep.size();
-  const bool rtree = rt_plan(lv, o, fp32(&pr), maxsm, c->nsm, o->class_factors ? &cph : nullptr, &rtp);
+  const bool rtree = !rows && rt_plan(lv, o, fp32(&pr), maxsm, c->nsm, o->class_factors ? &cph : nullptr, &rtp);
+  if (more) *more = rtree ? rtp.more : 0;
   if (rtree) {
     fac = (size_t)rtp.elems + RT_PAD;
     plan_bytes = (M + 1) * 8 + M * 4 + rtp.shapes.size() * sizeof(RtShape);
@@ -2709,7 +2745,9 @@ bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options
 // set-factor scratch it holds during setup); 0 if it would be rejected.
 size_t hms_problem_estimate_bytes(hms_context* c, const hms_lattice_desc* d, const hms_options* o) {
   size_t sh = 0, in = 0, sc = 0;
-  if (!estimate_parts(c, d, o, &sh, &in, &sc)) return 0;
+  long long more = 0;
+  if (!estimate_parts(c, d, o, false, &sh, &in, &sc, &more)) return 0;
+  if (more > 0 && sh + in + sc + RT_SLACK > free_bytes() && !estimate_parts(c, d, o, true, &sh, &in, &sc)) return 0;
   return sh + in + sc;
 }
 
@@ -2739,6 +2777,7 @@ struct hms_server {
     std::vector<cudaEvent_t> ev;
     uint64_t bytes = 0;
     int slot = 0;
+    bool rows = false;  // without nested dissection of the sets, to fit the budget
     bool ran = false;  // admitted and solved (u holds results)
     hms_status status = HMS_OK;
   };
@@ -2820,15 +2859,23 @@ hms_status hms_server_submit(hms_server* s, const hms_lattice_desc* d, const hms
   hms_context* c = s->ctx;
   if (o->profile) return fail(c, HMS_ERR_ARG, "hms_server_submit: profile mode is not served");
   size_t sh = 0, in = 0, sc = 0;
-  if (!estimate_parts(c, d, o, &sh, &in, &sc))
+  if (!estimate_parts(c, d, o, false, &sh, &in, &sc))
     return fail(c, HMS_ERR_ARG, "hms_server_submit: the problem would be rejected (lattice / sets / options)");
-  const uint64_t est = sh + (uint64_t)nrhs * in + sc;
+  uint64_t est = sh + (uint64_t)nrhs * in + sc;
+  bool rows = false;
+  if (est > s->budget && estimate_parts(c, d, o, true, &sh, &in, &sc)) {
+    // the row substitution's factors may be the smaller ones
+    const uint64_t est_rows = sh + (uint64_t)nrhs * in + sc;
+    rows = est_rows < est;
+    est = std::min(est, est_rows);
+  }
   if (est > s->budget)
     return fail(c, HMS_ERR_OOM, "hms_server_submit: the request needs " + std::to_string(est) +
                                     " bytes, more than the whole budget of " + std::to_string(s->budget));
   auto* r = new hms_server::Req();
   r->d = *d;
   r->o = *o;
+  r->rows = rows;
   const size_t nn = (size_t)d->nx * d->ny;
   if (d->ea) {
     r->ea.assign(d->ea, d->ea + 3 * nn);
@@ -2879,7 +2926,7 @@ hms_status hms_server_step(hms_server* s, int64_t* done_ids, int32_t cap, int32_
     if (s->used + r->bytes > s->budget) break;
     s->queue.pop_front();
     hms_problem* base = nullptr;
-    hms_status st = hms_problem_create(c, &r->d, &r->o, &base);
+    hms_status st = problem_create(c, &r->d, &r->o, r->rows, &base);
     if (st != HMS_OK) {
       retire(r, st);
       continue;
