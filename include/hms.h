@@ -307,9 +307,10 @@ hms_status hms_solve(hms_problem* pr, int32_t nrhs, const double* loads, const d
  * nrhs[i] load vectors loads[i] ([nrhs[i]][2*nx_i*ny_i]) from u0 = 0 into
  * u_out[i] (same shape), one after another, exactly as hms_solve would
  * (bitwise the same results).  Two engines (hms_context_set_batch_mode):
- *  - lockstep (default where it applies): every step of an update is one
- *    launch over a work list of (problem, tile) items of all running
- *    problems; 16 updates of all of them are one CUDA graph launch; after
+ *  - lockstep (default where it applies; up to 128 problems, some with the tree
+ *    of fronts, only if the largest lattice has at most twice the smallest
+ *    one's nodes): every step of an update is one launch over a work list of
+ *    (problem, tile) items of all running problems; 16 updates of all of them are one CUDA graph launch; after
  *    each, the host reads every problem's convergence flag (one gathered
  *    copy), takes finished load vectors out and starts the next ones, and
  *    rebuilds the work lists when the set of running problems has changed.
@@ -328,13 +329,16 @@ hms_status hms_solve(hms_problem* pr, int32_t nrhs, const double* loads, const d
 hms_status hms_solve_batch(hms_context* c, int32_t count, hms_problem* const* problems,
                            const int32_t* nrhs, const double* const* loads, double* const* u_out,
                            int32_t* iters, int32_t mem_kind);
-/* Engine of hms_solve_batch on c: HMS_BATCH_AUTO (lockstep where it applies,
- * else streams; the default), HMS_BATCH_STREAMS, HMS_BATCH_LOCKSTEP (fails
+/* Engine of hms_solve_batch on c: HMS_BATCH_AUTO (lockstep or streams by the
+ * rule above; the default), HMS_BATCH_STREAMS, HMS_BATCH_LOCKSTEP (fails
  * with HMS_ERR_ARG where it does not apply). */
 #define HMS_BATCH_AUTO 0
 #define HMS_BATCH_STREAMS 1
 #define HMS_BATCH_LOCKSTEP 2
 hms_status hms_context_set_batch_mode(hms_context* c, int32_t mode);
+/* The engine that hms_solve_batch would run these problems with on c now:
+ * HMS_BATCH_LOCKSTEP or HMS_BATCH_STREAMS. */
+int32_t hms_batch_engine(hms_context* c, int32_t count, hms_problem* const* problems);
 
 /* Upper-level updates of the last hms_solve call (all its load vectors)
  * whose FP64 refinement of the Eq. 8 solve used every solve

@@ -107,6 +107,7 @@ def lib():
         "hms_residual_noalloc": (ctypes.c_int32, [_P, _P, _P, _P, _P]),
         "hms_solve_batch": (ctypes.c_int32, [_P, ctypes.c_int32, _P, _P, _P, _P, _P, ctypes.c_int32]),
         "hms_context_set_batch_mode": (ctypes.c_int32, [_P, ctypes.c_int32]),
+        "hms_batch_engine": (ctypes.c_int32, [_P, ctypes.c_int32, _P]),
         "hms_context_tuned_shapes": (ctypes.c_int32, [_P]),
         "hms_problem_relax_form": (ctypes.c_int32, [_P]),
         "hms_problem_coarse_form": (ctypes.c_int32, [_P, ctypes.POINTER(ctypes.c_int32)]),
@@ -145,7 +146,8 @@ def exported_symbols():
             "hms_reactions", "hms_problem_refine_cap_hits", "hms_problem_set_relax_wait_limit",
             "hms_measure_fp64_rate", "hms_relax_force", "hms_problem_relax_balanced", "hms_relax_schedule",
             "hms_set_classes", "hms_nd_plan", "hms_context_tuned_shapes", "hms_problem_coarse_form",
-            "hms_context_set_tree_cluster", "hms_problem_relax_form"]
+            "hms_context_set_tree_cluster", "hms_problem_relax_form",
+            "hms_batch_engine"]
 
 
 # ---------------------------------------------------------------- marshalling
@@ -376,6 +378,11 @@ def hms_solve_batch(ctx, problems, loads, u_out, iters=None, allow_no_convergenc
     up = (_P * max(n, 1))(*[a.ptr for a in U])
     ok = (HMS_OK, HMS_ERR_NO_CONVERGENCE) if allow_no_convergence else (HMS_OK,)
     return _check(ctx, lib().hms_solve_batch(ctx, n, pp, nrhs, lp, up, I.ptr, mk), ok=ok)
+
+
+def hms_batch_engine(ctx, problems) -> int:
+    pp = (_P * max(len(problems), 1))(*[ctypes.cast(pr, _P) for pr in problems])
+    return int(lib().hms_batch_engine(ctx, len(problems), pp))
 
 
 def hms_server_create(ctx, hbm_budget_bytes, max_active=256):

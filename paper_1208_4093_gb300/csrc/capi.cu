@@ -1842,13 +1842,40 @@ static bool lockstep_applies(int32_t count, hms_problem* const* problems) {
   return true;
 }
 
+// Whether the automatic choice takes the lockstep engine where it applies.  A step
+// of it takes as long as its slowest problem's, and small trees' steps add to a
+// large one's, while a problem on its own stream goes on at its own pace: with
+// trees in the batch, streams unless the problems are of about one size, or more
+// than two for each of the 64 streams.  Measured lockstep / streams (ms, mixed; 32 x 32 sets):
+// 8 of 64^2 nodes 16.4 / 20.9, 32 of 256^2 326 / 351, 8 of 512^2 334 / 356, 8 of
+// 256^2 and 8 of 180^2 158 / 156; 8 of 256^2 and 8 of 128^2 142 / 129, 512^2 and 7
+// of 128^2 134 / 115, 32 load vectors of 16 lattices with sides 32 to 256 102 / 81
+// (FP64 181 / 128), 71 of 32 with sides 32 to 512 300 / 288, 539 of 128 1692 / 2198.
+static bool lockstep_pays(int32_t count, hms_problem* const* problems) {
+  bool tree = false;
+  size_t lo = SIZE_MAX, hi = 0;
+  for (int i = 0; i < count; ++i) {
+    tree = tree || problems[i]->tree;
+    lo = std::min(lo, nnodes(problems[i]));
+    hi = std::max(hi, nnodes(problems[i]));
+  }
+  return !tree || count > 128 || hi <= 2 * lo;
+}
+
+int32_t hms_batch_engine(hms_context* c, int32_t count, hms_problem* const* problems) {
+  if (!c || count < 1 || !problems) return HMS_BATCH_STREAMS;
+  for (int i = 0; i < count; ++i)
+    if (!problems[i] || problems[i]->ctx != c) return HMS_BATCH_STREAMS;
+  if (c->batch_mode == HMS_BATCH_STREAMS || !lockstep_applies(count, problems)) return HMS_BATCH_STREAMS;
+  return c->batch_mode == HMS_BATCH_LOCKSTEP || lockstep_pays(count, problems) ? HMS_BATCH_LOCKSTEP
+                                                                             : HMS_BATCH_STREAMS;
+}
+
 hms_status hms_solve_batch(hms_context* c, int32_t count, hms_problem* const* problems, const int32_t* nrhs,
                            const double* const* loads, double* const* u_out, int32_t* iters, int32_t mem_kind) {
   if (!c) return HMS_ERR_ARG;
   if (count > 0 && problems && c->batch_mode != HMS_BATCH_STREAMS) {
-    bool ok = true;
-    for (int i = 0; i < count && ok; ++i) ok = problems[i] && problems[i]->ctx == c;
-    if (ok && lockstep_applies(count, problems))
+    if (hms_batch_engine(c, count, problems) == HMS_BATCH_LOCKSTEP)
       return solve_batch_lockstep(c, count, problems, nrhs, loads, u_out, iters, mem_kind);
     if (c->batch_mode == HMS_BATCH_LOCKSTEP)
       return fail(c, HMS_ERR_ARG, "hms_solve_batch: lockstep needs one precision, one coarse_solves and the "
