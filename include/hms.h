@@ -310,14 +310,15 @@ hms_status hms_solve(hms_problem* pr, int32_t nrhs, const double* loads, const d
  *  - lockstep (default where it applies; up to 128 problems, some with the tree
  *    of fronts, only if the largest lattice has at most twice the smallest
  *    one's nodes): every step of an update is one launch over a work list of
- *    (problem, tile) items of all running problems; 16 updates of all of them are one CUDA graph launch; after
- *    each, the host reads every problem's convergence flag (one gathered
- *    copy), takes finished load vectors out and starts the next ones, and
- *    rebuilds the work lists when the set of running problems has changed.
+ *    (problem, tile) items of all running problems; 16 updates of all of them
+ *    are one CUDA graph launch; after each, the host reads every problem's
+ *    convergence flag (one gathered copy), takes finished load vectors out and
+ *    starts the next ones, and rebuilds the work lists when the set of running
+ *    problems has changed.
  *    It applies when all problems share precision and coarse_solves and use
  *    the FP32 one-SM factor with the 64-row block solve (coarse_factor = 4,
  *    or auto where that is its choice) or the tree of fronts (auto, or
- *    coarse_factor = 6 where it fits), with nine modes per set;
+ *    coarse_factor = 6 where it fits), with nine modes and per-set factors;
  *  - streams: each problem runs its own graph rounds on one of up to 64
  *    streams of the context at its own pace.
  * Clones (hms_problem_clone) let one lattice's load vectors run at the same

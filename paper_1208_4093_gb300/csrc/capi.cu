@@ -1878,8 +1878,9 @@ hms_status hms_solve_batch(hms_context* c, int32_t count, hms_problem* const* pr
     if (hms_batch_engine(c, count, problems) == HMS_BATCH_LOCKSTEP)
       return solve_batch_lockstep(c, count, problems, nrhs, loads, u_out, iters, mem_kind);
     if (c->batch_mode == HMS_BATCH_LOCKSTEP)
-      return fail(c, HMS_ERR_ARG, "hms_solve_batch: lockstep needs one precision, one coarse_solves and the "
-                                  "one-SM FP32 factor with the block solve for every problem");
+      return fail(c, HMS_ERR_ARG, "hms_solve_batch: lockstep needs one precision and one coarse_solves, and "
+                                  "of every problem nine modes, per-set factors and the tree of fronts "
+                                  "or the one-SM FP32 factor with the block solve");
   }
   return solve_batch_streams(c, count, problems, nrhs, loads, u_out, iters, mem_kind);
 }

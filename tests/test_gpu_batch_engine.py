@@ -55,3 +55,20 @@ def test_engine_by_sizes(hms_ctx, batch, prec):
     finally:
         for pr in many:
             capi.hms_problem_destroy(pr)
+
+
+def test_refusal_names_what_lockstep_needs(hms_ctx, batch):
+    """Each refused batch breaks one condition of the message; a batch of trees breaks none."""
+    from paper_1208_4093_gb300 import capi
+    shape = (48, 144)
+    tree, p = batch([shape])[0], loads(*shape, 3).reshape(1, -1)
+    capi.hms_context_set_batch_mode(hms_ctx, capi.HMS_BATCH_LOCKSTEP)
+    capi.hms_solve_batch(hms_ctx, [tree], [p], [np.empty_like(p)])
+    for kw, need in ((dict(precision=1), "one precision"), (dict(coarse_solves=3), "one coarse_solves"),
+                     (dict(mode_mask=0xFFF), "nine modes"), (dict(class_factors=1), "per-set factors"),
+                     (dict(coarse_factor=5), "the tree of fronts or the one-SM FP32 factor")):
+        other = batch([shape], **kw)[0]
+        with pytest.raises(capi.HmsError) as e:
+            capi.hms_solve_batch(hms_ctx, [tree, other], [p, p], [np.empty_like(p), np.empty_like(p)])
+        assert e.value.status == capi.HMS_ERR_ARG
+        assert need in capi.hms_last_error(hms_ctx), kw
