@@ -287,7 +287,7 @@ cudaError_t launch_relax_main(hms_problem* pr, cudaStream_t s, const IterCtl* ct
 // K_aa from the slots and the scaled system of Eq. 8 (scale, b, x = 0, drop
 // flags): by blocks for nested dissection, else as a band.
 cudaError_t launch_scaled_system(hms_problem* pr, cudaStream_t s, const IterCtl* ctl) {
-  if (pr->tree) return launch_tree_system(s, pr->lv.q, true, pr->tprob, nullptr, pr->lv.M, ctl != nullptr);
+  if (pr->tree) return launch_tree_system(s, pr->lv.q, true, pr->tprob, nullptr, pr->lv.M, ctl != nullptr, pr->lv.nsm);
   if (pr->nd) {
     cudaError_t e = launch_blocks_from_slots(s, pr->lv, pr->slots_base, pr->slots_it, pr->blk, ctl);
     if (e != cudaSuccess) return e;
@@ -1303,6 +1303,7 @@ static hms_status problem_create(hms_context* c, const hms_lattice_desc* d, cons
   lv.sy = d->set_sy;
   lv.Mx = (d->nx + d->set_sx - 1) / d->set_sx;
   lv.My = (d->ny + d->set_sy - 1) / d->set_sy;
+  lv.nsm = c->nsm;
   lv.rr = update_residual_rr(lv);
   lv.M = lv.Mx * lv.My;
   lv.ov = o->relax_overlap;
@@ -2301,10 +2302,10 @@ static hms_status solve_batch_lockstep(hms_context* c, int32_t count, hms_proble
         if (e == cudaSuccess) e = launch_batch_rtree(s, f32, rthreads, rchunks, sm_rt, P, L(BL_RT), N(BL_RT));
         if (e == cudaSuccess) e = launch_batch_relax(s, f32, rthreads, rchunks, sm_relax, P, L(BL_RS), N(BL_RS));
         if (e == cudaSuccess) e = launch_batch_slots(s, f32, sm_slots, P, L(BL_SETS), N(BL_SETS));
-        if (e == cudaSuccess) e = launch_tree_system(s, NMODES, true, TP, TI, tl.nsets, true);
+        if (e == cudaSuccess) e = launch_tree_system(s, NMODES, true, TP, TI, tl.nsets, true, c->nsm);
         for (size_t h = 0; h < tl.T.size() && e == cudaSuccess; ++h) {
           const int n = tl.begin[h + 1] - tl.begin[h];
-          e = launch_tree_level(s, tree_level_launch(n, tl.T[h], maxsm), TP, TI + tl.begin[h], n, true);
+          e = launch_tree_level(s, tree_level_launch(n, tl.T[h], maxsm, c->nsm), TP, TI + tl.begin[h], n, true);
         }
         for (size_t z = 0; z < tl.solves.size() && e == cudaSuccess; ++z)
           e = launch_tree_solve(s, NMODES, tl.solves[z][0], tl.solve_smem[z], TP, (const int*)dtwhich.p + tl.solves[z][1],
@@ -2601,7 +2602,7 @@ hms_status hms_coarse_solve(hms_problem* pr, const double* Kaa, const double* P,
   CKC(c, e);
   CKC(c, cudaMemcpyAsync(pr->P, P, n * sizeof(double), kind_in(mem_kind), s));
   if (pr->tree)
-    CKC(c, launch_tree_system(s, pr->lv.q, false, pr->tprob, nullptr, pr->lv.M, false));
+    CKC(c, launch_tree_system(s, pr->lv.q, false, pr->tprob, nullptr, pr->lv.M, false, pr->lv.nsm));
   else if (pr->nd)
     CKC(c, launch_blk_diag(s, pr->lv, pr->blk, pr->P, pr->scale, pr->b, pr->x, pr->dropped, pr->mode_mask, nullptr));
   else
@@ -2681,6 +2682,7 @@ bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options
   if (cudaSetDevice(c->device) != cudaSuccess) return false;
   hms_problem pr;
   LatView& lv = pr.lv;
+  lv.nsm = c->nsm;
   lv.nx = d->nx;
   lv.ny = d->ny;
   lv.sx = d->set_sx;

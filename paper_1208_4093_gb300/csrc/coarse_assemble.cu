@@ -19,6 +19,7 @@
 // order, so the result is the same on every run.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "coarse_blocks.cuh"
@@ -793,7 +794,7 @@ cudaError_t launch_coarse_slots(cudaStream_t s, const LatView& lv, const void* d
   float2* const f2 = nullptr;
   double2* const d2 = nullptr;
   if (!full) {
-    const int cl = lv.M > 76 ? 1 : (lv.M > 38 ? 152 / lv.M : 4);
+    const int cl = std::max(1, std::min(4, lv.nsm / lv.M));  // CTAs per set while SMs are free
     auto go = [&](auto k, auto* d) {
       using DT = std::remove_pointer_t<decltype(d)>;
       return launch_dep(k, s, lv.M * cl, 32 * ((SP + cl - 1) / cl), coarse_slots_it_smem(lv, delta_fp32),

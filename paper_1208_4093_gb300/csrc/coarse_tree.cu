@@ -924,7 +924,7 @@ namespace {
 // took 273 us with leaves of 4 x 4, 312 with 3 x 3, 289 with 2 x 2 and 345 with 1 x 1
 // (35 x 29 sets: 637, 652, 710, 725).
 constexpr int TREE_LEAF = 4, TREE_ROOT = 256;
-constexpr int TREE_FILL = 148;  // CTAs a level is spread over, if its fronts allow (152 SMs)
+constexpr int TREE_FREE = 4;    // SMs left over when a level is spread over CTAs
 constexpr int TREE_SROWS = 16;  // unknowns of a CTA of a solve, at least
 constexpr int TREE_PORTABLE = 8;  // a cluster size that every part can place
 }  // namespace
@@ -939,7 +939,7 @@ static size_t front_need(int T, int cl, int nbuf) {
 // the smallest cluster that holds the largest front, then more CTAs per front
 // while the launch leaves SMs idle and each CTA keeps a block row; two buffers
 // of the pivot column where a single CTA has room for them.
-TreeLaunch tree_level_launch(int n, int T, int max_smem) {
+TreeLaunch tree_level_launch(int n, int T, int max_smem, int nsm) {
   const size_t cap = (size_t)max_smem - 2048;
   auto need = [&](int cl, int nbuf) {
     size_t m = 0;
@@ -949,7 +949,7 @@ TreeLaunch tree_level_launch(int n, int T, int max_smem) {
   TreeLaunch L;
   L.cl = 1;
   while (L.cl < 8 && need(L.cl, 1) > cap) ++L.cl;
-  while (L.cl < 8 && (long long)n * (L.cl + 1) <= TREE_FILL && L.cl + 1 <= T) ++L.cl;
+  while (L.cl < 8 && (long long)n * (L.cl + 1) <= nsm - TREE_FREE && L.cl + 1 <= T) ++L.cl;
   L.nbuf = L.cl == 1 && need(1, 2) <= cap ? 2 : 1;
   L.smem = need(L.cl, L.nbuf);
   return L;
@@ -1057,7 +1057,7 @@ bool tree_plan_build(const LatView& lv, int max_smem, int max_cl, TreePlanHost* 
       P->items.push_back(TreeItem{0, k});
       Tmax = std::max(Tmax, blocks(hn[k]));
     }
-    const TreeLaunch tl = tree_level_launch((int)byh[h].size(), Tmax, max_smem);
+    const TreeLaunch tl = tree_level_launch((int)byh[h].size(), Tmax, max_smem, lv.nsm);
     P->level_cl[h] = tl.cl;
     P->level_nbuf[h] = tl.nbuf;
     P->level_T[h] = Tmax;
@@ -1154,12 +1154,12 @@ bool tree_plan_build(const LatView& lv, int max_smem, int max_cl, TreePlanHost* 
 size_t tree_arow_elems(const LatView& lv) { return (size_t)lv.q * lv.M * 9 * lv.q; }
 
 cudaError_t launch_tree_system(cudaStream_t s, int q, bool slots, const TreeProb* probs, const TreeItem* sets, int n,
-                               bool use_ctl) {
+                               bool use_ctl, int nsm) {
   if (n <= 0) return cudaSuccess;
   const int c = (int)use_ctl;
   const auto diag = q == NMODES_RF ? (slots ? k_tree_diag<NMODES_RF, true> : k_tree_diag<NMODES_RF, false>)
                                    : (slots ? k_tree_diag<NMODES, true> : k_tree_diag<NMODES, false>);
-  const int dt = n > 304 ? 128 : (q == NMODES_RF ? DIAG_T<NMODES_RF> : DIAG_T<NMODES>);
+  const int dt = n > 2 * nsm ? 128 : (q == NMODES_RF ? DIAG_T<NMODES_RF> : DIAG_T<NMODES>);
   const cudaError_t e = launch_dep(diag, s, n, dt, 0, 0, probs, sets, c);
   if (e != cudaSuccess) return e;
   return launch_dep(k_tree_rows, s, n, 256, 0, 0, probs, sets, c);

@@ -55,6 +55,7 @@ struct LatView {
   int ov;          // relaxation region: the set's tile grown by ov nodes (Sec. 2.2)
   int q = 9;       // incremental modes per set: 9, or 12 with the force-controlled modes
   int rr = 1;      // rows of a warp of the residual kernel (update_residual_rr)
+  int nsm = 1;     // SMs of the device (launch shapes)
   double L;        // bar length
   double k_u;      // EA/L when kbar == nullptr
   const double* kbar;
@@ -631,13 +632,13 @@ constexpr int TREE_SCL = 16;  // CTAs of a solve's cluster, at most
 bool tree_plan_build(const LatView& lv, int max_smem, int max_cl, TreePlanHost* P);
 size_t tree_arow_elems(const LatView& lv);
 cudaError_t configure_coarse_tree(int max_smem);
-TreeLaunch tree_level_launch(int n, int T, int max_smem);
+TreeLaunch tree_level_launch(int n, int T, int max_smem, int nsm);
 // The launches take problems probs and a work list: {problem, set}, {problem,
 // node} or problem indices (no list: the sets of the only problem).  use_ctl:
 // problems whose control block says done are passed over.
 // scale, b, x = 0, drop flags and the scaled rows, from the slots or the blocks
 cudaError_t launch_tree_system(cudaStream_t s, int q, bool slots, const TreeProb* probs, const TreeItem* sets, int n,
-                               bool use_ctl);
+                               bool use_ctl, int nsm);
 cudaError_t launch_tree_level(cudaStream_t s, const TreeLaunch& L, const TreeProb* probs, const TreeItem* nodes, int n,
                               bool use_ctl);
 cudaError_t launch_tree_factor(cudaStream_t s, const TreePlanHost& P, const TreeProb* prob, const TreeItem* items,

@@ -481,7 +481,7 @@ cudaError_t launch_reactions(cudaStream_t s, const LatView& lv, const double2* u
   return cudaGetLastError();
 }
 
-// Rows of a warp: the count (up to 32) that costs the busiest of the 152 SMs the
+// Rows of a warp: the count (up to 32) that costs the busiest SM the
 // fewest FP64 operations, with 34 per row of a warp and 26 for its two outer rows.
 // Small lattices get one or two rows (64 x 64 nodes: 1), 1024 x 1024 nodes 10.
 int update_residual_rr(const LatView& lv) {
@@ -489,7 +489,7 @@ int update_residual_rr(const LatView& lv) {
   long long best = -1;
   int rr = 1;
   for (int h = 1; h <= 32; ++h) {
-    const long long ctas = strips * ((lv.ny + RW * h - 1) / (RW * h)), cost = (ctas + 151) / 152 * (34 * h + 26);
+    const long long ctas = strips * ((lv.ny + RW * h - 1) / (RW * h)), cost = (ctas + lv.nsm - 1) / lv.nsm * (34 * h + 26);
     if (best < 0 || cost <= best) best = cost, rr = h;
   }
   return rr;
