@@ -106,9 +106,10 @@ typedef struct {
                                 4 = FP32 on one SM, 5 = FP32 two-sided: top and bottom
                                 segments eliminated at once on two SMs, then the
                                 separator between them, 6 = FP32 nested dissection of
-                                the set grid over K_aa kept as 9 x 9 blocks per set
+                                the set grid over K_aa kept as q x q blocks per set
                                 pair (no band).  Where the fronts fit the shared memory
-                                of a thread-block cluster (up to about 40 sets across):
+                                of a thread-block cluster (square set grids up to 39 x
+                                39, 29 x 29 with twelve modes; narrow ones of any length):
                                 boxes of sets cut by a middle column and row of sets at
                                 once, the fronts of one level of the tree factored at
                                 once, a cluster each, and all solves of an update in one
@@ -172,9 +173,12 @@ typedef struct {
   int32_t relax_balance;     /* schedule of the relaxation with per-set factors:
                                 0 = one CTA per set (sets in waves of the SM count), its
                                 nodes ordered by nested dissection: for set tiles of more
-                                than 64 nodes, unless its padded factors take more
-                                memory than those of the row substitution and that is
-                                more than 4 GB or more than is free; else, with
+                                than 64 nodes whose relaxation regions need at most 256
+                                inputs of a front (squares of up to 65 nodes a side; 64 x
+                                64-node tiles only with relax_overlap = 0), unless its
+                                padded factors take more memory than those of the row
+                                substitution and that is more than 4 GB or more than is
+                                free; else, with
                                 relax_threads = 0, the faster of 1 and 2 by timing where
                                 both apply, else 1;
                                 1 = substitution row by row of the lattice, one CTA per
@@ -347,7 +351,11 @@ int32_t hms_batch_engine(hms_context* c, int32_t count, hms_problem* const* prob
  * still above 1e-14 max|b|: the update then went on with the refined
  * solution as it stood.  0 when every update's refinement met the criterion
  * before its last solve, and always with coarse_solves = 1 (no
- * refinement). */
+ * refinement).  The tree of fronts inverts its pivot blocks, which in FP32 costs
+ * the refinement a little of its rate against the band's Cholesky factor: with
+ * five solves 7 to 14 of about 600 updates count on eight 1024 x 1024 lognormal
+ * lattices, 4 to 7 with the two-sided band.  The residual that decides convergence
+ * (Eq. 19) is FP64 either way, and the update counts are the same. */
 int64_t hms_problem_refine_cap_hits(const hms_problem* pr);
 
 /* Per-kernel CUDA-event time of the last hms_solve with options.profile = 1:
