@@ -353,8 +353,8 @@ int32_t hms_batch_engine(hms_context* c, int32_t count, hms_problem* const* prob
  * before its last solve, and always with coarse_solves = 1 (no
  * refinement).  The tree of fronts inverts its pivot blocks, which in FP32 costs
  * the refinement a little of its rate against the band's Cholesky factor: with
- * five solves 7 to 14 of about 600 updates count on eight 1024 x 1024 lognormal
- * lattices, 4 to 7 with the two-sided band.  The residual that decides convergence
+ * five solves 7 to 18 of about 600 updates count on twenty 1024 x 1024 lognormal
+ * problems, 4 to 7 with the two-sided band.  The residual that decides convergence
  * (Eq. 19) is FP64 either way, and the update counts are the same. */
 int64_t hms_problem_refine_cap_hits(const hms_problem* pr);
 

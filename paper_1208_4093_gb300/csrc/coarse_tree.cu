@@ -218,8 +218,8 @@ __device__ __forceinline__ void mm32(const float* A, int lda, const float* B, in
 // holding the block needs eight 16-byte loads a pivot and 230 cycles; with its
 // 32 pivots written out it is 60 KB of code run once, whose fetching takes 690
 // cycles a pivot.  A Newton step on the pivots' reciprocals (1 ulp as they are) does
-// not help the refinement: 80 of 4822 updates used every solve with it, 78 without (39
-// with the two-sided band factor); the explicit inverse is what costs it.
+// not help the refinement: 217 of 12060 updates used every solve with it, 194 without
+// and 97 with the two-sided band factor; the explicit inverse is what costs it.
 __device__ __forceinline__ unsigned sweep32(float (&a)[8], int kb, int w, int lane, float* buf) {
   unsigned dm = 0u;
 #pragma unroll 1
