@@ -657,6 +657,9 @@ RtSetup rt_setup(const RtPlanHost& P, int M, int nsm) {
   S.own = (S.grid - S.first) * P.scratch;
   return S;
 }
+// Bytes a problem takes beyond the row substitution's for M factors by nested
+// dissection: the padding (negative for larger tiles) and the work space.
+long long rt_more(const RtPlanHost& P, int M, int nsm) { return P.more + 8 * rt_setup(P, M, nsm).own; }
 
 // Nested dissection over the set grid: as a tree of fronts swept in the shared
 // memory of one cluster each (coarse_tree.cu) where they fit, else panel by
@@ -1395,7 +1398,8 @@ static hms_status problem_create(hms_context* c, const hms_lattice_desc* d, cons
     }
   }
   pr->rtree = !rows && rt_plan(lv, o, fp32(pr), maxsm, c->nsm, o->class_factors ? &cph : nullptr, &rtp) &&
-              (rtp.more <= 0 || rt_has_room(c, d, o, rtp, free_bytes() + pr->bytes));
+              (rt_more(rtp, pr->classes ? (int)cph.rep.size() : lv.M, c->nsm) <= 0 ||
+               rt_has_room(c, d, o, rtp, free_bytes() + pr->bytes));
   RtSetup rtsu;
   double* rtwork = nullptr;
   {
@@ -2658,8 +2662,8 @@ namespace {
 // Device bytes of a problem for (d, o), following hms_problem_create's
 // allocations one by one: the shared setup buffers, one instance's buffers
 // and the scratch held while the set factors are computed (rows: without nested
-// dissection; more: RtPlanHost::more, 0 without it).  False if the problem would
-// be rejected.
+// dissection; more: rt_more, 0 without it).  False if the problem would be
+// rejected.
 bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options* o, bool rows, size_t* shared,
                     size_t* inst, size_t* scratch, long long* more) {
   if (!c || !d || !o || d->nx < 2 || d->ny < 2 || d->set_sx < 1 || d->set_sx > MAX_SX || d->set_sy < 1) return false;
@@ -2712,7 +2716,7 @@ bool estimate_parts(hms_context* c, const hms_lattice_desc* d, const hms_options
   }
   const size_t nc = cph.rep.size();
   const bool rtree = !rows && rt_plan(lv, o, fp32(&pr), maxsm, c->nsm, o->class_factors ? &cph : nullptr, &rtp);
-  if (more) *more = rtree ? rtp.more : 0;
+  if (more) *more = rtree ? rt_more(rtp, o->class_factors ? (int)nc : lv.M, c->nsm) : 0;
   if (rtree) {
     fac = (size_t)rtp.elems + RT_PAD;
     plan_bytes = (M + 1) * 8 + M * 4 + rtp.shapes.size() * sizeof(RtShape);

@@ -96,3 +96,27 @@ def test_a_problem_that_fits_the_free_memory_only_by_rows_is_created(hms_ctx):
         capi.hms_problem_destroy(pr)
     # two updates from rounding: FP64 local solves agree to 1e-11 (test_gpu_parity)
     assert np.linalg.norm(u - low) < 1e-9 * np.linalg.norm(u)
+
+
+def test_work_space_of_the_factorisation_counts(hms_ctx):
+    """24 x 20-node tiles: the factors are smaller than the row substitution's, but with
+    the work space that their factorisation keeps the problem is larger."""
+    import torch
+    from paper_1208_4093_gb300 import capi
+    nsm = torch.cuda.get_device_properties(0).multi_processor_count
+    nx, ny, sx, sy = 24 * nsm, 20, 24, 20
+    rows = capi.hms_problem_estimate_bytes(hms_ctx, nx, ny, sx, sy, relax_balance=1)
+    tree = capi.hms_problem_estimate_bytes(hms_ctx, nx, ny, sx, sy)
+    assert tree > rows
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - tree - (128 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        assert capi.hms_problem_estimate_bytes(hms_ctx, nx, ny, sx, sy) == rows
+        pr = capi.hms_problem_create(hms_ctx, nx, ny, sx, sy)
+        try:
+            assert capi.hms_problem_relax_form(pr) == capi.HMS_RELAX_ROWS
+        finally:
+            capi.hms_problem_destroy(pr)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
